@@ -185,6 +185,7 @@ struct Params {
     // the oldest point, consecutive in its region.  Either way every child
     // survives and child c of group g goes to entry g of region c.
     int reg_fill, reg_merge;
+    int nnz0;                          // nonzero elements of rho(0): members of a group at the first full-mask merge
     unsigned long long full_n;
     unsigned long long *tile_state;    // [M*M][max_tiles] look-back words (a bucket's tiles contiguous)
     long long max_tiles;
@@ -940,65 +941,105 @@ __device__ __forceinline__ double2 *rho_part_of(const Params &P, unsigned long l
     return P.rho_part + (size_t)(tn & 1) * kMaxExpandBlocks * P.n_inst * (MM + 1);
 }
 
+// Sums of V values over the warp by halving (a power of two V <= 32): in round
+// o a lane keeps one half of its values and hands the other half to lane ^ o,
+// so the rounds cost V/2 + V/4 + ... additions instead of 5 V (FP64: the
+// pipe takes a warp's addition 16 cycles, and 24 warps per SM reduce their
+// accumulators at the end of a step kernel).  On return v[0] is the warp's
+// sum of value rs_index<V>(lane).  The result does not depend on the lane.
+template <int V>
+__device__ __forceinline__ int rs_index() {
+    int idx = 0;
+#pragma unroll
+    for (int n = V / 2, o = 16; n >= 1; n >>= 1, o >>= 1)
+        if (lane_id() & o) idx += n;
+    return idx;
+}
+template <int V>
+__device__ __forceinline__ void warp_reduce_scatter(double (&v)[V]) {
+    const unsigned lane = lane_id();
+    int o = 16;
+#pragma unroll
+    for (int n = V / 2; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0u;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double give = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+}
+// the same for FP32 pairs (s + e, the rounding error of every addition kept
+// in e: TwoSum)
+template <int V>
+__device__ __forceinline__ void warp_reduce_scatter(float (&s)[V], float (&e)[V]) {
+    const unsigned lane = lane_id();
+    int o = 16;
+#pragma unroll
+    for (int n = V / 2; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0u;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float gs = up ? s[i] : s[i + n], ge = up ? e[i] : e[i + n];
+            float ks = up ? s[i + n] : s[i], ke = up ? e[i + n] : e[i];
+            const float b = __shfl_xor_sync(0xffffffffu, gs, o), f = __shfl_xor_sync(0xffffffffu, ge, o);
+            two_sum_acc(ks, ke, b);
+            s[i] = ks;
+            e[i] = ke + f;
+        }
+    }
+    for (; o >= 1; o >>= 1) {
+        const float b = __shfl_xor_sync(0xffffffffu, s[0], o), f = __shfl_xor_sync(0xffffffffu, e[0], o);
+        two_sum_acc(s[0], e[0], b);
+        e[0] += f;
+    }
+}
+
 // Stream engine: each block stores its partial of rho per end point, C64 as
-// an FP32 sum and the rounding error of every addition (warp shuffles, then
-// the warps folded by one thread per end point, all with error-free TwoSum
-// additions, so no FP64 in the kernel's tail), FP64 as a double pair in the
-// same 16 bytes.  s_rt: [NW][M*M] scratch; dst = [M*M] of this block.  All
-// threads of the block call it.
+// an FP32 sum and the rounding error of every addition (the warps' sums by
+// halving, then the warps folded by one thread per component, all with
+// error-free TwoSum additions, so no FP64 in the kernel's tail), FP64 as a
+// double pair in the same 16 bytes.  s_rt: [NW][M*M] scratch; dst = [M*M] of
+// this block.  All threads of the block call it.
 template <int MM, int NW, bool C64>
 __device__ __forceinline__ void block_rho_pair(const typename std::conditional<C64, float2, double2>::type *hi,
                                                const float2 *lo, float4 (*s_rt)[MM], float4 *dst) {
-    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    constexpr int V = MM <= 4 ? 8 : 32;   // 2 M*M components, padded
+    const unsigned warp = threadIdx.x >> 5;
+    const int idx = rs_index<V>();
+    const bool mine = idx < 2 * MM && (lane_id() & (32 / V - 1)) == 0u;
+    if constexpr (C64) {
+        float sv[V], ev[V];
 #pragma unroll
-    for (int k = 0; k < MM; ++k) {
-        if constexpr (C64) {
-            float sx = hi[k].x, ex = lo[k].x, sy = hi[k].y, ey = lo[k].y;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float bx = __shfl_down_sync(0xffffffffu, sx, o), fx = __shfl_down_sync(0xffffffffu, ex, o);
-                const float by = __shfl_down_sync(0xffffffffu, sy, o), fy = __shfl_down_sync(0xffffffffu, ey, o);
-                const float tx = sx + bx, vx = tx - sx;
-                ex += fx + ((sx - (tx - vx)) + (bx - vx));
-                sx = tx;
-                const float ty = sy + by, vy = ty - sy;
-                ey += fy + ((sy - (ty - vy)) + (by - vy));
-                sy = ty;
-            }
-            if (lane == 0) s_rt[warp][k] = make_float4(sx, ex, sy, ey);
-        } else {
-            double x = hi[k].x, y = hi[k].y;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                x += __shfl_down_sync(0xffffffffu, x, o);
-                y += __shfl_down_sync(0xffffffffu, y, o);
-            }
-            if (lane == 0) reinterpret_cast<double2 *>(&s_rt[warp][0])[k] = make_double2(x, y);
+        for (int k = 0; k < V; ++k) {
+            sv[k] = k < 2 * MM ? ((k & 1) ? hi[k >> 1].y : hi[k >> 1].x) : 0.f;
+            ev[k] = k < 2 * MM ? ((k & 1) ? lo[k >> 1].y : lo[k >> 1].x) : 0.f;
         }
+        warp_reduce_scatter<V>(sv, ev);
+        if (mine) reinterpret_cast<float2 *>(&s_rt[warp][0])[idx] = make_float2(sv[0], ev[0]);
+    } else {
+        double v[V];
+#pragma unroll
+        for (int k = 0; k < V; ++k) v[k] = k < 2 * MM ? ((k & 1) ? hi[k >> 1].y : hi[k >> 1].x) : 0.0;
+        warp_reduce_scatter<V>(v);
+        if (mine) reinterpret_cast<double *>(&s_rt[warp][0])[idx] = v[0];
     }
     __syncthreads();
-    if ((int)threadIdx.x < MM) {
+    if ((int)threadIdx.x < 2 * MM) {
         const int k = threadIdx.x;
         if constexpr (C64) {
-            float4 a = s_rt[0][k];
+            float2 a = reinterpret_cast<const float2 *>(&s_rt[0][0])[k];
             for (int w = 1; w < NW; ++w) {
-                const float4 b = s_rt[w][k];
-                const float tx = a.x + b.x, vx = tx - a.x;
-                a.y += b.y + ((a.x - (tx - vx)) + (b.x - vx));
-                a.x = tx;
-                const float ty = a.z + b.z, vy = ty - a.z;
-                a.w += b.w + ((a.z - (ty - vy)) + (b.z - vy));
-                a.z = ty;
-            }
-            dst[k] = a;
-        } else {
-            double2 a = reinterpret_cast<const double2 *>(&s_rt[0][0])[k];
-            for (int w = 1; w < NW; ++w) {
-                const double2 b = reinterpret_cast<const double2 *>(&s_rt[w][0])[k];
-                a.x += b.x;
+                const float2 b = reinterpret_cast<const float2 *>(&s_rt[w][0])[k];
+                two_sum_acc(a.x, a.y, b.x);
                 a.y += b.y;
             }
-            reinterpret_cast<double2 *>(dst)[k] = a;
+            reinterpret_cast<float2 *>(dst)[k] = a;
+        } else {
+            double a = reinterpret_cast<const double *>(&s_rt[0][0])[k];
+            for (int w = 1; w < NW; ++w) a += reinterpret_cast<const double *>(&s_rt[w][0])[k];
+            reinterpret_cast<double *>(dst)[k] = a;
         }
     }
 }
@@ -1255,54 +1296,111 @@ __device__ __forceinline__ unsigned long long lb_word(unsigned epoch, unsigned s
 }
 
 // Regular steps of the stream engine (no filter, see Params): while the
-// window fills every stored path is its own group; with the full mask, once
-// all M^(2 dkmax) keys are stored, every group is the M*M consecutive values
-// of the oldest point.  Every child survives, so child c of group g goes to
-// entry g of output region c: a streaming map, one thread per group, no
+// window fills every stored path is its own group; with the full mask every
+// group is the consecutive values of the oldest point: the M*M values once
+// all M^(2 dkmax) keys are stored, and at the first merge the nnz0 values
+// that rho(0) has.  Every child survives, so child c of group g goes to entry
+// g of output region c: a streaming map, one thread per group, no
 // shared-memory tile, no look-back.  The representative does not
 // matter: members differ only in the oldest point, which the history sum
-// does not read and the child key drops.  Launched before the tile kernel on
-// configurations that allow regular steps; it decides on the device, takes
+// does not read and the child key drops.  It decides on the device, takes
 // the step (reg_done = new t + 1) or leaves it to the tile kernel
 // (reg_done = 0), and publishes the step it takes like the tile kernel.
+//
+// Work split: chunks of 32 groups (a warp's), dealt to the blocks in turn,
+// so that a small step uses as many SMs as it has chunks; blocks without a
+// chunk return at once, except the first of them, which sums the pending
+// rho of the previous step beside the others (a grid without a spare block
+// leaves that to its last block, after it has arrived).  At memory 8
+// (1.6e4 groups, complex64) and 5 (256 groups, FP64) the step is latency:
+// with every block of the grid reducing and arriving, and block 0 summing
+// the pending rho first, the kernel took 13.3 and 21.2 us (under ncu), and
+// 100 and 40 steps through qp_step 1.72 and 1.09 ms; now 1.16 and 0.50 ms,
+// with the tile kernel's empty launch gone (step_kind).
 template <int M, bool C64>
-__global__ void __launch_bounds__(kRegThreads, 3) k_stream_regular(Params P, int lut_smem) {
+__global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(Params P, int lut_smem) {
     using X = Expander<M, C64>;
     using AmpT = typename X::AmpT;
-    constexpr int MM = M * M, NT = kRegThreads;
-    static_assert(NT / 32 == kStreamWarps, "warp partials");
+    constexpr int MM = M * M, NT = kRegThreads, NW = kRegThreads / 32;
+    static_assert(NW == kStreamWarps, "warp partials");
     DevState *st = P.st;
-    if (st->err) return;
-    const unsigned long long t = st->t, tn = t + 1;
+    __shared__ unsigned long long s_rn[2 * MM], s_t, s_pend;
+    __shared__ unsigned s_err, s_pnblk;
+    __shared__ double2 s_w[C64 ? 1 : MM * MM];
+    __shared__ float4 s_wf[C64 ? MM * MM : 1];
+    __shared__ float4 s_rt[NW][MM];
+    // the state and both buffers' region sizes in one trip
+    if ((int)threadIdx.x < 2 * MM) s_rn[threadIdx.x] = __ldcg(P.reg_n + threadIdx.x);
+    if (threadIdx.x == 32) {
+        s_err = __ldcg(&st->err);
+        s_t = __ldcg(&st->t);
+        s_pend = __ldcg(&st->rho_pending);
+        s_pnblk = __ldcg(&st->rho_nblk);
+    }
+    for (int i = threadIdx.x; i < MM * MM; i += NT) {
+        if constexpr (C64) s_wf[i] = P.wtabf[i];
+        else s_w[i] = P.wtab[i];
+    }
+    __syncthreads();
+    if (s_err) return;
+    const unsigned long long t = s_t, tn = t + 1;
     const int in = (int)(t & 1), outp = (int)(tn & 1), cs = (int)(tn % 3);
     const bool merge = tn >= (unsigned long long)P.dkmax;
     const long long G = P.region_cap;
-    __shared__ long long s_gb[MM + 1];
-    __shared__ double2 s_w[C64 ? 1 : MM * MM];
-    __shared__ float4 s_wf[MM * MM];
-    __shared__ float4 s_rt[kRegThreads / 32][MM];
-    __shared__ bool s_last;
-    if (threadIdx.x == 0) {
-        long long acc = 0;
-        const int gsz = merge ? MM : 1;
-        unsigned long long n_in = 0;
-        for (int r = 0; r < MM; ++r) {
-            const long long nr = (long long)__ldcg(&P.reg_n[in * MM + r]);
-            n_in += (unsigned long long)nr;
-            s_gb[r] = acc;
-            acc += nr / gsz;
-        }
-        const bool regular = n_in > 0 && (merge ? (P.reg_merge && n_in == P.full_n) : (P.reg_fill != 0));
-        s_gb[MM] = regular ? acc : -1;
+    // groups before region r (gs members each)
+    unsigned long long n_in = 0;
+#pragma unroll
+    for (int r = 0; r < MM; ++r) n_in += s_rn[in * MM + r];
+    int gs = 0;   // members of a group; 0: not a regular step
+    if (n_in > 0) {
+        if (!merge) gs = P.reg_fill ? 1 : 0;
+        else if (P.reg_merge && n_in == P.full_n) gs = MM;
+        else if (P.reg_merge && tn == (unsigned long long)P.dkmax && n_in == P.full_n / MM * (unsigned long long)P.nnz0) gs = P.nnz0;
     }
-    __syncthreads();
-    const long long ngroups = s_gb[MM];
-    if (ngroups < 0) {   // not a regular step: the tile kernel takes it
+    if (gs == 0) {   // the tile kernel takes it
         if (blockIdx.x == 0 && threadIdx.x == 0) st->reg_done = 0;
         return;
     }
-    if (blockIdx.x == 0) finish_pending_rho<C64>(P, st, MM);   // rho of the previous step
-    const int gs = merge ? MM : 1;
+    // every region holds as many groups, except at t = 0 (the nonzero
+    // elements of rho(0), one path each)
+    const unsigned long long nr0 = n_in / MM;
+    long long gpr = (long long)nr0;   // groups per region
+    if (gs == MM) gpr = (long long)(nr0 / MM);
+    else if (gs > 1) gpr = (long long)((nr0 >> 32) == 0 ? (unsigned)nr0 / (unsigned)gs : nr0 / (unsigned)gs);
+    const long long ngroups = t == 0 ? (long long)n_in / gs : gpr * MM;
+    const long long nchunk = (ngroups + 31) / 32;
+    const bool spare = nchunk < (long long)gridDim.x;
+    const unsigned active = spare ? (unsigned)nchunk : gridDim.x;   // blocks with groups
+    const unsigned arrivals = active + (spare ? 1u : 0u);
+    if (blockIdx.x >= arrivals) return;
+    // the last block to arrive publishes the step, for which it needs the
+    // step's counters only; every block then writes its partial of rho, which
+    // the next step's kernel (or a read-time finalisation) sums once this
+    // kernel has ended.  One acquire-release add releases the block's writes
+    // (ordered before it by the barrier) and acquires the others' in the last
+    // block.
+    auto arrive = [&]() {
+        __syncthreads();
+        if (threadIdx.x == 0 && atom_add_acq_rel_gpu(P.fin_count, 1u) == arrivals - 1) {
+            if (__ldcg(&st->err)) {   // a failed step is not published
+                *P.fin_count = 0;
+            } else {
+                st->rho_nblk = active;
+                st->rho_pending = tn;
+                StepCounts c;
+                c.groups = (unsigned long long)(merge ? ngroups : (long long)n_in);
+                c.n_out = (unsigned long long)ngroups * MM;
+                st->cnt_out[cs] = c.n_out;
+                st->cnt_groups[cs] = (unsigned long long)ngroups;
+                publish_step(P, st, tn, MM, c);
+            }
+        }
+    };
+    if (blockIdx.x == active) {   // the spare block: the previous step's rho
+        arrive();
+        if (s_pend) phase_finalize_stream<C64>(P, s_pend, (int)s_pnblk, MM);
+        return;
+    }
     const int n_act = (int)min(tn, (unsigned long long)P.dkmax);
     const int L_child = (int)min(tn + 1, (unsigned long long)P.dkmax);
     const unsigned long long wmask = (P.b * L_child >= 64) ? ~0ull : ((1ull << (P.b * L_child)) - 1ull);
@@ -1311,36 +1409,32 @@ __global__ void __launch_bounds__(kRegThreads, 3) k_stream_regular(Params P, int
     unsigned long long *keys_out = P.keys[outp];
     AmpT *amps_out = static_cast<AmpT *>(P.amps[outp]);
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    for (int i = threadIdx.x; i < MM * MM; i += NT) {
-        if constexpr (!C64) s_w[i] = P.wtab[i];
-        s_wf[i] = P.wtabf[i];
-    }
     Tab tab = tab_global(P, n_act, 0);
-    if (lut_smem && P.ndelta) {
+    const long long step_chunks = (long long)active * NW;
+    const long long chunk0 = (long long)(threadIdx.x >> 5) * active + blockIdx.x;
+    // the history tables pay for their copy once a warp takes a few groups
+    if (lut_smem && P.ndelta && nchunk > 2 * step_chunks) {
         const int n = P.nchunks * kLutEntries;
         if constexpr (C64) {
             float2 *hi = reinterpret_cast<float2 *>(s_dyn), *lo = hi + n;
-            for (int i = threadIdx.x; i < n; i += NT) {
-                hi[i] = __ldg(tab.hi + i);
-                lo[i] = __ldg(tab.lo + i);
+            for (int i = threadIdx.x; i < n / 2; i += NT) {
+                cp_async16(hi + 2 * i, tab.hi + 2 * i);
+                cp_async16(lo + 2 * i, tab.lo + 2 * i);
             }
             tab.hi = hi;
             tab.lo = lo;
         } else {
             double2 *et = reinterpret_cast<double2 *>(s_dyn);
-            for (int i = threadIdx.x; i < n * P.ndelta; i += NT) et[i] = __ldg(tab.et + i);
+            for (int i = threadIdx.x; i < n * P.ndelta; i += NT) cp_async16(et + i, tab.et + i);
             tab.et = et;
         }
+        cp_async_wait_all();
+        __syncthreads();
     }
     if (blockIdx.x == 0) {
         if ((int)threadIdx.x < MM) P.reg_n[outp * MM + threadIdx.x] = (unsigned long long)ngroups;
-        if (threadIdx.x == 0) {
-            st->cnt_out[cs] = (unsigned long long)ngroups * MM;
-            st->cnt_groups[cs] = (unsigned long long)ngroups;
-            st->reg_done = tn + 1;
-        }
+        if (threadIdx.x == 0) st->reg_done = tn + 1;
     }
-    __syncthreads();
     constexpr bool kKahan = C64;
     typename X::AccT racc[MM], rcmp[MM];
 #pragma unroll
@@ -1356,11 +1450,30 @@ __global__ void __launch_bounds__(kRegThreads, 3) k_stream_regular(Params P, int
     };
     auto load = [&](long long g, Members &mb) {
         int r = 0;
-        while (r + 1 < MM && g >= s_gb[r + 1]) ++r;
-        const long long j = (g - s_gb[r]) * gs;
+        long long j = g;
+        if (t == 0) {
+            for (j = 0;; ++r) {   // the g-th nonempty region
+                if (s_rn[in * MM + r] && j++ == g) break;
+            }
+            j = 0;
+        } else {
+#pragma unroll
+            for (int k = 1; k < MM; ++k) {
+                if (j < gpr) break;
+                j -= gpr;
+                r = k;
+            }
+        }
+        j *= gs;
         mb.rk = __ldcs(keys_in + r * G + j);
         if (gs == 1) {
             mb.a[0] = __ldcs(amps_in + r * G + j);
+        } else if (gs < MM) {   // the first merge: nnz0 members
+#pragma unroll
+            for (int m = 0; m < MM; ++m) {
+                mb.a[m].x = mb.a[m].y = 0;
+                if (m < gs) mb.a[m] = __ldcs(amps_in + r * G + j + m);
+            }
         } else if constexpr (C64 && MM % 2 == 0) {
             const float4 *p4 = reinterpret_cast<const float4 *>(amps_in + r * G + j);
 #pragma unroll
@@ -1386,16 +1499,20 @@ __global__ void __launch_bounds__(kRegThreads, 3) k_stream_regular(Params P, int
             float sx = mb.a[0].x, sy = mb.a[0].y, ex = 0.f, ey = 0.f;
 #pragma unroll
             for (int m = 1; m < MM; ++m) {
-                two_sum_acc(sx, ex, mb.a[m].x);
-                two_sum_acc(sy, ey, mb.a[m].y);
+                if (m < gs) {
+                    two_sum_acc(sx, ex, mb.a[m].x);
+                    two_sum_acc(sy, ey, mb.a[m].y);
+                }
             }
             X::children_tab(P, tab, rk, make_float2(sx + ex, sy + ey), s_w, s_wf, v);
         } else {
             double sx = mb.a[0].x, sy = mb.a[0].y;
 #pragma unroll
             for (int m = 1; m < MM; ++m) {
-                sx += mb.a[m].x;
-                sy += mb.a[m].y;
+                if (m < gs) {
+                    sx += mb.a[m].x;
+                    sy += mb.a[m].y;
+                }
             }
             X::children_tab(P, tab, rk, make_double2(sx, sy), s_w, s_wf, v);
         }
@@ -1413,47 +1530,36 @@ __global__ void __launch_bounds__(kRegThreads, 3) k_stream_regular(Params P, int
             }
         }
     };
-    const long long stride = (long long)gridDim.x * NT;
     if (ngroups > G) {   // the outputs would not fit their regions
         if (threadIdx.x == 0) raise_err(st, kErrPaths);
     } else {
         // one group per thread at a time: three blocks of eight warps per SM
         // keep more bytes in flight than two groups per thread at two blocks
-        for (long long g = (long long)blockIdx.x * NT + threadIdx.x; g < ngroups; g += stride) {
-            Members m0;
-            load(g, m0);
-            group(g, m0);
-        }
-    }
-    // arrive first: the last block to arrive publishes the step, for which
-    // it needs the step's counters only; every block then writes its partial
-    // of rho, which the next step's block 0 (or a read-time finalisation)
-    // sums once this kernel has ended
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // one acquire-release add: releases this block's writes (ordered
-        // before it by the barrier), and the last block acquires the others'
-        s_last = atom_add_acq_rel_gpu(P.fin_count, 1u) == gridDim.x - 1;
-        if (s_last) {
-            if (__ldcg(&st->err)) {   // a failed step is not published
-                *P.fin_count = 0;
-            } else {
-                st->rho_nblk = gridDim.x;
-                st->rho_pending = tn;
-                publish_step(P, st, tn, MM, step_counts(P, st, tn));
+        for (long long ch = chunk0; ch < nchunk; ch += step_chunks) {
+            const long long g = ch * 32 + lane_id();
+            if (g < ngroups) {
+                Members m0;
+                load(g, m0);
+                group(g, m0);
             }
         }
     }
+    arrive();
     // block partials of rho(tn) and the children written by this block
-    float4 *mine = spart_of(P, tn, MM) + (size_t)blockIdx.x * MM;
     float2 lo[MM];
 #pragma unroll
     for (int k = 0; k < MM; ++k) lo[k] = C64 ? make_float2(-(float)rcmp[k].x, -(float)rcmp[k].y) : make_float2(0.f, 0.f);
-    block_rho_pair<MM, kRegThreads / 32, C64>(racc, lo, s_rt, mine);
+    block_rho_pair<MM, NW, C64>(racc, lo, s_rt, spart_of(P, tn, MM) + (size_t)blockIdx.x * MM);
     if (threadIdx.x == 0) {
-        long long mg = 0;
-        for (long long g0 = (long long)blockIdx.x * NT; g0 < ngroups; g0 += stride) mg += min((long long)NT, ngroups - g0);
+        // this block's chunks (every active-th), the last of all perhaps ragged
+        const long long nc = (nchunk - 1 - blockIdx.x) / active + 1;
+        long long mg = nc * 32;
+        if ((nchunk - 1) % active == blockIdx.x) mg -= nchunk * 32 - ngroups;
         scount_of(P, tn)[blockIdx.x] = mg * MM;
+    }
+    if (!spare && blockIdx.x == gridDim.x - 1) {   // no spare block: the previous step's rho
+        __syncthreads();
+        if (s_pend) phase_finalize_stream<C64>(P, s_pend, (int)s_pnblk, MM);
     }
 }
 
@@ -1629,10 +1735,13 @@ __device__ __forceinline__ unsigned long long ld_relaxed_gpu(const unsigned long
 // Output region c receives, in order, the children with newest point c of
 // all groups, so the next set is again sorted.  No atomics on the data.  The
 // last block to finish sums the blocks' partials of rho(t+1) and publishes
-// the step.  lut_smem: the history tables of this window length are copied
-// into shared memory once per block.
+// the step.  flags: kFlagLutSmem (the history tables of this window length
+// are copied into shared memory once per block), kFlagAfterRegular (the
+// regular kernel was launched for the same step and may have taken it).
+constexpr int kFlagLutSmem = 1, kFlagAfterRegular = 2;
 template <int M, bool C64, int NX, int S, bool BATCH>
-__device__ __forceinline__ void stream_step_body(const Params &P, int lut_smem) {
+__device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
+    const bool lut_smem = (flags & kFlagLutSmem) != 0;
     using X = Expander<M, C64>;
     using Lay = StreamLayout<M, C64, NX, S>;
     using AmpT = typename X::AmpT;
@@ -1650,9 +1759,9 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int lut_smem) 
     // several steps in one launch)
     if (__ldcg(&st->err)) return;
     const unsigned long long t = __ldcg(&st->t), tn = t + 1;
-    if (__ldcg(&st->reg_done) == tn) return;   // the regular kernel just took this step (its new t + 1)
+    // launched behind the regular kernel, which just took this step (its new t + 1)
+    if ((flags & kFlagAfterRegular) && __ldcg(&st->reg_done) == tn) return;
     if constexpr (BATCH) finish_pending_rho_batch(P, st, M * M, false);   // blocks b < n_inst: instance b
-    else if (blockIdx.x == 0) finish_pending_rho<C64>(P, st, M * M);   // rho of the previous step
     const int in = (int)(t & 1), outp = (int)(tn & 1), cs = (int)(tn % 3);
     const bool merge = tn >= (unsigned long long)P.dkmax;
     const unsigned long long pref = merge ? P.prefmask : ~0ull;   // filling: every path is its own group
@@ -1849,7 +1958,14 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int lut_smem) 
         if (threadIdx.x == 0) s_ticket = atomicAdd(&st->ticket[cs], 1u);
         __syncthreads();
         const long long ticket = s_ticket;
-        if (ticket >= ntiles) break;
+        if (ticket >= ntiles) {
+            // the first block without a tile sums the previous step's rho,
+            // beside the blocks that still have one (it has not arrived yet,
+            // so the mark it reads is the previous step's)
+            if constexpr (!BATCH)
+                if (ticket == ntiles) finish_pending_rho<C64>(P, st, M * M);
+            break;
+        }
         if (threadIdx.x == 0) s_any = 1;
         const int r = region_of(ticket);
         const long long e0 = (ticket - tile0_of(r)) * St;
@@ -2593,8 +2709,8 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int lut_smem) 
 
 template <int M, bool C64, int NX, int S>
 __global__ void __launch_bounds__(kStreamThreads, (M == 2 || (M == 3 && C64)) ? 2 : 1)
-    k_stream_step(Params P, int lut_smem) {
-    stream_step_body<M, C64, NX, S, false>(P, lut_smem);
+    k_stream_step(Params P, int flags) {
+    stream_step_body<M, C64, NX, S, false>(P, flags);
 }
 
 // Batched stream engine: nsteps steps of all instances, separated by
@@ -3399,9 +3515,10 @@ struct qp_ctx {
     bool use_stream = false;           // this propagation runs on the stream engine
     bool sym = false;                  // symmetric Trotter splitting (qp_set_end_points)
     qp::cplx eta00;                    // ... point 0's half-interval self coefficient
-    cudaGraphExec_t graph1 = nullptr;  // one-step graph for remainders
-    cudaGraphExec_t graph = nullptr;
-    bool graph_dirty = true;
+    cudaGraphExec_t graph1[3] = {};    // one-step graphs and graphs of graph_steps steps, by StepKind
+    cudaGraphExec_t graph[3] = {};
+    bool graph_dirty = true;           // none of them is current
+    bool reg_track = false;            // path counts of an unfiltered stream propagation known on the host (step_kind)
     bool use_graph = true;
     int64_t host_t = 0;                // steps enqueued since qp_set_rho0 (set from the device at every state read)
     void *hpin = nullptr;              // pinned host staging for rho reads (state + rows)
@@ -3421,6 +3538,14 @@ qp_status fail(qp_ctx *c, qp_status s, const std::string &msg) {
         cudaError_t e_ = (call);                                                              \
         if (e_ != cudaSuccess) return fail(ctx, QP_ERR_CUDA, std::string(#call ": ") + cudaGetErrorString(e_)); \
     } while (0)
+
+void drop_graphs(qp_ctx *c) {
+    for (int k = 0; k < 3; ++k) {
+        if (c->graph1[k]) cudaGraphExecDestroy(c->graph1[k]);
+        if (c->graph[k]) cudaGraphExecDestroy(c->graph[k]);
+        c->graph1[k] = c->graph[k] = nullptr;
+    }
+}
 
 constexpr int kStepKernels = 4;
 
@@ -3465,7 +3590,7 @@ size_t stream_lut_bytes(const qp_ctx *c, bool c64) {
 // ticket, so blocks beyond the co-resident count would only start after a
 // first wave), at most blocks_per_sm per SM and kMaxExpandBlocks in all.
 template <int M, bool C64, int NX, int S>
-cudaError_t launch_stream_kernel(qp_ctx *c, int blocks_per_sm) {
+cudaError_t launch_stream_kernel(qp_ctx *c, int blocks_per_sm, bool after_regular) {
     using Lay = StreamLayout<M, C64, NX, S>;
     const void *fn = (const void *)k_stream_step<M, C64, NX, S>;
     const size_t lutb = stream_lut_bytes(c, C64);
@@ -3485,7 +3610,8 @@ cudaError_t launch_stream_kernel(qp_ctx *c, int blocks_per_sm) {
         c->scache_res = nb;
     }
     const int g = std::min(c->nsm * std::min(blocks_per_sm, c->scache_res), kMaxExpandBlocks);
-    k_stream_step<M, C64, NX, S><<<g, kStreamThreads, sm, c->stream>>>(c->P, lutb ? 1 : 0);
+    const int flags = (lutb ? kFlagLutSmem : 0) | (after_regular ? kFlagAfterRegular : 0);
+    k_stream_step<M, C64, NX, S><<<g, kStreamThreads, sm, c->stream>>>(c->P, flags);
     return cudaGetLastError();
 }
 
@@ -3540,19 +3666,19 @@ cudaError_t launch_stream_batch(qp_ctx *c, int nsteps, bool coop) {
 }
 
 template <int M, bool C64, int NX>
-cudaError_t launch_stream_tile(qp_ctx *c) {
+cudaError_t launch_stream_tile(qp_ctx *c, bool after_regular) {
     switch (c->stream_tile) {
-        case 256: return launch_stream_kernel<M, C64, NX, 256>(c, c->bps_exp);
-        case 1024: return launch_stream_kernel<M, C64, NX, 1024>(c, c->bps_exp);
-        default: return launch_stream_kernel<M, C64, NX, 512>(c, c->bps_exp);
+        case 256: return launch_stream_kernel<M, C64, NX, 256>(c, c->bps_exp, after_regular);
+        case 1024: return launch_stream_kernel<M, C64, NX, 1024>(c, c->bps_exp, after_regular);
+        default: return launch_stream_kernel<M, C64, NX, 512>(c, c->bps_exp, after_regular);
     }
 }
 
-// The regular stream kernel (M = 2, no filter): every block resident, at
-// most kMaxExpandBlocks (block partials).
-template <bool C64>
+// The regular stream kernel (no filter): every block resident, at most
+// kMaxExpandBlocks (block partials).
+template <int M, bool C64>
 cudaError_t launch_stream_regular(qp_ctx *c) {
-    const void *fn = (const void *)k_stream_regular<2, C64>;
+    const void *fn = (const void *)k_stream_regular<M, C64>;
     const size_t lutb = stream_lut_bytes(c, C64);
     if (c->rcache_fn != fn || c->rcache_smem != lutb) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxStreamLut);
@@ -3566,20 +3692,38 @@ cudaError_t launch_stream_regular(qp_ctx *c) {
         c->rcache_res = nb;
     }
     const int g = std::min(c->nsm * c->rcache_res, kMaxExpandBlocks);
-    k_stream_regular<2, C64><<<g, kRegThreads, lutb, c->stream>>>(c->P, lutb ? 1 : 0);
+    k_stream_regular<M, C64><<<g, kRegThreads, lutb, c->stream>>>(c->P, lutb ? 1 : 0);
     return cudaGetLastError();
 }
 
-// One step of the stream engine: the regular kernel where the configuration
-// allows regular steps (events 0 -> 1), then the tile kernel (events 2 -> 3),
-// which returns at once when the regular kernel took the step.
+// The kernels that a step of the stream engine may need: the regular kernel,
+// the tile kernel, or the regular kernel and behind it the tile kernel, which
+// returns at once when the regular kernel took the step.
+enum StepKind { kStepBoth = 0, kStepRegular = 1, kStepTile = 2, kStepKinds = 3 };
+
+// Which of them step tn needs.  Without a filter every child survives, so
+// that the path counts, and with them the regular steps, are known here as
+// long as the mask has not changed since qp_set_rho0: every step of the
+// filling window, and with the full mask (and room for all keys) every step
+// (an empty launch behind the regular kernel costs 2 us of a 4 us step).
+StepKind step_kind(const qp_ctx *c, int64_t tn) {
+    const Params &P = c->P;
+    if (!c->use_stream || !P.reg_fill || c->cfg.M > 3) return kStepTile;
+    if (!c->reg_track) return kStepBoth;
+    if (P.nnz0 == 0) return kStepTile;
+    return tn < (int64_t)P.dkmax || P.reg_merge ? kStepRegular : kStepTile;
+}
+
+// One step of the stream engine (regular kernel: events 0 -> 1, tile kernel:
+// events 2 -> 3).
 template <int M, typename Amp>
-cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev) {
+cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind) {
     constexpr bool C64 = sizeof(Amp) == sizeof(float2);
+    const bool after_regular = kind == kStepBoth && c->P.reg_fill && M < 4;
     if (ev) cudaEventRecord(ev[0], c->stream);
-    if constexpr (M == 2) {
-        if (c->P.reg_fill) {
-            cudaError_t e = launch_stream_regular<C64>(c);
+    if constexpr (M < 4) {
+        if (kind == kStepRegular || after_regular) {
+            cudaError_t e = launch_stream_regular<M, C64>(c);
             if (e != cudaSuccess) return e;
         }
     }
@@ -3587,13 +3731,16 @@ cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev) {
         cudaEventRecord(ev[1], c->stream);
         cudaEventRecord(ev[2], c->stream);
     }
-    cudaError_t e;
+    cudaError_t e = cudaSuccess;
     if (c->P.n_inst > 1) {
         e = launch_stream_batch_t<M, C64>(c, 1, false);
-    } else if constexpr (M == 2) {
-        e = c->stream_nx == 4 ? launch_stream_tile<M, C64, 4>(c) : launch_stream_tile<M, C64, 1>(c);
-    } else {
-        e = launch_stream_tile<M, C64, 1>(c);
+    } else if (kind != kStepRegular) {
+        if constexpr (M == 2) {
+            e = c->stream_nx == 4 ? launch_stream_tile<M, C64, 4>(c, after_regular)
+                                  : launch_stream_tile<M, C64, 1>(c, after_regular);
+        } else {
+            e = launch_stream_tile<M, C64, 1>(c, after_regular);
+        }
     }
     if (e != cudaSuccess) return e;
     if (ev) {
@@ -3638,7 +3785,7 @@ cudaError_t launch_post_t(qp_ctx *c, cudaEvent_t *ev) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev = nullptr) {
+cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev = nullptr, StepKind kind = kStepBoth) {
     const bool c64 = c->cfg.precision == QP_C64;
     if (c->P.post) {
         switch (c->cfg.M) {
@@ -3649,9 +3796,9 @@ cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev = nullptr) {
     }
     if (c->use_stream) {
         switch (c->cfg.M) {
-            case 2: return c64 ? launch_stream_t<2, float2>(c, ev) : launch_stream_t<2, double2>(c, ev);
-            case 3: return c64 ? launch_stream_t<3, float2>(c, ev) : launch_stream_t<3, double2>(c, ev);
-            default: return c64 ? launch_stream_t<4, float2>(c, ev) : launch_stream_t<4, double2>(c, ev);
+            case 2: return c64 ? launch_stream_t<2, float2>(c, ev, kind) : launch_stream_t<2, double2>(c, ev, kind);
+            case 3: return c64 ? launch_stream_t<3, float2>(c, ev, kind) : launch_stream_t<3, double2>(c, ev, kind);
+            default: return c64 ? launch_stream_t<4, float2>(c, ev, kind) : launch_stream_t<4, double2>(c, ev, kind);
         }
     }
     switch (c->cfg.M) {
@@ -3961,8 +4108,7 @@ qp_status qp_create(const qp_config *cfg, void *d_workspace, size_t bytes, void 
 
 void qp_destroy(qp_ctx *ctx) {
     if (!ctx) return;
-    if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
-    if (ctx->graph1) cudaGraphExecDestroy(ctx->graph1);
+    drop_graphs(ctx);
     if (ctx->hpin) cudaFreeHost(ctx->hpin);
     delete ctx;
 }
@@ -4161,6 +4307,7 @@ qp_status qp_set_mask(qp_ctx *c, const int *positions, int n) {
         return fail(c, QP_ERR_STATE, "the running stream-engine propagation cannot take this mask (restart with "
                                      "qp_set_rho0 after choosing the merge-table engine)");
     }
+    if (c->mask != old) c->reg_track = false;
     c->graph_dirty = true;
     return QP_OK;
 }
@@ -4200,6 +4347,8 @@ qp_status qp_set_rho0(qp_ctx *c, const double *re, const double *im) {
                     (c->cfg.engine == QP_ENGINE_STREAM || (c->cfg.engine == QP_ENGINE_AUTO && c->stream_nx > 0));
     if (c->use_stream && c->P.region_cap < 1) return fail(c, QP_ERR_CAPACITY, "max_paths < 16 M*M (stream engine)");
     c->P.stream = c->use_stream ? 1 : 0;
+    c->P.nnz0 = (int)nnz;
+    c->reg_track = c->use_stream;
     c->graph_dirty = true;
     const size_t n = keys.size();
     const size_t ab = c->cfg.precision == QP_C64 ? sizeof(float2) : sizeof(double2);
@@ -4257,7 +4406,7 @@ qp_status qp_set_rho0(qp_ctx *c, const double *re, const double *im) {
     return QP_OK;
 }
 
-static qp_status capture_graph(qp_ctx *c, int steps, cudaGraphExec_t *out) {
+static qp_status capture_graph(qp_ctx *c, int steps, StepKind kind, cudaGraphExec_t *out) {
     if (*out) {
         cudaGraphExecDestroy(*out);
         *out = nullptr;
@@ -4265,7 +4414,7 @@ static qp_status capture_graph(qp_ctx *c, int steps, cudaGraphExec_t *out) {
     cudaGraph_t g;
     QP_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = cudaSuccess;
-    for (int s = 0; s < steps && le == cudaSuccess; ++s) le = launch_step(c);
+    for (int s = 0; s < steps && le == cudaSuccess; ++s) le = launch_step(c, nullptr, kind);
     cudaError_t ce = cudaStreamEndCapture(c->stream, &g);
     if (le != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(le));
     if (ce != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(ce));
@@ -4281,6 +4430,7 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
     if (!c->have_state) return fail(c, QP_ERR_STATE, "qp_set_rho0 must come before qp_step");
     if (c->failed) return fail(c, QP_ERR_STATE, "context holds a device error; call qp_set_rho0");
     if (nsteps == 0) return QP_OK;
+    const int64_t t0 = c->host_t;
     c->host_t += nsteps;
     if (c->use_persistent && !c->use_stream && !c->P.post) {
         const cudaError_t e = launch_persistent(c, nsteps);
@@ -4292,25 +4442,27 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
         if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("persistent launch: ") + cudaGetErrorString(e));
         return QP_OK;
     }
-    if (c->use_graph) {
-        if (c->graph_dirty || !c->graph1 || (c->graph_steps > 1 && !c->graph)) {
-            qp_status st = capture_graph(c, 1, &c->graph1);
-            if (st != QP_OK) return st;
-            if (c->graph_steps > 1) {
-                st = capture_graph(c, c->graph_steps, &c->graph);
-                if (st != QP_OK) return st;
-            }
-            c->graph_dirty = false;
-        }
-        int left = nsteps;
-        if (c->graph_steps > 1)
-            for (; left >= c->graph_steps; left -= c->graph_steps) QP_CUDA(c, cudaGraphLaunch(c->graph, c->stream));
-        for (; left > 0; --left) QP_CUDA(c, cudaGraphLaunch(c->graph1, c->stream));
-    } else {
-        for (int s = 0; s < nsteps; ++s) {
-            cudaError_t e = launch_step(c);
+    if (c->use_graph && c->graph_dirty) {
+        drop_graphs(c);
+        c->graph_dirty = false;
+    }
+    for (int s = 0; s < nsteps;) {
+        const StepKind kind = step_kind(c, t0 + s + 1);
+        if (!c->use_graph) {
+            const cudaError_t e = launch_step(c, nullptr, kind);
             if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
+            ++s;
+            continue;
         }
+        // as many steps as need the same kernels in one graph
+        const bool many = c->graph_steps > 1 && nsteps - s >= c->graph_steps && kind == step_kind(c, t0 + s + c->graph_steps);
+        cudaGraphExec_t &g = many ? c->graph[kind] : c->graph1[kind];
+        if (!g) {
+            const qp_status st = capture_graph(c, many ? c->graph_steps : 1, kind, &g);
+            if (st != QP_OK) return st;
+        }
+        QP_CUDA(c, cudaGraphLaunch(g, c->stream));
+        s += many ? c->graph_steps : 1;
     }
     return QP_OK;
 }

@@ -1,0 +1,91 @@
+"""The regular stream kernel (unfiltered steps) against the oracle: M = 2 and
+3, every number of nonzero elements of rho(0) (the members of a group at the
+first merge), windows from one point up, steps on both sides of the window's
+fill, and a mask taken up or dropped in mid-run (the step counts are then no
+longer known on the host)."""
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import iquapi
+
+pytestmark = pytest.mark.gpu
+
+
+def _rho0(M, nnz, seed):
+    rng = np.random.default_rng(seed)
+    r = W.random_density_matrix(rng, M)
+    keep = np.zeros(M * M, dtype=bool)
+    keep[[0] + list(1 + rng.permutation(M * M - 1)[:nnz - 1])] = True
+    return np.where(keep.reshape(M, M), r, 0.0)
+
+
+def _run(c, mask, rho0, parts, precision="fp64"):
+    from paper_2506_03127_gb300 import Propagator
+    p = Propagator(c["M"], c["dkmax"], c["dt"], c["q"], c["hs"], 0.0, precision, "stream", max_paths=1 << 18)
+    p.set_eta(c["eta"])
+    p.set_mask(mask)
+    p.set_rho0(rho0)
+    for n in parts:
+        p.step(n)
+    T = sum(parts)
+    out = p.rho(0, T + 1), p.stats(1, T)
+    p.close()
+    return out
+
+
+@pytest.mark.parametrize("M,dkmax,nnz", [(2, d, n) for d in (1, 2, 3, 6) for n in (1, 2, 3, 4)]
+                         + [(3, d, n) for d in (1, 2, 4) for n in (1, 2, 5, 9)])
+@pytest.mark.parametrize("precision", ["fp64", "c64"])
+def test_unfiltered_steps(M, dkmax, nnz, precision):
+    c = W.random_case(40 + dkmax, M, dkmax)
+    rho0, T = _rho0(M, nnz, 7 * nnz + dkmax), dkmax + 4
+    rho, st = _run(c, None, rho0, (1, T - 2, 1), precision)
+    ref = iquapi.propagate(M, c["q"], c["hs"], c["dt"], c["eta"], dkmax, None, 0.0, rho0, T)
+    # FP64: the bar of the other engine tests; complex64: 2^-24 per operation, a few tens of them per step
+    assert np.abs(rho - ref.rho).max() <= (1e-10 if precision == "fp64" else 2e-6 * max(1.0, np.abs(ref.rho).max()))
+    n = nnz
+    for t, row in enumerate(st, 1):
+        groups = n if t < dkmax or dkmax == 1 else n // (nnz if t == dkmax else M * M)
+        assert row[1] == groups and row[3] == groups * M * M
+        n = row[3]
+
+
+def test_steps_in_graphs_of_several_match():
+    """graph_steps > 1: runs of steps that need different kernels."""
+    from paper_2506_03127_gb300 import Propagator
+    c = W.random_case(51, 2, 5)
+    rho0 = _rho0(2, 1, 3)
+    for mask in (None, (0, 1, 2)):
+        out = []
+        for gs in (1, 4):
+            p = Propagator(2, 5, c["dt"], c["q"], c["hs"], 0.0, "fp64", "stream", max_paths=1 << 14)
+            p.set_eta(c["eta"])
+            p.set_mask(mask)
+            p.set_rho0(rho0)
+            p.set_tuning(graph_steps=gs)
+            p.step(3)
+            p.step(14)
+            out.append(p.rho(0, 18))
+            p.close()
+        assert np.array_equal(*out)
+
+
+@pytest.mark.parametrize("first,then", [(None, (0, 1, 2)), ((0, 1, 2), None)])
+def test_mask_changed_in_mid_run(first, then):
+    from paper_2506_03127_gb300 import Propagator
+    c = W.random_case(53, 2, 5)
+    rho0 = _rho0(2, 4, 5)
+    out = []
+    for engine in ("stream", "hash"):
+        p = Propagator(2, 5, c["dt"], c["q"], c["hs"], 0.0, "fp64", engine, max_paths=1 << 14)
+        p.set_eta(c["eta"])
+        p.set_mask(first)
+        p.set_rho0(rho0)
+        p.step(7)
+        p.set_mask(then)
+        p.step(6)
+        out.append((p.rho(0, 14), [r[3] for r in p.stats(1, 13)]))
+        p.close()
+    assert np.abs(out[0][0] - out[1][0]).max() <= 1e-10
+    assert out[0][1] == out[1][1]
