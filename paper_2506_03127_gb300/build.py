@@ -2,7 +2,7 @@
 
     python -m paper_2506_03127_gb300.build
 
-The four translation units (qp.cu, mlp.cu, wide.cu, host_numerics.cpp) are compiled in parallel, then linked into
+The translation units (qp.cu in seven parts, mlp.cu, wide.cu, host_numerics.cpp) are compiled in parallel, then linked into
 paper_2506_03127_gb300/libqp.so.  A rebuild happens only when a source is
 newer than the library (or force=True).
 """
@@ -22,6 +22,8 @@ BUILD = os.path.join(PKG, "_build")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["qp.cu", "mlp.cu", "wide.cu", "host_numerics.cpp"]
+# qp.cu is compiled once per unit: its tile kernels are spread over units 1 .. 6
+JOBS = [("qp.cu", u) for u in range(7)] + [(s, None) for s in SOURCES[1:]]
 HEADERS = ["internal.h"]
 
 
@@ -47,9 +49,12 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
     nvcc = _nvcc()
     common = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]
 
-    def compile_one(src):
-        obj = os.path.join(BUILD, src + ".o")
+    def compile_one(job):
+        src, unit = job
+        obj = os.path.join(BUILD, src + (".o" if unit is None else f".{unit}.o"))
         cmd = [nvcc, "-c", os.path.join(CSRC, src), "-o", obj] + common
+        if unit is not None:
+            cmd += [f"-DQP_UNIT={unit}"]
         if src.endswith(".cu"):
             cmd += ARCH + ["-lineinfo"]
             if ptxas_info:
@@ -61,8 +66,8 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
             print(r.stdout + r.stderr, file=sys.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(compile_one, SOURCES))
+    with ThreadPoolExecutor(max_workers=len(JOBS)) as ex:
+        objs = list(ex.map(compile_one, JOBS))
     tmp = LIB + ".tmp"
     cmd = [nvcc, "-shared", "-o", tmp] + objs + ARCH + ["-lcudart_static", "-lrt", "-lpthread", "-ldl"]
     r = subprocess.run(cmd, capture_output=True, text=True)

@@ -27,4 +27,17 @@ int eta_from_bath(const qp_bath &b, double dt, int n, std::vector<cplx> &eta);
 // Q(j h), j = 0 .. n-1: the double integral of the bath correlation from 0.
 int Q_from_bath(const qp_bath &b, double h, int n, std::vector<cplx> &Q);
 
+// A tile kernel of the stream engine (k_stream_step or k_stream_batch) and
+// the shared memory of its tile.
+struct StreamKernel {
+    const void *fn;
+    size_t bytes;
+};
+StreamKernel stream_kernel_m2_c64(int nx, int tile);
+StreamKernel stream_kernel_m2_fp64(int nx, int tile);
+StreamKernel stream_kernel_m3(bool c64, int tile);
+StreamKernel stream_kernel_m4(bool c64, int tile);
+StreamKernel stream_kernel_batch_m2(bool c64, int tile);
+StreamKernel stream_kernel_batch_m34(int M, bool c64, int tile);
+
 }  // namespace qp

@@ -63,6 +63,14 @@
 
 #include "internal.h"
 
+// This file is compiled once per QP_UNIT, in parallel: unit 0 holds
+// everything but the stream engine's tile kernels, whose instantiations take
+// most of the compile time and are spread over the other units, which only
+// export them (qp::stream_kernel_*).
+#ifndef QP_UNIT
+#define QP_UNIT 0
+#endif
+
 namespace {
 
 constexpr unsigned long long kEmpty = ~0ull;
@@ -1176,6 +1184,7 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand(Params P) {
     phase_expand<M, C64, kExpandThreads, BATCH>(P, t, n, merge, &st->cnt_out[tn % 3], rho_part_of(P, tn, M * M));
 }
 
+#if QP_UNIT == 0
 // Step finalisation of the multi-kernel path: block i finalises instance i;
 // the last block to finish publishes the step (counts, t, next counters).
 __global__ void __launch_bounds__(256) k_finalize(Params P, int MM, int nblk) {
@@ -1193,6 +1202,8 @@ __global__ void __launch_bounds__(256) k_finalize(Params P, int MM, int nblk) {
     if (!s_last || threadIdx.x != 0) return;
     publish_step(P, st, tn, MM, step_counts(P, st, tn));
 }
+
+#endif
 
 // Grid-wide barrier of the persistent kernel (all blocks are co-resident: the
 // kernel is launched cooperatively).  The wait is bounded: after
@@ -2728,6 +2739,60 @@ __global__ void __launch_bounds__(kStreamThreads, (M == 2 || (M == 3 && C64)) ? 
     }
 }
 
+// The tile kernels of this unit: kernel and bytes of its tile in shared
+// memory.  (Fixed part of the dynamic shared memory; the launch adds the
+// staged tables or the batch's sums.)
+template <int M, bool C64, bool BATCH>
+qp::StreamKernel stream_kernel_of(int nx, int tile) {
+    auto of = [](auto *fn, size_t bytes) { return qp::StreamKernel{(const void *)fn, bytes}; };
+    if constexpr (BATCH) {
+        (void)nx;
+        return tile == 1024 ? of(k_stream_batch<M, C64, 1024>, StreamLayout<M, C64, 1, 1024>::bytes)
+                            : of(k_stream_batch<M, C64, 512>, StreamLayout<M, C64, 1, 512>::bytes);
+    } else {
+        if constexpr (M == 2)
+            if (nx == 4) switch (tile) {
+                case 256: return of(k_stream_step<M, C64, 4, 256>, StreamLayout<M, C64, 4, 256>::bytes);
+                case 1024: return of(k_stream_step<M, C64, 4, 1024>, StreamLayout<M, C64, 4, 1024>::bytes);
+                default: return of(k_stream_step<M, C64, 4, 512>, StreamLayout<M, C64, 4, 512>::bytes);
+            }
+        switch (tile) {
+            case 256: return of(k_stream_step<M, C64, 1, 256>, StreamLayout<M, C64, 1, 256>::bytes);
+            case 1024: return of(k_stream_step<M, C64, 1, 1024>, StreamLayout<M, C64, 1, 1024>::bytes);
+            default: return of(k_stream_step<M, C64, 1, 512>, StreamLayout<M, C64, 1, 512>::bytes);
+        }
+    }
+}
+
+#if QP_UNIT != 0
+}  // namespace
+
+namespace qp {
+#if QP_UNIT == 1
+StreamKernel stream_kernel_m2_c64(int nx, int tile) { return stream_kernel_of<2, true, false>(nx, tile); }
+#elif QP_UNIT == 2
+StreamKernel stream_kernel_m2_fp64(int nx, int tile) { return stream_kernel_of<2, false, false>(nx, tile); }
+#elif QP_UNIT == 3
+StreamKernel stream_kernel_m3(bool c64, int tile) {
+    return c64 ? stream_kernel_of<3, true, false>(1, tile) : stream_kernel_of<3, false, false>(1, tile);
+}
+#elif QP_UNIT == 4
+StreamKernel stream_kernel_m4(bool c64, int tile) {
+    return c64 ? stream_kernel_of<4, true, false>(1, tile) : stream_kernel_of<4, false, false>(1, tile);
+}
+#elif QP_UNIT == 5
+StreamKernel stream_kernel_batch_m2(bool c64, int tile) {
+    return c64 ? stream_kernel_of<2, true, true>(1, tile) : stream_kernel_of<2, false, true>(1, tile);
+}
+#elif QP_UNIT == 6
+StreamKernel stream_kernel_batch_m34(int M, bool c64, int tile) {
+    if (M == 3) return c64 ? stream_kernel_of<3, true, true>(1, tile) : stream_kernel_of<3, false, true>(1, tile);
+    return c64 ? stream_kernel_of<4, true, true>(1, tile) : stream_kernel_of<4, false, true>(1, tile);
+}
+#endif
+}  // namespace qp
+#else   // QP_UNIT == 0: the rest of the file
+
 // The kernels' FP32 -> FP64 widening over an array (test hook).
 __global__ void k_widen(const float *in, double *out, long long n) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -3586,92 +3651,68 @@ size_t stream_lut_bytes(const qp_ctx *c, bool c64) {
     return b <= kMaxStreamLut ? b : 0;
 }
 
+// The tile kernel of this context (instantiated in the other units).
+qp::StreamKernel stream_kernel(const qp_ctx *c) {
+    const bool c64 = c->cfg.precision == QP_C64;
+    const int M = c->cfg.M, tile = c->stream_tile;
+    if (c->P.n_inst > 1)
+        return M == 2 ? qp::stream_kernel_batch_m2(c64, tile) : qp::stream_kernel_batch_m34(M, c64, tile);
+    if (M == 2) return c64 ? qp::stream_kernel_m2_c64(c->stream_nx, tile) : qp::stream_kernel_m2_fp64(c->stream_nx, tile);
+    return M == 3 ? qp::stream_kernel_m3(c64, tile) : qp::stream_kernel_m4(c64, tile);
+}
+
+// Co-resident blocks per SM of a stream kernel at a dynamic shared memory
+// size, and the function's limit (a property of the function: set to the
+// most any context may ask for, so that contexts do not undo each other).
+cudaError_t stream_residency(qp_ctx *c, const void *fn, size_t sm, size_t sm_most) {
+    if (c->scache_fn == fn && c->scache_smem == sm) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_most);
+    if (e != cudaSuccess) return e;
+    int nb = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kStreamThreads, sm);
+    if (e != cudaSuccess) return e;
+    if (nb < 1) return cudaErrorInvalidConfiguration;
+    c->scache_fn = fn;
+    c->scache_smem = sm;
+    c->scache_res = nb;
+    return cudaSuccess;
+}
+
 // Grid of the stream kernel: every block resident (tiles are taken by
 // ticket, so blocks beyond the co-resident count would only start after a
-// first wave), at most blocks_per_sm per SM and kMaxExpandBlocks in all.
-template <int M, bool C64, int NX, int S>
-cudaError_t launch_stream_kernel(qp_ctx *c, int blocks_per_sm, bool after_regular) {
-    using Lay = StreamLayout<M, C64, NX, S>;
-    const void *fn = (const void *)k_stream_step<M, C64, NX, S>;
-    const size_t lutb = stream_lut_bytes(c, C64);
-    const size_t sm = Lay::bytes + lutb;
-    if (c->scache_fn != fn || c->scache_smem != sm) {
-        // the attribute is a property of the function: set it to the most
-        // any context may ask for, so that contexts do not undo each other
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(Lay::bytes + kMaxStreamLut));
-        if (e != cudaSuccess) return e;
-        int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kStreamThreads, sm);
-        if (e != cudaSuccess) return e;
-        if (nb < 1) return cudaErrorInvalidConfiguration;
-        c->scache_fn = fn;
-        c->scache_smem = sm;
-        c->scache_res = nb;
-    }
-    const int g = std::min(c->nsm * std::min(blocks_per_sm, c->scache_res), kMaxExpandBlocks);
-    const int flags = (lutb ? kFlagLutSmem : 0) | (after_regular ? kFlagAfterRegular : 0);
-    k_stream_step<M, C64, NX, S><<<g, kStreamThreads, sm, c->stream>>>(c->P, flags);
-    return cudaGetLastError();
+// first wave), at most bps_exp per SM and kMaxExpandBlocks in all.
+cudaError_t launch_stream_tile(qp_ctx *c, bool after_regular) {
+    const qp::StreamKernel k = stream_kernel(c);
+    const size_t lutb = stream_lut_bytes(c, c->cfg.precision == QP_C64);
+    const size_t sm = k.bytes + lutb;
+    const cudaError_t e = stream_residency(c, k.fn, sm, k.bytes + kMaxStreamLut);
+    if (e != cudaSuccess) return e;
+    const int g = std::min(c->nsm * std::min(c->bps_exp, c->scache_res), kMaxExpandBlocks);
+    int flags = (lutb ? kFlagLutSmem : 0) | (after_regular ? kFlagAfterRegular : 0);
+    void *args[] = {(void *)&c->P, (void *)&flags};
+    return cudaLaunchKernel(k.fn, dim3(g), dim3(kStreamThreads), args, sm, c->stream);
 }
 
 // Batched stream kernel: an ordinary launch of one step (every block
-// resident, at most blocks_per_sm per SM), or (coop) one cooperative launch
-// of nsteps steps over at most persistent_blocks co-resident blocks.
+// resident, at most bps_exp per SM), or (coop) one cooperative launch of
+// nsteps steps over at most persistent_blocks co-resident blocks.
 // Dynamic shared memory: the tile buffers, then the per-instance sums and
 // the regions' first tiles.
-template <int M, bool C64, int S>
-cudaError_t launch_stream_batch_kernel(qp_ctx *c, int nsteps, bool coop) {
-    using Lay = StreamLayout<M, C64, 1, S>;
-    constexpr int MM = M * M;
-    const void *fn = (const void *)k_stream_batch<M, C64, S>;
-    auto extra = [](int ni) { return Lay::a16((size_t)ni * (MM + 1) * 16) + ((size_t)ni * MM + 1) * 4; };
-    const size_t sm = Lay::bytes + extra(c->P.n_inst);
-    if (c->scache_fn != fn || c->scache_smem != sm) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(Lay::bytes + extra(kMaxInst)));
-        if (e != cudaSuccess) return e;
-        int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kStreamThreads, sm);
-        if (e != cudaSuccess) return e;
-        if (nb < 1) return cudaErrorInvalidConfiguration;
-        c->scache_fn = fn;
-        c->scache_smem = sm;
-        c->scache_res = nb;
-    }
+cudaError_t launch_stream_batch(qp_ctx *c, int nsteps, bool coop) {
+    const int MM = c->cfg.M * c->cfg.M;
+    const qp::StreamKernel k = stream_kernel(c);
+    auto extra = [MM](int ni) { return (((size_t)ni * (MM + 1) * 16 + 15) & ~(size_t)15) + ((size_t)ni * MM + 1) * 4; };
+    const size_t sm = k.bytes + extra(c->P.n_inst);
+    const cudaError_t e = stream_residency(c, k.fn, sm, k.bytes + extra(kMaxInst));
+    if (e != cudaSuccess) return e;
+    void *args[] = {(void *)&c->P, (void *)&nsteps};
     if (coop) {
         const int g = std::min(std::min(c->persist_grid, c->nsm * c->scache_res), kMaxExpandBlocks);
-        Params P = c->P;
-        void *args[] = {(void *)&P, (void *)&nsteps};
-        return cudaLaunchCooperativeKernel(fn, dim3(g), dim3(kStreamThreads), args, sm, c->stream);
+        return cudaLaunchCooperativeKernel(k.fn, dim3(g), dim3(kStreamThreads), args, sm, c->stream);
     }
     const int g = std::min(c->nsm * std::min(c->bps_exp, c->scache_res), kMaxExpandBlocks);
-    k_stream_batch<M, C64, S><<<g, kStreamThreads, sm, c->stream>>>(c->P, 1);
-    return cudaGetLastError();
-}
-
-template <int M, bool C64>
-cudaError_t launch_stream_batch_t(qp_ctx *c, int nsteps, bool coop) {
-    return c->stream_tile == 1024 ? launch_stream_batch_kernel<M, C64, 1024>(c, nsteps, coop)
-                                  : launch_stream_batch_kernel<M, C64, 512>(c, nsteps, coop);
-}
-
-cudaError_t launch_stream_batch(qp_ctx *c, int nsteps, bool coop) {
-    const bool c64 = c->cfg.precision == QP_C64;
-    switch (c->cfg.M) {
-        case 2: return c64 ? launch_stream_batch_t<2, true>(c, nsteps, coop) : launch_stream_batch_t<2, false>(c, nsteps, coop);
-        case 3: return c64 ? launch_stream_batch_t<3, true>(c, nsteps, coop) : launch_stream_batch_t<3, false>(c, nsteps, coop);
-        default: return c64 ? launch_stream_batch_t<4, true>(c, nsteps, coop) : launch_stream_batch_t<4, false>(c, nsteps, coop);
-    }
-}
-
-template <int M, bool C64, int NX>
-cudaError_t launch_stream_tile(qp_ctx *c, bool after_regular) {
-    switch (c->stream_tile) {
-        case 256: return launch_stream_kernel<M, C64, NX, 256>(c, c->bps_exp, after_regular);
-        case 1024: return launch_stream_kernel<M, C64, NX, 1024>(c, c->bps_exp, after_regular);
-        default: return launch_stream_kernel<M, C64, NX, 512>(c, c->bps_exp, after_regular);
-    }
+    nsteps = 1;
+    return cudaLaunchKernel(k.fn, dim3(g), dim3(kStreamThreads), args, sm, c->stream);
 }
 
 // The regular stream kernel (no filter): every block resident, at most
@@ -3732,16 +3773,8 @@ cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind) {
         cudaEventRecord(ev[2], c->stream);
     }
     cudaError_t e = cudaSuccess;
-    if (c->P.n_inst > 1) {
-        e = launch_stream_batch_t<M, C64>(c, 1, false);
-    } else if (kind != kStepRegular) {
-        if constexpr (M == 2) {
-            e = c->stream_nx == 4 ? launch_stream_tile<M, C64, 4>(c, after_regular)
-                                  : launch_stream_tile<M, C64, 1>(c, after_regular);
-        } else {
-            e = launch_stream_tile<M, C64, 1>(c, after_regular);
-        }
-    }
+    if (c->P.n_inst > 1) e = launch_stream_batch(c, 1, false);
+    else if (kind != kStepRegular) e = launch_stream_tile(c, after_regular);
     if (e != cudaSuccess) return e;
     if (ev) {
         cudaEventRecord(ev[3], c->stream);
@@ -5250,3 +5283,4 @@ extern "C" qp_status qp_step_noalloc(const qp_config *cfg, const double *eta_re,
     }
     return QP_OK;
 }
+#endif   // QP_UNIT
