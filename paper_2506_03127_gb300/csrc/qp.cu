@@ -1574,30 +1574,12 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     }
 }
 
-// The groups of runs of at most this many stored paths are summed by one
-// owner thread each (stream engine); longer runs, which occur only while the
-// window fills, by shared FP64 atomics.
-constexpr int kOwnRun = 32;
-// A group sum formed in FP32 by its run's thread is stored as the float2 in
-// the low 8 bytes of its double2 slot and this signalling-NaN pattern in the
-// high 8 (arithmetic never yields a signalling NaN, so an FP64 atomic sum
-// cannot carry it).
-constexpr unsigned long long kOwnMark = 0x7FF00000514D0001ull;
-
-__device__ __forceinline__ void store_own_sum(double2 *slot, float2 S) {
-    reinterpret_cast<float2 *>(slot)[0] = S;
-    reinterpret_cast<unsigned long long *>(slot)[1] = kOwnMark;
-}
-
-// The C64 group sum of a slot: the FP32 sum of its run's thread, else the
-// FP64 atomic sum rounded once.
-__device__ __forceinline__ float2 group_sum_f2(double2 d) {
-    if ((unsigned long long)__double_as_longlong(d.y) == kOwnMark) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(d.x);
-        return make_float2(__uint_as_float((unsigned)b), __uint_as_float((unsigned)(b >> 32)));
-    }
-    return to_f2(d);
-}
+// The groups of runs of at most kOwnRun stored paths are summed by one owner
+// thread each (stream engine; the prefetch past the tile end holds as many),
+// runs of up to kWarpRun by a warp, longer ones by the block.
+constexpr int kOwnRun = 32, kWarpRun = 512;
+// A C64 group sum is the float2 in the low 8 bytes of its double2 slot.
+__device__ __forceinline__ void store_own_sum(double2 *slot, float2 S) { reinterpret_cast<float2 *>(slot)[0] = S; }
 
 // Dynamic shared memory of the stream kernel for a tile of S stored paths
 // (16-byte aligned arrays).  A tile holds at most NG = S + NX - 1 groups: every
@@ -1738,7 +1720,7 @@ __device__ __forceinline__ unsigned long long ld_relaxed_gpu(const unsigned long
 // paths past the tile end), find run heads; for NX > 1 give each sub-group
 // present a compact slot; sum each group and elect its representative, one
 // owner thread per group (runs start in the tile and may extend past it;
-// runs longer than 32 paths use shared FP64 atomics); compute
+// longer runs by a warp or the whole block); compute
 // the children of every group once, keep them in shared memory, count the
 // survivors per new point and accumulate rho(t+1); get the tile's output
 // offsets per region by a decoupled look-back (one warp, a window of
@@ -1814,6 +1796,11 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
     __shared__ float4 s_wrho[kTileAccS ? NW : 1][MM];   // M >= 3 single problems: per-warp sums of rho(t+1)
     __shared__ bool s_last;
     __shared__ int s_any;   // the block processed a tile
+    // runs of more than kOwnRun members that start in the tile, and the warps'
+    // sums of a run that the whole block adds
+    __shared__ int s_nlong, s_long[S / kOwnRun + 2];
+    __shared__ typename X::AccT s_lsum[NW][NX], s_lerr[C64 ? NW : 1][C64 ? NX : 1];
+    __shared__ WT s_lwm[NW][NX];
     __shared__ int s_lbfail;   // the tile's look-back gave up (timeout, or another block's error)
     const double tie_d = 1.0 - P.tie_rel;   // R4 window, once per thread
     const unsigned stall = __ldcg(&st->stall_tile);   // test hook (0 in normal operation)
@@ -2092,38 +2079,57 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
                 if (u < ept && i < cnt && sg >= 0) {
                     const unsigned x = xval(s_key[i]);
                     if (i - rs < 32) atomicOr(&s_xmask[sg * NX + x], 1u << (i - rs));
-                    else atomicOr(&s_xm[sg], 1u << x);
+                    else if (!(*(volatile unsigned *)&s_xm[sg] & (1u << x))) atomicOr(&s_xm[sg], 1u << x);
                 }
             }
         }
         if (warp == 0 && nseg > 0 && cnt == St) {
-            unsigned long long key = s_key[cnt + lane];
-            bool inrun = lane < s_ra_n && (key & pref) == plast;
-            for (int round = 0;; ++round) {
-                if (round > 0) {
-                    const long long i = e0 + ahead + lane;
-                    inrun = i < nr;
-                    if (inrun) {
-                        key = __ldcg(kin + i);
-                        inrun = (key & pref) == plast;
-                    }
+            const unsigned long long key = s_key[cnt + lane];
+            const bool inrun = lane < s_ra_n && (key & pref) == plast;
+            const unsigned inm = __ballot_sync(0xffffffffu, inrun);
+            const int nin = inm == 0xffffffffu ? 32 : __ffs(~inm) - 1;   // leading members of the run
+            if constexpr (NX > 1) {
+                if ((int)lane < nin) {
+                    const long long off = ahead + lane - s_seg[nseg - 1];
+                    if (off < 32) atomicOr(&s_xmask[(nseg - 1) * NX + xval(key)], 1u << off);
+                    else atomicOr(&s_xm[nseg - 1], 1u << xval(key));
                 }
-                const unsigned inm = __ballot_sync(0xffffffffu, inrun);
-                const int nin = inm == 0xffffffffu ? 32 : __ffs(~inm) - 1;   // leading members of the run
-                if constexpr (NX > 1) {
-                    if ((int)lane < nin) {
-                        const long long off = ahead + lane - s_seg[nseg - 1];
-                        if (off < 32) atomicOr(&s_xmask[(nseg - 1) * NX + xval(key)], 1u << off);
-                        else atomicOr(&s_xm[nseg - 1], 1u << xval(key));
+            }
+            ahead += nin;
+            if (nin == 32) {
+                // the run goes on past the prefetch: its members are
+                // contiguous, so the end is found by 32 probes per round at
+                // strides 32, 1024, ... and back to 1 (one 32-member round
+                // after the other took 0.7 us per 32 members)
+                long long stride = 32;
+                for (bool up = true;;) {
+                    const long long i = e0 + ahead + ((long long)lane + 1) * stride - 1;
+                    const bool in = i < nr && (__ldcg(kin + i) & pref) == plast;
+                    const unsigned m = __ballot_sync(0xffffffffu, in);
+                    const int k = m == 0xffffffffu ? 32 : __ffs(~m) - 1;
+                    ahead += k * stride;
+                    if (k == 32 && up) {
+                        stride *= 32;
+                        continue;
                     }
+                    up = false;
+                    if (stride == 1) break;
+                    stride /= 32;
                 }
-                ahead += nin;
-                if (nin < 32) break;
             }
         }
         if (threadIdx.x == 0) s_ahead = ahead;
         __syncthreads();
         ahead = s_ahead;
+        if constexpr (NX > 1) {
+            if (ahead > cnt + 32) {   // sub-groups among the members past the prefetch
+                unsigned bits = 0;
+                for (long long i = cnt + 32 + threadIdx.x; i < ahead; i += NT) bits |= 1u << xval(__ldcg(kin + e0 + i));
+                bits = __reduce_or_sync(0xffffffffu, bits);
+                if (lane == 0 && bits) atomicOr(&s_xm[nseg - 1], bits);
+                __syncthreads();
+            }
+        }
         // compact slots: sub-groups of run sg are slots sb[sg] + rank of x
         int ngroups = nseg;
         if constexpr (NX > 1) {
@@ -2249,27 +2255,208 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
                 s_grep[sl] = kmin;
             }
         }
-        // longer runs (only while the window fills): every member adds to its
-        // group in FP64 with shared atomics (consecutive members of a thread
-        // in the same slot combined first), then, after a barrier, the members
-        // within the tie window compete for the representative
-        if (__syncthreads_or(any_long)) {
-            auto run_long = [&](int g) -> bool {
-                if constexpr (!kOwners) return true;
+        // runs of more than kOwnRun members (mostly at the first merge, when
+        // the whole filled window collapses onto P'): up to kWarpRun members
+        // by one warp, longer ones by the block, the members dealt to the
+        // lanes.  Pass 1 adds them per sub-group (C64: FP32 TwoSum pairs
+        // merged error-free and rounded once, FP64: FP64) and takes the
+        // largest weights, pass 2 elects the representatives.  Members past
+        // the tile and its prefetch are read from global memory.  (Shared FP64
+        // atomics, a compare-and-swap loop under contention, with one warp
+        // for the members past the tile end, took 1.42 ms for the first merge
+        // of the headline model (7.7e5 paths, c64) and 7.5 ms for the chain's
+        // (3.9e7 paths).)
+        const bool any_runs = __syncthreads_or(any_long);
+        if (any_runs) {
+            if (threadIdx.x == 0) s_nlong = 0;
+            __syncthreads();
+            for (int g = threadIdx.x; g < nseg; g += NT) {
                 const long long b1 = g + 1 < nseg ? (long long)s_seg[g + 1] : ahead;
-                return b1 - s_seg[g] > kOwnRun;
+                if (b1 - s_seg[g] > kOwnRun) s_long[atomicAdd(&s_nlong, 1)] = g;
+            }
+            __syncthreads();
+            const int nlong = s_nlong;
+            const int in_tile = cnt + (cnt == St ? (int)s_ra_n : 0);   // entries in shared memory
+            using AccT = typename X::AccT;
+            // this lane's members m0, m0 + step, ... of run g
+            auto each = [&](int g, int m0, int step, auto &&f) {
+                const int b0 = s_seg[g];
+                const long long b1 = g + 1 < nseg ? (long long)s_seg[g + 1] : ahead;
+                const long long bs = b1 < in_tile ? b1 : in_tile;
+                long long i = b0 + m0;
+                for (; i < bs; i += step) f(s_key[i], s_amp[i]);
+                for (; i + 3 * (long long)step < b1; i += 4 * (long long)step) {
+                    unsigned long long k[4];
+                    AmpT a[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        k[u] = __ldcg(kin + e0 + i + u * (long long)step);
+                        a[u] = __ldcg(ain + e0 + i + u * (long long)step);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) f(k[u], a[u]);
+                }
+                for (; i < b1; i += step) f(__ldcg(kin + e0 + i), __ldcg(ain + e0 + i));
             };
-            const bool last_long = nseg > 0 && run_long(nseg - 1);
+            // warp sums and largest weights per sub-group (in every lane)
+            auto warp_sums = [&](int g, int m0, int step, AccT *sh, AccT *se, WT *wmx) {
+#pragma unroll
+                for (int x = 0; x < NX; ++x) {
+                    sh[x].x = sh[x].y = 0;
+                    se[x].x = se[x].y = 0;
+                    wmx[x] = 0;
+                }
+                each(g, m0, step, [&](unsigned long long key, const AmpT &a) {
+                    const unsigned xv = xval(key);
+                    const WT wb = weight_bits(a);
+#pragma unroll
+                    for (int x = 0; x < NX; ++x)
+                        if (NX == 1 || xv == (unsigned)x) {
+                            if constexpr (C64) {
+                                two_sum_acc(sh[x].x, se[x].x, a.x);
+                                two_sum_acc(sh[x].y, se[x].y, a.y);
+                            } else {
+                                sh[x].x += a.x;
+                                sh[x].y += a.y;
+                            }
+                            wmx[x] = wb > wmx[x] ? wb : wmx[x];
+                        }
+                });
+#pragma unroll
+                for (int x = 0; x < NX; ++x) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        if constexpr (C64) {
+                            const float bx = __shfl_xor_sync(0xffffffffu, sh[x].x, o), by = __shfl_xor_sync(0xffffffffu, sh[x].y, o);
+                            se[x].x += __shfl_xor_sync(0xffffffffu, se[x].x, o);
+                            se[x].y += __shfl_xor_sync(0xffffffffu, se[x].y, o);
+                            two_sum_acc(sh[x].x, se[x].x, bx);
+                            two_sum_acc(sh[x].y, se[x].y, by);
+                        } else {
+                            sh[x].x += __shfl_xor_sync(0xffffffffu, sh[x].x, o);
+                            sh[x].y += __shfl_xor_sync(0xffffffffu, sh[x].y, o);
+                        }
+                        const WT w = __shfl_xor_sync(0xffffffffu, wmx[x], o);
+                        wmx[x] = w > wmx[x] ? w : wmx[x];
+                    }
+                }
+            };
+            // smallest key within the tie window, per sub-group (in every lane)
+            auto warp_reps = [&](int g, int m0, int step, const WT *wmx, unsigned long long *kmin) {
+#pragma unroll
+                for (int x = 0; x < NX; ++x) kmin[x] = kEmpty;
+                each(g, m0, step, [&](unsigned long long key, const AmpT &a) {
+                    const unsigned xv = xval(key);
+                    const WT wb = weight_bits(a);
+#pragma unroll
+                    for (int x = 0; x < NX; ++x)
+                        if ((NX == 1 || xv == (unsigned)x) && within_tie(wb, wmx[x]) && key < kmin[x]) kmin[x] = key;
+                });
+#pragma unroll
+                for (int x = 0; x < NX; ++x)
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const unsigned long long k = __shfl_xor_sync(0xffffffffu, kmin[x], o);
+                        kmin[x] = k < kmin[x] ? k : kmin[x];
+                    }
+            };
+            auto slot = [&](int g, int x) -> int {   // -1: the run has no such sub-group
+                if constexpr (NX > 1) {
+                    const unsigned m = s_xm[g];
+                    return (m >> x) & 1u ? s_sb[g] + __popc(m & ((1u << x) - 1u)) : -1;
+                } else {
+                    return g;
+                }
+            };
+            auto put_sum = [&](int sl, const AccT &sh, const AccT &se) {
+                if constexpr (C64) store_own_sum(s_gS + sl, make_float2(sh.x + se.x, sh.y + se.y));
+                else s_gS[sl] = make_double2(sh.x, sh.y);
+            };
+            auto length = [&](int g) { return (g + 1 < nseg ? (long long)s_seg[g + 1] : ahead) - s_seg[g]; };
+            for (int l = (int)warp; l < nlong; l += NW) {
+                const int g = s_long[l];
+                if (length(g) > kWarpRun) continue;
+                AccT sh[NX], se[NX];
+                WT wmx[NX];
+                unsigned long long kmin[NX];
+                warp_sums(g, (int)lane, 32, sh, se, wmx);
+                warp_reps(g, (int)lane, 32, wmx, kmin);
+                if (lane == 0) {
+#pragma unroll
+                    for (int x = 0; x < NX; ++x) {
+                        const int sl = slot(g, x);
+                        if (sl >= 0) {
+                            put_sum(sl, sh[x], se[x]);
+                            s_grep[sl] = kmin[x];
+                        }
+                    }
+                }
+            }
+            for (int l = 0; l < nlong; ++l) {   // block-uniform
+                const int g = s_long[l];
+                if (length(g) <= kWarpRun) continue;
+                AccT sh[NX], se[NX];
+                WT wmx[NX];
+                unsigned long long kmin[NX];
+                warp_sums(g, (int)threadIdx.x, NT, sh, se, wmx);
+                if (lane == 0) {
+#pragma unroll
+                    for (int x = 0; x < NX; ++x) {
+                        s_lsum[warp][x] = sh[x];
+                        if constexpr (C64) s_lerr[warp][x] = se[x];
+                        s_lwm[warp][x] = wmx[x];
+                    }
+                }
+                __syncthreads();
+#pragma unroll
+                for (int x = 0; x < NX; ++x) {   // every thread: the warps in order
+                    sh[x] = s_lsum[0][x];
+                    if constexpr (C64) se[x] = s_lerr[0][x];
+                    wmx[x] = s_lwm[0][x];
+                    for (int w = 1; w < NW; ++w) {
+                        if constexpr (C64) {
+                            se[x].x += s_lerr[w][x].x;
+                            se[x].y += s_lerr[w][x].y;
+                            two_sum_acc(sh[x].x, se[x].x, s_lsum[w][x].x);
+                            two_sum_acc(sh[x].y, se[x].y, s_lsum[w][x].y);
+                        } else if (threadIdx.x == 0) {
+                            sh[x].x += s_lsum[w][x].x;
+                            sh[x].y += s_lsum[w][x].y;
+                        }
+                        wmx[x] = s_lwm[w][x] > wmx[x] ? s_lwm[w][x] : wmx[x];
+                    }
+                }
+                warp_reps(g, (int)threadIdx.x, NT, wmx, kmin);
+#pragma unroll
+                for (int x = 0; x < NX; ++x) {
+                    const int sl = slot(g, x);
+                    if (sl < 0) continue;
+                    if (threadIdx.x == 0) put_sum(sl, sh[x], se[x]);
+                    if (lane == 0 && kmin[x] != kEmpty) atomicMin(&s_grep[sl], kmin[x]);
+                }
+                __syncthreads();
+            }
+        }
+        // FP64 sub-groups in short runs: every member adds to its group with
+        // shared FP64 atomics (consecutive members of a thread in the same
+        // slot combined first), then, after a barrier, the members within
+        // the tie window compete for the representative
+        if (!kOwners && any_runs) {
+            auto short_run = [&](int g) -> bool {
+                const long long b1 = g + 1 < nseg ? (long long)s_seg[g + 1] : ahead;
+                return b1 - s_seg[g] <= kOwnRun;
+            };
+            const bool last_short = nseg > 0 && short_run(nseg - 1);
             {
                 int sg = segbase, cur = -1;
-                bool lng = sg >= 0 && run_long(sg);
+                bool shrt = sg >= 0 && short_run(sg);
                 double ax = 0.0, ay = 0.0;
                 WT wmx = 0;
 #pragma unroll
                 for (int u = 0; u < EPT; ++u) {
                     const int i = threadIdx.x * ept + u;
-                    if (hmask & (1u << u)) lng = run_long(++sg);
-                    if (u < ept && i < cnt && lng) {
+                    if (hmask & (1u << u)) shrt = short_run(++sg);
+                    if (u < ept && i < cnt && shrt) {
                         const AmpT a = s_amp[i];
                         const int sl = slot_of(sg, s_key[i]);
                         const WT wb = weight_bits(a);
@@ -2296,36 +2483,25 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
                     atomicMax(&s_wm[cur], wmx);
                 }
             }
-            if (warp == 0 && last_long && ahead > cnt) {   // members of the last run past the tile end
-                for (long long base = cnt; base < ahead; base += 32) {
-                    const long long i = base + lane;
-                    if (i < ahead) {
-                        unsigned long long key;
-                        AmpT a;
-                        if (base == cnt) {
-                            key = s_key[cnt + lane];
-                            a = s_amp[cnt + lane];
-                        } else {
-                            key = __ldcg(kin + e0 + i);
-                            a = __ldcg(ain + e0 + i);
-                        }
-                        const int sl = slot_of(nseg - 1, key);
-                        atomicAdd(&s_gS[sl].x, to_d(a.x));
-                        atomicAdd(&s_gS[sl].y, to_d(a.y));
-                        atomicMax(&s_wm[sl], weight_bits(a));
-                    }
-                }
+            // a short last run's members past the tile end are in the prefetch
+            const bool tail = warp == 0 && last_short && cnt + (int)lane < ahead;
+            if (tail) {
+                const AmpT a = s_amp[cnt + lane];
+                const int sl = slot_of(nseg - 1, s_key[cnt + lane]);
+                atomicAdd(&s_gS[sl].x, to_d(a.x));
+                atomicAdd(&s_gS[sl].y, to_d(a.y));
+                atomicMax(&s_wm[sl], weight_bits(a));
             }
             __syncthreads();
             {
                 int sg = segbase, cur = -1;
-                bool lng = sg >= 0 && run_long(sg);
+                bool shrt = sg >= 0 && short_run(sg);
                 unsigned long long kmin = kEmpty;
 #pragma unroll
                 for (int u = 0; u < EPT; ++u) {
                     const int i = threadIdx.x * ept + u;
-                    if (hmask & (1u << u)) lng = run_long(++sg);
-                    if (u < ept && i < cnt && lng) {
+                    if (hmask & (1u << u)) shrt = short_run(++sg);
+                    if (u < ept && i < cnt && shrt) {
                         const unsigned long long key = s_key[i];
                         const int sl = slot_of(sg, key);
                         if (sl != cur) {
@@ -2338,26 +2514,13 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
                 }
                 if (cur >= 0 && kmin != kEmpty) atomicMin(&s_grep[cur], kmin);
             }
-            if (warp == 0 && last_long && ahead > cnt) {
-                for (long long base = cnt; base < ahead; base += 32) {
-                    const long long i = base + lane;
-                    if (i < ahead) {
-                        unsigned long long key;
-                        AmpT a;
-                        if (base == cnt) {
-                            key = s_key[cnt + lane];
-                            a = s_amp[cnt + lane];
-                        } else {
-                            key = __ldcg(kin + e0 + i);
-                            a = __ldcg(ain + e0 + i);
-                        }
-                        const int sl = slot_of(nseg - 1, key);
-                        if (within_tie(weight_bits(a), s_wm[sl])) atomicMin(&s_grep[sl], key);
-                    }
-                }
+            if (tail) {
+                const unsigned long long key = s_key[cnt + lane];
+                const int sl = slot_of(nseg - 1, key);
+                if (within_tie(weight_bits(s_amp[cnt + lane]), s_wm[sl])) atomicMin(&s_grep[sl], key);
             }
-            __syncthreads();
         }
+        if (any_runs) __syncthreads();
         // pass A: children of a contiguous range of groups per thread, once;
         // survivors counted per new point, amplitudes kept in shared memory
         // for pass B (the first NSTG groups)
@@ -2375,9 +2538,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
             AmpT v[MM];
             if (rk != kEmpty) {
                 if constexpr (C64) {
-                    const float2 Sf = group_sum_f2(s_gS[g]);
-                    reinterpret_cast<float2 *>(s_gS)[2 * g] = Sf;   // for pass B, if not staged
-                    keep = X::children_tab(P, tab_t, rk, Sf, w_t, wf_t, v);
+                    keep = X::children_tab(P, tab_t, rk, reinterpret_cast<const float2 *>(s_gS)[2 * g], w_t, wf_t, v);
                 } else {
                     keep = X::children_tab(P, tab_t, rk, s_gS[g], w_t, wf_t, v);
                 }
