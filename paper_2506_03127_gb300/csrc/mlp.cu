@@ -34,6 +34,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -222,15 +223,20 @@ struct ParamBlock {
     int ldb, ldt;
 };
 
+// One parameter's moments and new value.  The products are fused as written,
+// so that every kernel that updates parameters rounds alike (a last bit of a
+// weight can move its BF16 copy by 2^-8).
+__device__ __forceinline__ float adam_value(float w, float &mom, float &vel, float g, float lr, float b1, float b2,
+                                            float eps, float bc1, float bc2) {
+    mom = __fmaf_rn(1.f - b1, g, __fmul_rn(b1, mom));
+    vel = __fmaf_rn(__fmul_rn(1.f - b2, g), g, __fmul_rn(b2, vel));
+    return w - lr * (mom / bc1) / (sqrtf(vel / bc2) + eps);
+}
+
 __global__ void k_adam(ParamBlock p, float lr, float b1, float b2, float eps, float bc1, float bc2) {
     const int n = p.rows * p.cols;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float g = p.g[i];
-        const float m = b1 * p.m[i] + (1.f - b1) * g;
-        const float v = b2 * p.v[i] + (1.f - b2) * g * g;
-        p.m[i] = m;
-        p.v[i] = v;
-        const float w = p.w[i] - lr * (m / bc1) / (sqrtf(v / bc2) + eps);
+        const float w = adam_value(p.w[i], p.m[i], p.v[i], p.g[i], lr, b1, b2, eps, bc1, bc2);
         p.w[i] = w;
         if (p.wb) {
             const int r = i / p.cols, c = i % p.cols;
@@ -248,6 +254,412 @@ __global__ void k_round_weights(ParamBlock p) {
         const __nv_bfloat16 wb = __float2bfloat16_rn(p.w[i]);
         p.wb[(size_t)r * p.ldb + c] = wb;
         p.wbT[(size_t)c * p.ldt + r] = wb;
+    }
+}
+
+// ---------------------------------------------------------------- training step
+//
+// Networks of up to 256 x 256 with up to 512 inputs and 32 outputs (the
+// surrogate's) take a training step in two launches:
+//   k_train_rows  32 rows of the batch per block through the whole network
+//                 and back: x, h1, h2, dy, dh2 stay in shared memory, the
+//                 FP32 tanh outputs in registers (the thread that formed h
+//                 forms dh at the same place), the weights stream through a
+//                 ring of 32-column chunks;
+//   k_train_update  the three weight gradients x^T dh1, h1^T dh2, h2^T dy in
+//                 one grid of 32 x 32 squares, operands read row-major and
+//                 transposed by ldmatrix, the batch in ascending order in
+//                 one accumulator per element (splitting the batch over
+//                 blocks was no faster and moves the last bits, which Adam's
+//                 first steps turn into the sign of small gradients), then
+//                 Adam on the square and its BF16 copies; the biases and the
+//                 loss in blocks of their own.
+// What bounds it: latency (2.2 GFLOP per epoch of the bench's fit, a few us
+// of the tensor cores).  One launch per product (18 per step), with
+// transposed copies stored two bytes at a time and column sums by global
+// atomics, took 435 us per step at 3312 rows of 258-256-256-8.
+constexpr int kTrRows = 32, kTrThreads = 256, kTrChunk = 32, kTrStages = 3;
+constexpr int kTrMaxW = 256, kTrMaxIn = 512, kTrMaxOut = 32;
+constexpr int kDwRows = 64, kDwStages = 4, kDwTile = 32, kDwThreads = 128;   // k_train_update
+
+__host__ __device__ inline bool train_fused(int d_in, int width, int d_out) {
+    return width <= kTrMaxW && d_in <= kTrMaxIn && d_out <= kTrMaxOut;
+}
+
+__device__ __forceinline__ void mlp_cp16(void *smem, const void *gmem, bool ok) {   // zeros where !ok
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem)), "l"(gmem), "r"(ok ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void mlp_cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void mlp_cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void ldmatrix_x4_t(unsigned &r0, unsigned &r1, unsigned &r2, unsigned &r3, const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                 : "r"(smem_u32(p)));
+}
+
+struct TrainArgs {
+    const float *x, *tgt;
+    int batch, d_in, width, d_out, K1, Kw, Ko;
+    const __nv_bfloat16 *w1t, *w2t, *w3t;   // W^T: [width][K1], [width][Kw], [d_out][Kw]
+    const __nv_bfloat16 *w2, *w3;           // W: [width][Kw], [width][Ko]
+    const float *b1, *b2, *b3;
+    __nv_bfloat16 *xb, *h1b, *h2b, *dyb, *dh2b, *dh1b;   // row-major, pads zero
+    float *colpart;   // [row blocks][2 width + d_out] partial bias gradients: b1, b2, b3
+    double *losspart; // [row blocks]
+};
+
+inline size_t train_rows_smem(int K1, int Kw, int Ko) {
+    return ((size_t)kTrRows * (K1 + 8) + (size_t)2 * kTrRows * (Kw + 8) + (size_t)kTrRows * (Ko + 8) +
+            (size_t)kTrMaxOut * (Kw + 8) + (size_t)kTrMaxW * (Ko + 8) + (size_t)kTrStages * kTrMaxW * (kTrChunk + 8)) * 2;
+}
+
+__global__ void __launch_bounds__(kTrThreads) k_train_rows(TrainArgs a) {
+    extern __shared__ __align__(16) unsigned char s_tr[];
+    const int l1 = a.K1 + 8, lw = a.Kw + 8, lo = a.Ko + 8;
+    constexpr int lc = kTrChunk + 8;
+    __nv_bfloat16 *sX = reinterpret_cast<__nv_bfloat16 *>(s_tr);
+    __nv_bfloat16 *sH1 = sX + kTrRows * l1, *sH2 = sH1 + kTrRows * lw;   // sH2: h2, then dh2
+    __nv_bfloat16 *sDY = sH2 + kTrRows * lw, *sW3T = sDY + kTrRows * lo, *sW3 = sW3T + kTrMaxOut * lw;
+    __nv_bfloat16 *sC = sW3 + kTrMaxW * lo;                              // weight chunks [stage][n][32]
+    __shared__ double s_loss[kTrThreads / 32];
+    __shared__ float s_db[2][kTrMaxOut];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
+    const int m0 = blockIdx.x * kTrRows, n0 = warp * 32;
+    const int width = a.width;
+    const bool busy = n0 < a.Kw;   // this warp's columns hold some of the layer
+    const int nc1 = a.K1 / kTrChunk, ncw = a.Kw / kTrChunk, ncs = nc1 + 2 * ncw;
+    // chunk c of the weights, in order of use: W1^T, W2^T, W2
+    auto issue = [&](int c) {
+        if (c < ncs) {
+            const __nv_bfloat16 *src;
+            int ld, k0;
+            if (c < nc1) { src = a.w1t; ld = a.K1; k0 = c * kTrChunk; }
+            else if (c < nc1 + ncw) { src = a.w2t; ld = a.Kw; k0 = (c - nc1) * kTrChunk; }
+            else { src = a.w2; ld = a.Kw; k0 = (c - nc1 - ncw) * kTrChunk; }
+            const int in = tid >> 2, ik = (tid & 3) * 8;   // rows in, in + 64, ...
+            __nv_bfloat16 *dst = sC + (c % kTrStages) * (kTrMaxW * lc) + in * lc + ik;
+            src += in * ld + k0 + ik;
+#pragma unroll
+            for (int u = 0; u < kTrMaxW; u += kTrThreads / 4)
+                if (u < a.Kw) {   // (rows in .. Kw: zeros past the width)
+                    const bool ok = in + u < width;
+                    mlp_cp16(dst + u * lc, ok ? src + u * ld : a.w1t, ok);
+                }
+        }
+        mlp_cp_commit();
+    };
+    for (int i = tid; i < kTrMaxOut * (a.Kw / 8); i += kTrThreads) {
+        const int n = i / (a.Kw / 8), kc = (i % (a.Kw / 8)) * 8;
+        const bool ok = n < a.d_out;
+        mlp_cp16(sW3T + n * lw + kc, a.w3t + (size_t)(ok ? n : 0) * a.Kw + kc, ok);
+    }
+    for (int i = tid; i < a.Kw * (a.Ko / 8); i += kTrThreads) {
+        const int n = i / (a.Ko / 8), kc = (i % (a.Ko / 8)) * 8;
+        const bool ok = n < width;
+        mlp_cp16(sW3 + n * lo + kc, a.w3 + (size_t)(ok ? n : 0) * a.Ko + kc, ok);
+    }
+    issue(0);   // (W3 in the same group)
+    issue(1);
+    // x rounded to BF16: shared memory and, for the weight gradient, global
+    // (a warp per row, two neighbouring columns per lane)
+    for (int r = warp; r < kTrRows; r += kTrThreads / 32) {
+        const int m = m0 + r;
+        const float *xr = a.x + (size_t)m * a.d_in;
+#pragma unroll 6
+        for (int k = 2 * lane; k < a.K1; k += 64) {
+            const float v0 = m < a.batch && k < a.d_in ? xr[k] : 0.f;
+            const float v1 = m < a.batch && k + 1 < a.d_in ? xr[k + 1] : 0.f;
+            const __nv_bfloat162 vb = __floats2bfloat162_rn(v0, v1);
+            *reinterpret_cast<__nv_bfloat162 *>(sX + r * l1 + k) = vb;
+            if (m < a.batch) *reinterpret_cast<__nv_bfloat162 *>(a.xb + (size_t)m * a.K1 + k) = vb;
+        }
+    }
+    for (int i = tid; i < kTrRows * lo; i += kTrThreads) sDY[i] = __float2bfloat16_rn(0.f);
+    if (tid < 2 * kTrMaxOut) s_db[tid / kTrMaxOut][tid % kTrMaxOut] = 0.f;
+    float acc[2][4][4], h1[2][4][4], h2[2][4][4];
+    auto zero = [&]() {
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.f;
+    };
+    // acc += A[32 rows][k .. k+16) B[n0 .. n0+32)[k .. k+16)^T
+    auto mma_step = [&](const __nv_bfloat16 *A, int lda, int ka, const __nv_bfloat16 *B, int ldb, int kb) {
+        unsigned af[2][4], bf[4][2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            ldmatrix_x4(af[i][0], af[i][1], af[i][2], af[i][3], A + (i * 16 + (lane & 15)) * lda + ka + (lane >> 4) * 8);
+#pragma unroll
+        for (int j = 0; j < 4; j += 2)
+            ldmatrix_x4(bf[j][0], bf[j][1], bf[j + 1][0], bf[j + 1][1],
+                        B + (n0 + j * 8 + ((lane >> 4) & 1) * 8 + (lane & 7)) * ldb + kb + ((lane >> 3) & 1) * 8);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], af[i][0], af[i][1], af[i][2], af[i][3], bf[j][0], bf[j][1]);
+    };
+    int c = 0;   // next chunk to use
+    // one layer: nk chunks against A (k ascending, as one launch per product)
+    auto layer = [&](const __nv_bfloat16 *A, int lda, int nk) {
+        zero();
+        for (int k = 0; k < nk; ++k, ++c) {
+            mlp_cp_wait<1>();
+            __syncthreads();   // chunk c is there, and every warp is done with chunk c - 1
+            issue(c + 2);
+            if (busy) {
+                const __nv_bfloat16 *B = sC + (size_t)(c % kTrStages) * kTrMaxW * lc;
+#pragma unroll
+                for (int kk = 0; kk < kTrChunk; kk += 16) mma_step(A, lda, k * kTrChunk + kk, B, lc, kk);
+            }
+        }
+    };
+    // element (i, j, r) of acc: row and column
+    auto row_of = [&](int i, int r) { return i * 16 + g + (r >= 2 ? 8 : 0); };
+    auto col_of = [&](int j, int r) { return n0 + j * 8 + 2 * tq + (r & 1); };
+    // a pair of neighbouring columns to shared memory and global
+    auto store2 = [&](__nv_bfloat16 *sm, __nv_bfloat16 *gm, int i, int j, int r, float v0, float v1) {
+        const int m = row_of(i, r), n = col_of(j, r);
+        const __nv_bfloat162 p = __floats2bfloat162_rn(v0, v1);
+        if (sm) *reinterpret_cast<__nv_bfloat162 *>(sm + m * lw + n) = p;
+        if (m0 + m < a.batch) *reinterpret_cast<__nv_bfloat162 *>(gm + (size_t)(m0 + m) * a.Kw + n) = p;
+    };
+    auto tanh_layer = [&](const float *bias, float (&h)[2][4][4], __nv_bfloat16 *sm, __nv_bfloat16 *gm) {
+        if (!busy) return;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int n = col_of(j, 0);
+            const float b0 = n < width ? bias[n] : 0.f, b1 = n + 1 < width ? bias[n + 1] : 0.f;
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int r = 0; r < 4; r += 2) {
+                    h[i][j][r] = n < width ? tanhf(acc[i][j][r] + b0) : 0.f;
+                    h[i][j][r + 1] = n + 1 < width ? tanhf(acc[i][j][r + 1] + b1) : 0.f;
+                    store2(sm, gm, i, j, r, h[i][j][r], h[i][j][r + 1]);
+                }
+        }
+    };
+    // acc * (1 - h^2): BF16 out, and the rows' FP32 sums per column
+    auto dtanh_layer = [&](const float (&h)[2][4][4], __nv_bfloat16 *sm, __nv_bfloat16 *gm, float *colsum) {
+        if (!busy) return;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int r = 0; r < 4; r += 2) {
+                    const float v0 = acc[i][j][r] * (1.f - h[i][j][r] * h[i][j][r]);
+                    const float v1 = acc[i][j][r + 1] * (1.f - h[i][j][r + 1] * h[i][j][r + 1]);
+                    s0 += v0;
+                    s1 += v1;
+                    store2(sm, gm, i, j, r, v0, v1);
+                }
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) {
+                s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            }
+            const int n = col_of(j, 0);
+            if (g == 0) {
+                if (n < width) colsum[n] = s0;
+                if (n + 1 < width) colsum[n + 1] = s1;
+            }
+        }
+    };
+    float *colp = a.colpart + (size_t)blockIdx.x * (2 * width + a.d_out);
+    layer(sX, l1, nc1);
+    tanh_layer(a.b1, h1, sH1, a.h1b);
+    layer(sH1, lw, ncw);   // (its first barrier orders sH1)
+    tanh_layer(a.b2, h2, sH2, a.h2b);
+    __syncthreads();
+    // layer 3 and the loss: warp (mt, nt) takes rows 16 mt, outputs 8 nt
+    double l = 0.0;
+    {
+        const int mt = warp & 1, nt = warp >> 1;
+        if (nt * 8 < a.d_out) {
+            float y[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int kk = 0; kk < a.Kw; kk += 16) {
+                unsigned a0, a1, a2, a3, b0, b1;
+                ldmatrix_x4(a0, a1, a2, a3, sH2 + (mt * 16 + (lane & 15)) * lw + kk + (lane >> 4) * 8);
+                ldmatrix_x2(b0, b1, sW3T + (nt * 8 + (lane & 7)) * lw + kk + ((lane >> 3) & 1) * 8);
+                mma_bf16(y, a0, a1, a2, a3, b0, b1);
+            }
+            const float scale = 2.f / (float)(a.batch * a.d_out);
+            float cs[2] = {0.f, 0.f};
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int mr = mt * 16 + g + (r >= 2 ? 8 : 0), m = m0 + mr, n = nt * 8 + 2 * tq + (r & 1);
+                if (m < a.batch && n < a.d_out) {
+                    const float e = (y[r] + a.b3[n]) - a.tgt[(size_t)m * a.d_out + n];
+                    l += (double)e * e;
+                    const float d = scale * e;
+                    const __nv_bfloat16 db = __float2bfloat16_rn(d);
+                    sDY[mr * lo + n] = db;
+                    a.dyb[(size_t)m * a.Ko + n] = db;
+                    cs[r & 1] += d;
+                }
+            }
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) {
+                cs[0] += __shfl_xor_sync(0xffffffffu, cs[0], o);
+                cs[1] += __shfl_xor_sync(0xffffffffu, cs[1], o);
+            }
+            if (g == 0) {
+                s_db[mt][nt * 8 + 2 * tq] = cs[0];
+                s_db[mt][nt * 8 + 2 * tq + 1] = cs[1];
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) s_loss[warp] = l;
+    }
+    __syncthreads();   // dy complete, h2 read
+    if (tid < a.d_out) colp[2 * width + tid] = s_db[0][tid] + s_db[1][tid];
+    if (tid == 0) {
+        double t = 0.0;
+        for (int w = 0; w < kTrThreads / 32; ++w) t += s_loss[w];
+        a.losspart[blockIdx.x] = t;
+    }
+    // dh2 = (dy W3^T)(1 - h2^2)
+    zero();
+    if (busy)
+        for (int kk = 0; kk < a.Ko; kk += 16) mma_step(sDY, lo, kk, sW3, lo, kk);
+    dtanh_layer(h2, sH2, a.dh2b, colp + width);
+    // dh1 = (dh2 W2^T)(1 - h1^2)
+    layer(sH2, lw, ncw);
+    dtanh_layer(h1, nullptr, a.dh1b, colp);
+    mlp_cp_wait<0>();
+}
+
+struct ApplyArgs {
+    float *par, *mom, *vel, *grad;          // grad: written instead of the update when not null
+    __nv_bfloat16 *wb[3], *wbT[3];
+    int ldb[3], ldt[3], rows[3], cols[3];
+    double *loss;
+    int nrow;                               // row blocks of k_train_rows
+    float lr, b1, b2, eps, bc1, bc2;
+};
+
+// The gradient of every parameter and its update.  Blocks 0 .. nbias-1: the
+// biases (a warp each: the row blocks' sums, lanes over the blocks) and, block
+// 0, the loss; the rest: a 32 x 32 square C[m][n] = sum over the batch of
+// A[row][m] B[row][n] of one of the three weight matrices.
+__global__ void __launch_bounds__(kDwThreads) k_train_update(TrainArgs a, ApplyArgs p, int nbias) {
+    __shared__ __align__(16) __nv_bfloat16 sA[kDwStages][kDwRows][kDwTile + SPAD], sB[kDwStages][kDwRows][kDwTile + SPAD];
+    __shared__ float s_g[kDwTile][kDwTile + 1];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
+    const int w = a.width, d_out = a.d_out;
+    auto update = [&](long long i, float gr) -> float {
+        if (p.grad) {
+            p.grad[i] = gr;
+            return 0.f;
+        }
+        return p.par[i] = adam_value(p.par[i], p.mom[i], p.vel[i], gr, p.lr, p.b1, p.b2, p.eps, p.bc1, p.bc2);
+    };
+    if ((int)blockIdx.x < nbias) {
+        const int nb = 2 * w + d_out, k = blockIdx.x * (kDwThreads / 32) + warp;
+        if (k < nb) {
+            float s = 0.f;
+#pragma unroll 4
+            for (int r = lane; r < p.nrow; r += 32) s += a.colpart[(size_t)r * nb + k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) {
+                const int l = k < w ? 0 : k < 2 * w ? 1 : 2;
+                long long i = (long long)p.rows[0] * w;
+                if (l > 0) i += w + (long long)w * w;
+                if (l > 1) i += w + (long long)w * d_out;
+                update(i + (k - l * w), s);
+            }
+        }
+        if (blockIdx.x == 0 && warp == 0) {
+            double t = 0.0;
+            for (int r = lane; r < p.nrow; r += 32) t += a.losspart[r];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) *p.loss = t / (double)(a.batch * d_out);
+        }
+        return;
+    }
+    int q = blockIdx.x - nbias, l = 0;
+    long long off = 0;
+    for (; l < 2; ++l) {
+        const int n = ((p.rows[l] + kDwTile - 1) / kDwTile) * ((p.cols[l] + kDwTile - 1) / kDwTile);
+        if (q < n) break;
+        q -= n;
+        off += (long long)p.rows[l] * p.cols[l] + p.cols[l];
+    }
+    const int M = p.rows[l], N = p.cols[l], nq = (N + kDwTile - 1) / kDwTile;
+    const int m0 = (q / nq) * kDwTile, n0 = (q % nq) * kDwTile;
+    const __nv_bfloat16 *A = l == 0 ? a.xb : l == 1 ? a.h1b : a.h2b, *B = l == 0 ? a.dh1b : l == 1 ? a.dh2b : a.dyb;
+    const int lda = l == 0 ? a.K1 : a.Kw, ldb = l == 2 ? a.Ko : a.Kw;   // multiples of 32: a tile's columns exist
+    const int nch = (a.batch + kDwRows - 1) / kDwRows;
+    // this thread's 16 bytes of rows tid / 4 and tid / 4 + 32 of every chunk
+    // (rows past the batch are zero and add nothing)
+    const int ir = tid >> 2, ic = (tid & 3) * 8;
+    const __nv_bfloat16 *pa = A + (size_t)ir * lda + m0 + ic, *pb = B + (size_t)ir * ldb + n0 + ic;
+    auto issue = [&](int ch) {
+        if (ch < nch) {
+            __nv_bfloat16 *da = &sA[ch % kDwStages][ir][ic], *db = &sB[ch % kDwStages][ir][ic];
+#pragma unroll
+            for (int u = 0; u < kDwRows; u += kDwThreads / 4) {
+                const bool ok = ch * kDwRows + ir + u < a.batch;
+                mlp_cp16(da + u * (kDwTile + SPAD), ok ? pa + u * lda : A, ok);
+                mlp_cp16(db + u * (kDwTile + SPAD), ok ? pb + u * ldb : B, ok);
+            }
+            pa += kDwRows * lda;
+            pb += kDwRows * ldb;
+        }
+        mlp_cp_commit();
+    };
+    float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};   // 16 x 16 per warp
+    const int wm = (warp >> 1) * 16, wn = (warp & 1) * 16;
+#pragma unroll
+    for (int c = 0; c < kDwStages - 1; ++c) issue(c);
+    for (int ch = 0; ch < nch; ++ch) {
+        mlp_cp_wait<kDwStages - 2>();
+        __syncthreads();
+        issue(ch + kDwStages - 1);
+        const int st = ch % kDwStages;
+        unsigned af[kDwRows / 16][4], bf[kDwRows / 16][4];
+#pragma unroll
+        for (int k = 0; k < kDwRows / 16; ++k) {
+            ldmatrix_x4_t(af[k][0], af[k][1], af[k][2], af[k][3],
+                          &sA[st][k * 16 + (lane & 7) + ((lane >> 4) & 1) * 8][wm + ((lane >> 3) & 1) * 8]);
+            ldmatrix_x4_t(bf[k][0], bf[k][1], bf[k][2], bf[k][3],
+                          &sB[st][k * 16 + (lane & 7) + ((lane >> 3) & 1) * 8][wn + ((lane >> 4) & 1) * 8]);
+        }
+#pragma unroll
+        for (int k = 0; k < kDwRows / 16; ++k)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) mma_bf16(acc[j], af[k][0], af[k][1], af[k][2], af[k][3], bf[k][2 * j], bf[k][2 * j + 1]);
+    }
+    mlp_cp_wait<0>();
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s_g[wm + g + (r >= 2 ? 8 : 0)][wn + j * 8 + 2 * tq + (r & 1)] = acc[j][r];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kDwTile / 4; ++u) {
+        const int mr = warp + 4 * u, m = m0 + mr, n = n0 + lane;
+        if (m < M && n < N) {
+            const float v = update(off + (long long)m * N + n, s_g[mr][lane]);
+            s_g[mr][lane] = v;
+            if (!p.grad) p.wb[l][(size_t)m * p.ldb[l] + n] = __float2bfloat16_rn(v);
+        }
+    }
+    if (p.grad) return;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kDwTile / 4; ++u) {   // the transposed copy
+        const int nr = warp + 4 * u, n = n0 + nr, m = m0 + lane;
+        if (m < M && n < N) p.wbT[l][(size_t)n * p.ldt[l] + m] = __float2bfloat16_rn(s_g[lane][nr]);
     }
 }
 
@@ -593,6 +1005,8 @@ struct qp_mlp {
     __nv_bfloat16 *xb, *xT, *h1b, *h1T, *h2b, *h2T, *dyb, *dyT, *dh2b, *dh2T, *dh1b, *dh1T;
     float *h1, *h2, *y;
     double *loss;
+    float *tr_col = nullptr;       // fused training step: the row blocks' sums
+    double *tr_loss = nullptr;
     int *tstep;                   // rollout step index and block counter (device)
     unsigned *tdone;
     // rollout graph: steps captured once, replayed (key: arguments it bakes in)
@@ -648,7 +1062,15 @@ size_t mlp_layout(qp_mlp *m, int d_in, int width, int d_out, int max_batch, char
     char *h1 = take((size_t)max_batch * width * 4), *h2 = take((size_t)max_batch * width * 4);
     char *y = take((size_t)max_batch * d_out * 4), *loss = take(8);
     char *tstep = take(16);
+    char *trc = nullptr, *trl = nullptr;
+    if (train_fused(d_in, width, d_out)) {
+        const size_t nrow = (max_batch + kTrRows - 1) / kTrRows;
+        trc = take(nrow * (2 * width + d_out) * 4);
+        trl = take(nrow * 8);
+    }
     if (m && base) {
+        m->tr_col = (float *)trc;
+        m->tr_loss = (double *)trl;
         m->par = (float *)par;
         m->grad = (float *)grad;
         m->mom = (float *)mom;
@@ -813,6 +1235,79 @@ cudaError_t backward(qp_mlp *m, const float *d_t, int batch) {
     return gemm<EPI_STORE>(m, m->xT, m->Bp, m->dh1T, m->Bp, m->d_in, m->width, Kb, st);
 }
 
+// The training step of a network that fits the fused kernels; grad_only: the
+// gradients into m->grad instead of the Adam update.
+cudaError_t train_fused_step(qp_mlp *m, const float *d_x, const float *d_t, int batch, bool grad_only, float lr,
+                             float b1, float b2, float eps, float bc1, float bc2) {
+    TrainArgs a;
+    a.x = d_x;
+    a.tgt = d_t;
+    a.batch = batch;
+    a.d_in = m->d_in;
+    a.width = m->width;
+    a.d_out = m->d_out;
+    a.K1 = m->K1;
+    a.Kw = m->Kw;
+    a.Ko = m->Ko;
+    a.w1t = m->WbT[0];
+    a.w2t = m->WbT[1];
+    a.w3t = m->WbT[2];
+    a.w2 = m->Wb[1];
+    a.w3 = m->Wb[2];
+    a.b1 = m->b[0];
+    a.b2 = m->b[1];
+    a.b3 = m->b[2];
+    a.xb = m->xb;
+    a.h1b = m->h1b;
+    a.h2b = m->h2b;
+    a.dyb = m->dyb;
+    a.dh2b = m->dh2b;
+    a.dh1b = m->dh1b;
+    a.colpart = m->tr_col;
+    a.losspart = m->tr_loss;
+    const size_t sm = train_rows_smem(m->K1, m->Kw, m->Ko);
+    cudaError_t e = cudaFuncSetAttribute(k_train_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)train_rows_smem(pad32(kTrMaxIn), kTrMaxW, kTrMaxOut));
+    if (e != cudaSuccess) return e;
+    const int nrow = (batch + kTrRows - 1) / kTrRows;
+    k_train_rows<<<nrow, kTrThreads, sm, m->stream>>>(a);
+    ApplyArgs p;
+    p.par = m->par;
+    p.mom = m->mom;
+    p.vel = m->vel;
+    p.grad = grad_only ? m->grad : nullptr;
+    int squares = 0;
+    for (int l = 0; l < 3; ++l) {
+        const ParamBlock b = weight_block(m, l, true);
+        p.wb[l] = b.wb;
+        p.wbT[l] = b.wbT;
+        p.ldb[l] = b.ldb;
+        p.ldt[l] = b.ldt;
+        p.rows[l] = b.rows;
+        p.cols[l] = b.cols;
+        squares += ((b.rows + kDwTile - 1) / kDwTile) * ((b.cols + kDwTile - 1) / kDwTile);
+    }
+    p.loss = m->loss;
+    p.nrow = nrow;
+    p.lr = lr;
+    p.b1 = b1;
+    p.b2 = b2;
+    p.eps = eps;
+    p.bc1 = bc1;
+    p.bc2 = bc2;
+    const int per = kDwThreads / 32, nbias = (2 * m->width + m->d_out + per - 1) / per;
+    k_train_update<<<nbias + squares, kDwThreads, 0, m->stream>>>(a, p, nbias);
+    return cudaGetLastError();
+}
+
+// Gradients of a network beyond the fused kernels: one launch per product.
+cudaError_t train_passes(qp_mlp *m, const float *d_x, const float *d_t, int batch) {
+    cudaError_t e = clear_transposed(m, batch);
+    if (e == cudaSuccess) e = forward(m, d_x, batch);
+    if (e == cudaSuccess) e = backward(m, d_t, batch);
+    return e;
+}
+
 qp_status mfail(qp_mlp *m, qp_status s, const std::string &msg) {
     if (m) m->err = msg;
     return s;
@@ -897,9 +1392,10 @@ qp_status qp_mlp_forward(qp_mlp *m, const float *d_x, int batch, float *d_y) {
 
 qp_status qp_mlp_gradients(qp_mlp *m, const float *d_x, const float *d_t, int batch, float *h_grads, double *loss) {
     if (!m || !d_x || !d_t || batch < 1 || batch > m->max_batch) return QP_ERR_ARG;
-    if (clear_transposed(m, batch) != cudaSuccess || forward(m, d_x, batch) != cudaSuccess ||
-        backward(m, d_t, batch) != cudaSuccess)
-        return mfail(m, QP_ERR_CUDA, "forward/backward");
+    const cudaError_t e = train_fused(m->d_in, m->width, m->d_out)
+                              ? train_fused_step(m, d_x, d_t, batch, true, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f)
+                              : train_passes(m, d_x, d_t, batch);
+    if (e != cudaSuccess) return mfail(m, QP_ERR_CUDA, "forward/backward");
     if (h_grads && cudaMemcpyAsync(h_grads, m->grad, m->npar * 4, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
         return mfail(m, QP_ERR_CUDA, "copy");
     if (loss && cudaMemcpyAsync(loss, m->loss, 8, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
@@ -913,16 +1409,20 @@ qp_status qp_mlp_train_step(qp_mlp *m, const float *d_x, const float *d_t, int b
     if (!m || !d_x || !d_t || batch < 1 || batch > m->max_batch) return QP_ERR_ARG;
     if (!(lr > 0.f) || !(beta1 >= 0.f && beta1 < 1.f) || !(beta2 >= 0.f && beta2 < 1.f) || !(eps > 0.f))
         return mfail(m, QP_ERR_ARG, "bad Adam hyper-parameters");
-    if (clear_transposed(m, batch) != cudaSuccess || forward(m, d_x, batch) != cudaSuccess ||
-        backward(m, d_t, batch) != cudaSuccess)
-        return mfail(m, QP_ERR_CUDA, "forward/backward");
+    const bool fused = train_fused(m->d_in, m->width, m->d_out);
+    if (!fused && train_passes(m, d_x, d_t, batch) != cudaSuccess) return mfail(m, QP_ERR_CUDA, "forward/backward");
     ++m->step;
     const float bc1 = 1.f - powf(beta1, (float)m->step), bc2 = 1.f - powf(beta2, (float)m->step);
-    for (int l = 0; l < 3; ++l) {
-        k_adam<<<128, 256, 0, m->stream>>>(weight_block(m, l, true), lr, beta1, beta2, eps, bc1, bc2);
-        k_adam<<<8, 256, 0, m->stream>>>(bias_block(m, l), lr, beta1, beta2, eps, bc1, bc2);
+    if (fused) {
+        if (train_fused_step(m, d_x, d_t, batch, false, lr, beta1, beta2, eps, bc1, bc2) != cudaSuccess)
+            return mfail(m, QP_ERR_CUDA, "training step");
+    } else {
+        for (int l = 0; l < 3; ++l) {
+            k_adam<<<128, 256, 0, m->stream>>>(weight_block(m, l, true), lr, beta1, beta2, eps, bc1, bc2);
+            k_adam<<<8, 256, 0, m->stream>>>(bias_block(m, l), lr, beta1, beta2, eps, bc1, bc2);
+        }
+        if (cudaGetLastError() != cudaSuccess) return mfail(m, QP_ERR_CUDA, "adam");
     }
-    if (cudaGetLastError() != cudaSuccess) return mfail(m, QP_ERR_CUDA, "adam");
     if (loss) {
         if (cudaMemcpyAsync(loss, m->loss, 8, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess ||
             cudaStreamSynchronize(m->stream) != cudaSuccess)
