@@ -15,15 +15,11 @@
 //               FP64 sums, largest weight (Sec. 3.1 "Pre-merging");
 //   k_w_tie     members within the tie window of the largest weight compete
 //               on a 64-bit tie key (the positions outside P', in key order);
-//   (k_w_tie<true>: the winner becomes the group's representative)
-//   k_w_expand  the M^2 children of each group (Eqs. SysP, inf_fun), one at
-//               a time: one lane per group, or sub_n lanes sharing a group,
-//               each forming every sub_n-th child; the history part H of the
-//               influence exponent from per-position tables; filtered
-//               (|amp| >= theta, Sec. 2.1) and appended in output ranges
-//               reserved once per block and round;
-//   k_w_rho     rho(t) from the appended children by newest point (Eq.
-//               quapi_red_rho), per-block sums;
+//               the representative's key is its group key and the winning
+//               tie key put together again;
+//   k_w_expand  the M^2 children of each group (Eqs. SysP, inf_fun), the
+//               filter (|amp| >= theta, Sec. 2.1), the output and rho(t) by
+//               newest point (Eq. quapi_red_rho);
 //   k_w_finalize the step's rho, counts and state.
 // While the window fills every stored path is its own group (reading R3).
 #include <cuda_runtime.h>
@@ -43,7 +39,8 @@ namespace {
 constexpr int kWMaxM = 8, kWMaxDk = 16, kWMaxMM = 64;
 constexpr int kWThreads = 256;
 constexpr int kWProbe = 64;
-constexpr int kWMaxTabDelta = 16;   // distinct coupling differences up to which a group tabulates its factors
+constexpr int kWMaxRuns = 16;       // runs of consecutive positions, each within one word of eight
+constexpr int kWMaxBlocks = 2048;   // blocks of the expansion (partials of rho)
 constexpr unsigned long long kWEmpty = ~0ull;
 constexpr unsigned kWErrPaths = 1u, kWErrGroups = 2u, kWErrProbe = 4u;
 
@@ -64,27 +61,35 @@ struct __align__(32) WSlot {
     double sre, sim;
 };
 
+// A set of window positions as runs of consecutive ones: run r takes the
+// bits mask[r] of word word[r] (compacted to 6 bits per position, eight
+// positions per word) from shift[r] to off[r] of the packed key.
+struct WRuns {
+    int n, npos;
+    unsigned char word[kWMaxRuns], shift[kWMaxRuns], off[kWMaxRuns];
+    unsigned long long mask[kWMaxRuns];
+};
+
 struct WParams {
     int M, dkmax, c64, rho_hist;
     long long max_paths, max_groups;
-    unsigned long long tcap_mask;
-    int npp, nco;                      // positions of P' and of its complement (ascending)
-    int pp[kWMaxDk], co[kWMaxDk];
+    unsigned long long tcap;           // slots of the merge table
+    WRuns pp, co;                      // positions of P' and of its complement
     double theta2, tie_rel;
     float theta2f;
     double q[kWMaxM];
-    int ndelta;                        // distinct nonzero q_a - q_b (tabulated per group when <= kWMaxTabDelta)
-    double delta[kWMaxMM];
-    signed char dsel[kWMaxMM];         // child c -> its difference (-1: q_a = q_b)
+    float dq2[kWMaxMM];                // -2 log2(e) (q_a - q_b) of child (a, b)
+    float log2_theta2;                 // log2 theta^2; -inf: no bound is taken (see k_w_expand)
     unsigned long long *klo[2], *khi[2];
     void *amps[2];
-    unsigned int *slot_of, *groups, *trep;
+    unsigned int *slot_of, *groups;
     WSlot *slots;
     unsigned long long *ttie;
     const double2 *lut;                // [dkmax][dkmax - 1][256] FP64 history tables
     const float2 *lutf, *lutlo;        // FP32 hi part and residual
     const double2 *w;                  // [M*M child][M*M parent newest]
     const float4 *wf;                  // FP32 hi/lo pairs of w
+    const float *lw;                   // [M*M parent][M*M child] log2 |w|^2
     double2 *rho_part;                 // [blocks][M*M]
     double2 *rho_ring;                 // [rho_hist][M*M]
     WRec *stats;                       // [rho_hist]
@@ -94,17 +99,34 @@ struct WParams {
 __device__ __forceinline__ unsigned key_byte(unsigned long long lo, unsigned long long hi, int j) {
     return (unsigned)((j < 8 ? lo >> (8 * j) : hi >> (8 * (j - 8))) & 0xffull);
 }
-// 6-bit code of a position (forward | backward << 3), positions in ascending
-// order at ascending bits: equal on P' <=> equal group keys; on the
-// complement the order of the full keys
-__device__ __forceinline__ unsigned long long pack6(unsigned long long lo, unsigned long long hi, const int *pos,
-                                                    int n) {
+// Eight positions of a key word (one byte each) as 6-bit codes (forward |
+// backward << 3), and back.
+__device__ __forceinline__ unsigned long long compact6(unsigned long long x) {
+    x = (x & 0x0707070707070707ull) | ((x >> 1) & 0x3838383838383838ull);
+    x = (x & 0x003f003f003f003full) | ((x & 0x3f003f003f003f00ull) >> 2);
+    x = (x & 0x00000fff00000fffull) | ((x & 0x0fff00000fff0000ull) >> 4);
+    return (x & 0xffffffull) | ((x >> 8) & 0xffffff000000ull);
+}
+__device__ __forceinline__ unsigned long long expand6(unsigned long long x) {
+    x = (x & 0xffffffull) | ((x & 0xffffff000000ull) << 8);
+    x = (x & 0x00000fff00000fffull) | ((x & 0x00fff00000fff000ull) << 4);
+    x = (x & 0x003f003f003f003full) | ((x & 0x0fc00fc00fc00fc0ull) << 2);
+    return (x & 0x0707070707070707ull) | ((x & 0x3838383838383838ull) << 1);
+}
+// The codes of a set of positions packed in ascending order: equal on P' <=>
+// equal group keys; on the complement the order of the full keys.
+__device__ __forceinline__ unsigned long long pack_runs(const WRuns &R, unsigned long long c0, unsigned long long c1) {
     unsigned long long k = 0;
-    for (int i = 0; i < n; ++i) {
-        const unsigned v = key_byte(lo, hi, pos[i]);
-        k |= (unsigned long long)((v & 7u) | (((v >> 4) & 7u) << 3)) << (6 * i);
-    }
+    for (int r = 0; r < R.n; ++r) k |= (((R.word[r] ? c1 : c0) >> R.shift[r]) & R.mask[r]) << R.off[r];
     return k;
+}
+__device__ __forceinline__ void unpack_runs(const WRuns &R, unsigned long long k, unsigned long long &c0,
+                                            unsigned long long &c1) {
+    for (int r = 0; r < R.n; ++r) {
+        const unsigned long long v = ((k >> R.off[r]) & R.mask[r]) << R.shift[r];
+        if (R.word[r]) c1 |= v;
+        else c0 |= v;
+    }
 }
 __device__ __forceinline__ unsigned long long wmix(unsigned long long x) {
     x ^= x >> 31;
@@ -113,6 +135,12 @@ __device__ __forceinline__ unsigned long long wmix(unsigned long long x) {
     x *= 0x81dadef4bc2dd44dull;
     x ^= x >> 33;
     return x;
+}
+// s + e += b with the rounding error of the addition carried into e (TwoSum)
+__device__ __forceinline__ void two_sum_w(float &s, float &e, float b) {
+    const float t = s + b, v = t - s;
+    e += (s - (t - v)) + (b - v);
+    s = t;
 }
 __device__ __forceinline__ double weight_of(const WParams &P, const void *amps, unsigned long long i) {
     if (P.c64) {
@@ -130,48 +158,78 @@ __device__ __forceinline__ double2 amp_of(const WParams &P, const void *amps, un
     return static_cast<const double2 *>(amps)[i];
 }
 
+// The part of the table that a step of n paths uses: two slots per path at
+// most (at least a page), so that a small step stays near the L2.
+__device__ __forceinline__ unsigned long long table_slots(const WParams &P, unsigned long long n) {
+    return min(P.tcap, max(2ull * n, 1024ull));
+}
+
 // pre-merge, pass 1: claim or find the group's slot, add the amplitude,
-// raise the largest weight
-__global__ void k_w_insert(WParams P) {
+// raise the largest weight; the new groups of a block's round are listed with
+// one atomic.  Bound: the latency of a random 32-byte slot per path.
+__global__ void __launch_bounds__(kWThreads) k_w_insert(WParams P) {
+    __shared__ unsigned s_wc[kWThreads / 32];
+    __shared__ unsigned long long s_base;
     WState *st = P.st;
     if (st->err) return;
     const int in = (int)(st->t & 1);
-    const unsigned long long n = st->n_cur;
-    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n;
-         i += (unsigned long long)gridDim.x * blockDim.x) {
-        const unsigned long long lo = P.klo[in][i], hi = P.khi[in][i];
-        const unsigned long long gk = pack6(lo, hi, P.pp, P.npp);
-        unsigned long long h = wmix(gk) & P.tcap_mask;
-        int probe = 0;
-        for (; probe < kWProbe; ++probe, h = (h + 1) & P.tcap_mask) {
-            unsigned long long cur = P.slots[h].gk;
-            if (cur == kWEmpty) {
-                cur = atomicCAS(&P.slots[h].gk, kWEmpty, gk);
-                if (cur == kWEmpty) {   // claimed: a new group
-                    const unsigned long long g = atomicAdd(&st->n_groups, 1ull);
-                    if ((long long)g < P.max_groups) P.groups[g] = (unsigned)h;
-                    else atomicOr(&st->err, kWErrGroups);
-                    break;
+    const unsigned long long n = st->n_cur, slots = table_slots(P, n);
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    for (unsigned long long base = blockIdx.x * (unsigned long long)kWThreads; base < n;
+         base += (unsigned long long)gridDim.x * kWThreads) {
+        const unsigned long long i = base + threadIdx.x;
+        bool claimed = false;
+        unsigned long long h = 0;
+        if (i < n) {
+            const unsigned long long lo = P.klo[in][i], hi = P.khi[in][i];
+            const unsigned long long gk = pack_runs(P.pp, compact6(lo), compact6(hi));
+            const double2 a = amp_of(P, P.amps[in], i);
+            h = __umul64hi(wmix(gk), slots);
+            int probe = 0;
+            for (; probe < kWProbe; ++probe, h = h + 1 == slots ? 0 : h + 1) {
+                unsigned long long cur = *(volatile unsigned long long *)&P.slots[h].gk;
+                if (cur == kWEmpty) {
+                    cur = atomicCAS(&P.slots[h].gk, kWEmpty, gk);
+                    if (cur == kWEmpty) {   // a new group
+                        claimed = true;
+                        break;
+                    }
                 }
+                if (cur == gk) break;
             }
-            if (cur == gk) break;
+            if (probe == kWProbe) {
+                atomicOr(&st->err, kWErrProbe);
+            } else {
+                atomicAdd(&P.slots[h].sre, a.x);
+                atomicAdd(&P.slots[h].sim, a.y);
+                atomicMax(&P.slots[h].wm, (unsigned long long)__double_as_longlong(weight_of(P, P.amps[in], i)));
+                P.slot_of[i] = (unsigned)h;
+            }
         }
-        if (probe == kWProbe) {
-            atomicOr(&st->err, kWErrProbe);
-            return;
+        const unsigned cm = __ballot_sync(0xffffffffu, claimed);
+        if (lane == 0) s_wc[warp] = __popc(cm);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned tot = 0;
+            for (int w = 0; w < kWThreads / 32; ++w) {
+                const unsigned v = s_wc[w];
+                s_wc[w] = tot;
+                tot += v;
+            }
+            s_base = tot ? atomicAdd(&st->n_groups, (unsigned long long)tot) : 0ull;
         }
-        const double2 a = amp_of(P, P.amps[in], i);
-        atomicAdd(&P.slots[h].sre, a.x);
-        atomicAdd(&P.slots[h].sim, a.y);
-        atomicMax(&P.slots[h].wm, (unsigned long long)__double_as_longlong(weight_of(P, P.amps[in], i)));
-        P.slot_of[i] = (unsigned)h;
+        __syncthreads();
+        if (claimed) {
+            const unsigned long long g = s_base + s_wc[warp] + __popc(cm & ((1u << lane) - 1u));
+            if ((long long)g < P.max_groups) P.groups[g] = (unsigned)h;
+            else atomicOr(&st->err, kWErrGroups);
+        }
+        __syncthreads();   // s_wc and s_base are rewritten in the next round
     }
 }
 
 // pre-merge, pass 2: members within the tie window compete on the tie key
-// (pass 3: the winner, unique in its group, becomes the representative)
-template <bool REP>
-__global__ void k_w_tie(WParams P) {
+__global__ void __launch_bounds__(kWThreads) k_w_tie(WParams P) {
     WState *st = P.st;
     if (st->err) return;
     const int in = (int)(st->t & 1);
@@ -181,258 +239,379 @@ __global__ void k_w_tie(WParams P) {
         const unsigned h = P.slot_of[i];
         const double wm = __longlong_as_double((long long)P.slots[h].wm);
         if (weight_of(P, P.amps[in], i) < (1.0 - P.tie_rel) * wm) continue;
-        const unsigned long long tk = pack6(P.klo[in][i], P.khi[in][i], P.co, P.nco);
-        if (!REP) atomicMin(&P.ttie[h], tk);
-        else if (tk == P.ttie[h]) P.trep[h] = (unsigned)i;
+        atomicMin(&P.ttie[h], pack_runs(P.co, compact6(P.klo[in][i]), compact6(P.khi[in][i])));
     }
 }
 
-// children of one group, appended in warp-aggregated blocks; thread-uniform
-// loops (every lane of a warp runs every child, valid or not)
-template <bool C64, bool TAB>
-__global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge, int sub_n) {
-    // sub_n consecutive lanes share a group (a power of two dividing 32), lane
-    // s taking its children c = s, s + sub_n, ...; each lane forms the
-    // group's history sum itself.  TAB: the influence factors exp(-delta H)
-    // of the group's distinct coupling differences, computed once per lane
-    // (the same arithmetic as per child), in shared memory [delta][thread]
+// log2 of a non-negative double to FP32 accuracy, off the FP64 pipe (zero and
+// subnormals: -inf; infinities and NaNs: +inf, which no bound drops)
+__device__ __forceinline__ float log2_d(double d) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+    const int e = (int)((u >> 52) & 0x7ffull);
+    if (e == 0) return -INFINITY;
+    if (e == 0x7ff) return INFINITY;
+    return (float)(e - 1023) + log2f(__uint_as_float(0x3f800000u | (unsigned)((u >> 29) & 0x7fffffull)));
+}
+
+inline size_t expand_smem(int MM, int nb, bool c64) {
+    const size_t ct = c64 ? 8 : 16, lw = (size_t)MM * ((MM + 7) & ~3) * 4;
+    return (size_t)nb * 64 * 16 + (size_t)(kWThreads / 32) * MM * 16 + 2 * kWThreads * ct + 2 * kWThreads * 8 +
+           ((lw + 15) & ~(size_t)15) + (size_t)MM * (kWThreads / 32) * 8 + kWThreads + (size_t)kWThreads * MM * 2;
+}
+
+// The children of the step's groups (merge) or stored paths (window filling).
+// A block takes 256 groups per round.  With most of the M^2 children below
+// the filter (the reaction-coordinate model keeps about 2 of 64) each thread
+// first bounds the 64 weights of its group,
+//   log2 |child|^2 = log2 |S|^2 + log2 |W|^2 - 2 log2(e) (q_a - q_b) Re H,
+// one table entry, one multiply-add and one comparison per child in FP32,
+// with a margin of 2^0.002 (the terms are good to about 2^-16); the children
+// above the bound are listed child-major for the block, so that they are
+// dealt evenly to the threads and a warp's children share their newest
+// point; each is formed once in full precision, filtered, added to rho(t)
+// (segments of equal newest point, then one lane's addition to its warp's
+// bin; C64: FP32 pairs, TwoSum) and written to a range reserved per 256
+// candidates.  (Forming all 64 children twice, four lanes per group, with
+// rho from a second pass over the children took 0.88 ms per step and launch
+// at 2e6 groups, the two passes of rho and of its block sums 0.30 ms.)
+template <bool C64>
+__global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
     using CT = typename std::conditional<C64, float2, double2>::type;
-    extern __shared__ __align__(16) unsigned char s_wtab[];
-    CT *sE = reinterpret_cast<CT *>(s_wtab);
-    __shared__ unsigned s_wc[kWThreads / 32];
+    constexpr int NW = kWThreads / 32;
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ unsigned s_wc[NW], s_tot;
     __shared__ unsigned long long s_base;
     WState *st = P.st;
+    const int M = P.M, MM = M * M;
+    const int nb = P.dkmax - 1;                       // history bytes of a key
+    const int lws = (MM + 7) & ~3;                    // row of the bound table (rows on different banks)
+    float4 *s_lut = reinterpret_cast<float4 *>(s_dyn);   // [nb][64] history terms (C64: hi, lo; FP64: double2)
+    float4 *s_rho = s_lut + nb * 64;                     // [NW][MM] (C64: re, err, im, err; FP64: double2)
+    CT *s_S = reinterpret_cast<CT *>(s_rho + NW * MM), *s_H = s_S + kWThreads;
+    unsigned long long *s_lo = reinterpret_cast<unsigned long long *>(s_H + kWThreads), *s_hi = s_lo + kWThreads;
+    float *s_lw = reinterpret_cast<float *>(s_hi + kWThreads);
+    unsigned *s_mask = reinterpret_cast<unsigned *>(s_lw + ((MM * lws + 3) & ~3));   // [MM][NW] candidates of a warp
+    unsigned *s_off = s_mask + MM * NW;                                              // [MM][NW] their offsets
+    unsigned char *s_par = reinterpret_cast<unsigned char *>(s_off + MM * NW);
+    unsigned short *s_list = reinterpret_cast<unsigned short *>(s_par + kWThreads);
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    double2 *part = P.rho_part + (size_t)blockIdx.x * MM;
     if (st->err) return;
     const unsigned long long t = st->t, tn = t + 1;
     const int in = (int)(t & 1), outp = (int)(tn & 1);
     const unsigned long long ng = merge ? st->n_groups : st->n_cur;
-    const int M = P.M, MM = M * M;
     const int n_act = (int)min(tn, (unsigned long long)P.dkmax);
     const int L_child = (int)min(tn + 1, (unsigned long long)P.dkmax);
-    const int nb = P.dkmax - 1;                       // history bytes of a key
-    const unsigned lane = threadIdx.x & 31u;
     const size_t row = (size_t)(n_act - 1) * nb * 256;
-    const int sub = (int)(threadIdx.x & (unsigned)(sub_n - 1));
-    for (unsigned long long base = blockIdx.x * (unsigned long long)blockDim.x; base < ng * sub_n;
-         base += (unsigned long long)gridDim.x * blockDim.x) {
-        const unsigned long long g = (base + threadIdx.x) / (unsigned)sub_n;
+    for (int i = threadIdx.x; i < nb * 64; i += kWThreads) {
+        const size_t j = row + (size_t)(i >> 6) * 256 + ((i & 7) | ((i & 56) << 1));
+        if constexpr (C64) {
+            const float2 a = P.lutf[j], b = P.lutlo[j];
+            s_lut[i] = make_float4(a.x, a.y, b.x, b.y);
+        } else {
+            reinterpret_cast<double2 *>(s_lut)[i] = P.lut[j];
+        }
+    }
+    for (int i = threadIdx.x; i < MM * lws; i += kWThreads)
+        s_lw[i] = i % lws < MM ? P.lw[(size_t)(i / lws) * MM + i % lws] : -INFINITY;
+    for (int i = threadIdx.x; i < NW * MM; i += kWThreads) s_rho[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    for (unsigned long long base = blockIdx.x * (unsigned long long)kWThreads; base < ng;
+         base += (unsigned long long)gridDim.x * kWThreads) {
+        const unsigned long long g = base + threadIdx.x;
         const bool valid = g < ng;
-        unsigned long long lo = 0, hi = 0;
-        double2 S = make_double2(0.0, 0.0);
-        unsigned h = 0;
+        float thr = INFINITY, hre = 0.f;   // a child is a candidate unless its bound is below thr
+        int parc = 0;
         if (valid) {
-            unsigned long long r = g;
+            unsigned long long lo, hi;
+            double2 S;
             if (merge) {
-                h = P.groups[g];
-                r = P.trep[h];
-                S = make_double2(P.slots[h].sre, P.slots[h].sim);
+                const unsigned h = P.groups[g];
+                const WSlot sl = P.slots[h];
+                S = make_double2(sl.sre, sl.sim);
+                unsigned long long c0 = 0, c1 = 0;
+                unpack_runs(P.pp, sl.gk, c0, c1);
+                unpack_runs(P.co, P.ttie[h], c0, c1);
+                lo = expand6(c0);
+                hi = expand6(c1);
+                WSlot fresh;   // the slot is this group's: free for the next step
+                fresh.gk = kWEmpty;
+                fresh.wm = 0ull;
+                fresh.sre = fresh.sim = 0.0;
+                P.slots[h] = fresh;
+                P.ttie[h] = kWEmpty;
             } else {
-                S = amp_of(P, P.amps[in], r);
+                S = amp_of(P, P.amps[in], g);
+                lo = P.klo[in][g];
+                hi = P.khi[in][g];
             }
-            lo = P.klo[in][r];
-            hi = P.khi[in][r];
-        }
-        __syncwarp();   // every lane of the group has read the slot
-        if (valid && merge && sub == 0) {   // read by this group only: reset it for the next step
-            WSlot fresh;
-            fresh.gk = kWEmpty;
-            fresh.wm = 0ull;
-            fresh.sre = fresh.sim = 0.0;
-            P.slots[h] = fresh;
-            P.ttie[h] = kWEmpty;
-        }
-        const int par = (int)(lo & 0xffull);
-        const int parc = (par & 15) * M + (par >> 4);   // (forward, backward) of the newest point
-        // history part H of the influence exponent: FP64, or FP32 with the
-        // rounding of every addition kept (Kahan) from the hi/lo tables
-        double Hx = 0.0, Hy = 0.0;
-        float hx = 0.f, hy = 0.f, cx = 0.f, cy = 0.f;
-        for (int j = 0; j < nb; ++j) {
-            const unsigned v = key_byte(lo, hi, j);
+            const int par = (int)(lo & 0xffull);
+            parc = (par & 15) * M + (par >> 4);   // (forward, backward) of the newest point
+            // history part H of the influence exponent: FP64, or FP32 with the
+            // rounding of every addition kept (Kahan) from the hi/lo tables
             if constexpr (C64) {
-                const float2 a = P.lutf[row + (size_t)j * 256 + v], b = P.lutlo[row + (size_t)j * 256 + v];
-                float yx = (a.x - cx), tx = hx + yx;
-                cx = (tx - hx) - yx;
-                hx = tx;
-                yx = (b.x - cx);
-                tx = hx + yx;
-                cx = (tx - hx) - yx;
-                hx = tx;
-                float yy = (a.y - cy), ty = hy + yy;
-                cy = (ty - hy) - yy;
-                hy = ty;
-                yy = (b.y - cy);
-                ty = hy + yy;
-                cy = (ty - hy) - yy;
-                hy = ty;
+                float hx = 0.f, hy = 0.f, cx = 0.f, cy = 0.f;
+                for (int j = 0; j < nb; ++j) {
+                    const unsigned v = key_byte(lo, hi, j);
+                    const float4 e = s_lut[j * 64 + ((v & 7u) | ((v >> 1) & 56u))];
+                    float yx = (e.x - cx), tx = hx + yx;
+                    cx = (tx - hx) - yx;
+                    hx = tx;
+                    yx = (e.z - cx);
+                    tx = hx + yx;
+                    cx = (tx - hx) - yx;
+                    hx = tx;
+                    float yy = (e.y - cy), ty = hy + yy;
+                    cy = (ty - hy) - yy;
+                    hy = ty;
+                    yy = (e.w - cy);
+                    ty = hy + yy;
+                    cy = (ty - hy) - yy;
+                    hy = ty;
+                }
+                s_H[threadIdx.x] = make_float2(hx, hy);
+                s_S[threadIdx.x] = make_float2((float)S.x, (float)S.y);
+                hre = hx;
             } else {
-                const double2 e = P.lut[row + (size_t)j * 256 + v];
-                Hx += e.x;
-                Hy += e.y;
-            }
-        }
-        if constexpr (TAB) {
-            for (int d = 0; d < P.ndelta; ++d) {
-                if constexpr (C64) {
-                    const float dqf = (float)P.delta[d];
-                    const float zr = -dqf * hx, zi = -dqf * hy;
-                    float sn, cs;
-                    sincosf(zi, &sn, &cs);
-                    const float m = expf(zr);
-                    sE[d * kWThreads + threadIdx.x] = make_float2(m * cs, m * sn);
-                } else {
-                    const double zr = -P.delta[d] * Hx, zi = -P.delta[d] * Hy;
-                    double sn, cs;
-                    sincos(zi, &sn, &cs);
-                    const double m = exp(zr);
-                    sE[d * kWThreads + threadIdx.x] = make_double2(m * cs, m * sn);
+                double Hx = 0.0, Hy = 0.0;
+                for (int j = 0; j < nb; ++j) {
+                    const unsigned v = key_byte(lo, hi, j);
+                    const double2 e = reinterpret_cast<const double2 *>(s_lut)[j * 64 + ((v & 7u) | ((v >> 1) & 56u))];
+                    Hx += e.x;
+                    Hy += e.y;
                 }
+                s_H[threadIdx.x] = make_double2(Hx, Hy);
+                s_S[threadIdx.x] = S;
+                hre = (float)Hx;
             }
+            thr = P.log2_theta2 == -INFINITY ? -INFINITY : P.log2_theta2 - 0.002f - log2_d(S.x * S.x + S.y * S.y);
+            // child key: the parent shifted up one position, the new point in
+            // the lowest byte, cut to L_child positions
+            unsigned long long chi = (hi << 8) | (lo >> 56), clo = lo << 8;
+            if (8 * L_child <= 64) {
+                chi = 0;
+                if (8 * L_child < 64) clo &= (1ull << (8 * L_child)) - 1ull;
+            } else if (8 * L_child < 128) {
+                chi &= (1ull << (8 * L_child - 64)) - 1ull;
+            }
+            s_lo[threadIdx.x] = clo;
+            s_hi[threadIdx.x] = chi;
+            s_par[threadIdx.x] = (unsigned char)parc;
         }
-        // child key: the parent shifted up one position, the new point in
-        // the lowest byte, cut to L_child positions
-        unsigned long long chi = (hi << 8) | (lo >> 56), clo = lo << 8;
-        if (8 * L_child <= 64) {
-            chi = 0;
-            if (8 * L_child < 64) clo &= (1ull << (8 * L_child)) - 1ull;
-        } else if (8 * L_child < 128) {
-            chi &= (1ull << (8 * L_child - 64)) - 1ull;
-        }
-        // child c of the group: its amplitude and whether it survives the filter
-        auto child_of = [&](int c, double2 &child) -> bool {
-            const int a = c / M, b = c % M;
-            const double dq = P.q[a] - P.q[b];
-            if constexpr (C64) {
-                float fx, fy;
-                if constexpr (TAB) {
-                    const int d = P.dsel[c];
-                    const float2 e = d < 0 ? make_float2(1.f, 0.f) : sE[d * kWThreads + threadIdx.x];
-                    fx = e.x;
-                    fy = e.y;
-                } else {
-                    const float dqf = (float)dq;
-                    const float zr = -dqf * hx, zi = -dqf * hy;
-                    float sn, cs;
-                    sincosf(zi, &sn, &cs);
-                    const float m = expf(zr);
-                    fx = m * cs;
-                    fy = m * sn;
-                }
-                const float4 wv = P.wf[(size_t)c * MM + parc];
-                const float Sx = (float)S.x, Sy = (float)S.y;
-                // S (W_hi + W_lo) f
-                const float px = fmaf(Sx, wv.x, -Sy * wv.y) + fmaf(Sx, wv.z, -Sy * wv.w);
-                const float py = fmaf(Sx, wv.y, Sy * wv.x) + fmaf(Sx, wv.w, Sy * wv.z);
-                const float ox = px * fx - py * fy, oy = px * fy + py * fx;
-                child = make_double2(ox, oy);
-                return ox * ox + oy * oy >= P.theta2f;
-            } else {
-                double fx, fy;
-                if constexpr (TAB) {
-                    const int d = P.dsel[c];
-                    const double2 e = d < 0 ? make_double2(1.0, 0.0) : sE[d * kWThreads + threadIdx.x];
-                    fx = e.x;
-                    fy = e.y;
-                } else {
-                    const double zr = -dq * Hx, zi = -dq * Hy;
-                    double sn, cs;
-                    sincos(zi, &sn, &cs);
-                    const double m = exp(zr);
-                    fx = m * cs;
-                    fy = m * sn;
-                }
-                const double2 wv = P.w[(size_t)c * MM + parc];
-                const double px = S.x * wv.x - S.y * wv.y, py = S.x * wv.y + S.y * wv.x;
-                child = make_double2(px * fx - py * fy, px * fy + py * fx);
-                return child.x * child.x + child.y * child.y >= P.theta2;
-            }
-        };
-        // pass 1: the survivors of each group, counted; one output range per
-        // block and round (a block scan and one atomic), then pass 2 forms
-        // the survivors again (the same arithmetic) and writes them
-        unsigned long long kmask = 0ull;
-        if (valid)
-            for (int c = sub; c < MM; c += sub_n) {
-                double2 child;
-                if (child_of(c, child)) kmask |= 1ull << c;
-            }
-        const unsigned cnt = (unsigned)__popcll(kmask);
-        unsigned inc = cnt;
+        // the candidates of each child as warp masks
+        unsigned long long mine = 0ull;
+        for (int c0 = 0; c0 < MM; c0 += 4) {
+            const float4 l4 = *reinterpret_cast<const float4 *>(s_lw + parc * lws + c0);
+            const float lv[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
-            if ((int)lane >= o) inc += y;
-        }
-        if (lane == 31) s_wc[threadIdx.x >> 5] = inc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long tot = 0;
-            for (int w = 0; w < kWThreads / 32; ++w) {
-                const unsigned v = s_wc[w];
-                s_wc[w] = (unsigned)tot;
-                tot += v;
+            for (int u = 0; u < 4; ++u) {
+                const int c = c0 + u;
+                if (c >= MM) break;
+                const bool cand = valid && !(fmaf(P.dq2[c], hre, lv[u]) < thr);
+                const unsigned m = __ballot_sync(0xffffffffu, cand);
+                if (cand) mine |= 1ull << c;
+                if (lane == 0) s_mask[c * NW + warp] = m;
             }
-            s_base = tot ? atomicAdd(&st->n_out, tot) : 0ull;
         }
         __syncthreads();
-        unsigned long long o = s_base + s_wc[threadIdx.x >> 5] + (inc - cnt);
-        __syncthreads();   // s_wc and s_base are rewritten in the next round
-        if (cnt && (long long)(o + cnt) > P.max_paths) {
-            atomicOr(&st->err, kWErrPaths);
-            kmask = 0ull;
+        {   // exclusive scan of the MM * NW counts, two per thread
+            const int i0 = 2 * (int)threadIdx.x;
+            const unsigned n0 = i0 < MM * NW ? __popc(s_mask[i0]) : 0u, n1 = i0 + 1 < MM * NW ? __popc(s_mask[i0 + 1]) : 0u;
+            unsigned inc = n0 + n1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+                if ((int)lane >= o) inc += y;
+            }
+            if (lane == 31) s_wc[warp] = inc;
+            __syncthreads();
+            unsigned before = 0;
+            for (int w = 0; w < NW; ++w)
+                if (w < (int)warp) before += s_wc[w];
+            const unsigned ex = before + inc - n0 - n1;
+            if (i0 < MM * NW) s_off[i0] = ex;
+            if (i0 + 1 < MM * NW) s_off[i0 + 1] = ex + n0;
+            if (threadIdx.x == kWThreads - 1) s_tot = ex + n0 + n1;
         }
-        for (unsigned long long m = kmask; m; m &= m - 1ull, ++o) {
-            const int c = __ffsll((long long)m) - 1;
-            double2 child;
-            child_of(c, child);
-            P.klo[outp][o] = clo | (unsigned long long)((c / M) | ((c % M) << 4));
-            P.khi[outp][o] = chi;
-            if constexpr (C64) static_cast<float2 *>(P.amps[outp])[o] = make_float2((float)child.x, (float)child.y);
-            else static_cast<double2 *>(P.amps[outp])[o] = child;
+        __syncthreads();
+        for (unsigned long long m = mine; m; m &= m - 1ull) {
+            const int c = __ffsll((long long)m) - 1, q = c * NW + (int)warp;
+            s_list[s_off[q] + __popc(s_mask[q] & ((1u << lane) - 1u))] = (unsigned short)(threadIdx.x | (c << 8));
+        }
+        __syncthreads();
+        const unsigned total = s_tot;
+        for (unsigned p0 = 0; p0 < total; p0 += kWThreads) {
+            const unsigned p = p0 + threadIdx.x;
+            const bool have = p < total;
+            const unsigned e = have ? s_list[p] : 0u;
+            const int c = have ? (int)(e >> 8) : 0xff, src = (int)(e & 0xffu);
+            bool kept = false;
+            CT child;
+            child.x = child.y = 0;
+            int code = 0;
+            if (have) {
+                const int a = c / M, b = c - a * M;
+                code = a | (b << 4);
+                const double dq = P.q[a] - P.q[b];
+                const CT H = s_H[src], S = s_S[src];
+                if constexpr (C64) {
+                    float fx = 1.f, fy = 0.f;
+                    if (dq != 0.0) {
+                        const float dqf = (float)dq;
+                        const float zr = -dqf * H.x, zi = -dqf * H.y;
+                        float sn, cs;
+                        sincosf(zi, &sn, &cs);
+                        const float m = expf(zr);
+                        fx = m * cs;
+                        fy = m * sn;
+                    }
+                    const float4 wv = P.wf[(size_t)c * MM + s_par[src]];
+                    // S (W_hi + W_lo) f
+                    const float px = fmaf(S.x, wv.x, -S.y * wv.y) + fmaf(S.x, wv.z, -S.y * wv.w);
+                    const float py = fmaf(S.x, wv.y, S.y * wv.x) + fmaf(S.x, wv.w, S.y * wv.z);
+                    child = make_float2(px * fx - py * fy, px * fy + py * fx);
+                    kept = child.x * child.x + child.y * child.y >= P.theta2f;
+                } else {
+                    double fx = 1.0, fy = 0.0;
+                    if (dq != 0.0) {
+                        const double zr = -dq * H.x, zi = -dq * H.y;
+                        double sn, cs;
+                        sincos(zi, &sn, &cs);
+                        const double m = exp(zr);
+                        fx = m * cs;
+                        fy = m * sn;
+                    }
+                    const double2 wv = P.w[(size_t)c * MM + s_par[src]];
+                    const double px = S.x * wv.x - S.y * wv.y, py = S.x * wv.y + S.y * wv.x;
+                    child = make_double2(px * fx - py * fy, px * fy + py * fx);
+                    kept = child.x * child.x + child.y * child.y >= P.theta2;
+                }
+            }
+            // rho(t+1): the kept children of a segment of equal c, added by
+            // its last lane to the warp's bin
+            {
+                CT s = child, er;
+                er.x = er.y = 0;
+                if (!kept) s.x = s.y = 0;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int cu = __shfl_up_sync(0xffffffffu, c, o);
+                    const bool add = (int)lane >= o && cu == c;
+                    if constexpr (C64) {
+                        const float bx = __shfl_up_sync(0xffffffffu, s.x, o), by = __shfl_up_sync(0xffffffffu, s.y, o);
+                        const float ex = __shfl_up_sync(0xffffffffu, er.x, o), ey = __shfl_up_sync(0xffffffffu, er.y, o);
+                        if (add) {
+                            two_sum_w(s.x, er.x, bx);
+                            two_sum_w(s.y, er.y, by);
+                            er.x += ex;
+                            er.y += ey;
+                        }
+                    } else {
+                        const double bx = __shfl_up_sync(0xffffffffu, s.x, o), by = __shfl_up_sync(0xffffffffu, s.y, o);
+                        if (add) {
+                            s.x += bx;
+                            s.y += by;
+                        }
+                    }
+                }
+                const int cn = __shfl_down_sync(0xffffffffu, c, 1);
+                if (have && (lane == 31u || cn != c)) {
+                    float4 &bin = s_rho[warp * MM + c];
+                    if constexpr (C64) {
+                        float4 v = bin;
+                        two_sum_w(v.x, v.y, s.x);
+                        two_sum_w(v.z, v.w, s.y);
+                        v.y += er.x;
+                        v.w += er.y;
+                        bin = v;
+                    } else {
+                        double2 v = reinterpret_cast<double2 &>(bin);
+                        v.x += s.x;
+                        v.y += s.y;
+                        reinterpret_cast<double2 &>(bin) = v;
+                    }
+                }
+            }
+            const unsigned km = __ballot_sync(0xffffffffu, kept);
+            if (lane == 0) s_wc[warp] = __popc(km);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                unsigned tot = 0;
+                for (int w = 0; w < NW; ++w) {
+                    const unsigned v = s_wc[w];
+                    s_wc[w] = tot;
+                    tot += v;
+                }
+                s_base = tot ? atomicAdd(&st->n_out, (unsigned long long)tot) : 0ull;
+            }
+            __syncthreads();
+            if (kept) {
+                const unsigned long long o = s_base + s_wc[warp] + __popc(km & ((1u << lane) - 1u));
+                if ((long long)o >= P.max_paths) {
+                    atomicOr(&st->err, kWErrPaths);
+                } else {
+                    P.klo[outp][o] = s_lo[src] | (unsigned long long)code;
+                    P.khi[outp][o] = s_hi[src];
+                    static_cast<CT *>(P.amps[outp])[o] = child;
+                }
+            }
+            __syncthreads();   // s_wc and s_base are rewritten
+        }
+        // (the loop's last barrier, or none of its shared arrays read: the
+        // next round may overwrite them)
+        __syncthreads();
+    }
+    // this block's sums of rho, the warps in order
+    for (int k = threadIdx.x; k < MM; k += kWThreads) {
+        if constexpr (C64) {
+            float4 v = s_rho[k];
+            for (int w = 1; w < NW; ++w) {
+                const float4 b = s_rho[w * MM + k];
+                two_sum_w(v.x, v.y, b.x);
+                two_sum_w(v.z, v.w, b.z);
+                v.y += b.y;
+                v.w += b.w;
+            }
+            part[k] = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+        } else {
+            double2 v = reinterpret_cast<const double2 *>(s_rho)[k];
+            for (int w = 1; w < NW; ++w) {
+                const double2 b = reinterpret_cast<const double2 *>(s_rho)[w * MM + k];
+                v.x += b.x;
+                v.y += b.y;
+            }
+            part[k] = v;
         }
     }
 }
 
-// rho(t+1) by newest point from the appended children: per-block FP64 sums
-__global__ void __launch_bounds__(kWThreads) k_w_rho(WParams P) {
-    __shared__ double2 s_r[kWMaxMM];
-    WState *st = P.st;
-    const int MM = P.M * P.M;
-    for (int k = threadIdx.x; k < MM; k += blockDim.x) s_r[k] = make_double2(0.0, 0.0);
-    __syncthreads();
-    if (!st->err) {
-        const int outp = (int)((st->t + 1) & 1);
-        const unsigned long long n = min(st->n_out, (unsigned long long)P.max_paths);
-        for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n;
-             i += (unsigned long long)gridDim.x * blockDim.x) {
-            const unsigned v = (unsigned)(P.klo[outp][i] & 0xffull);
-            const double2 a = amp_of(P, P.amps[outp], i);
-            const int k = (int)(v & 15u) * P.M + (int)(v >> 4);
-            atomicAdd(&s_r[k].x, a.x);
-            atomicAdd(&s_r[k].y, a.y);
-        }
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < MM; k += blockDim.x) P.rho_part[(size_t)blockIdx.x * MM + k] = s_r[k];
-}
-
-// one block: rho(t+1) from the block sums, the step's record, the new state
-__global__ void k_w_finalize(WParams P, int nblk, int merge) {
+// one block of 1024 threads: rho(t+1) from the block sums (1024 / M^2 threads
+// per component, then in order), the step's record, the new state
+__global__ void __launch_bounds__(1024) k_w_finalize(WParams P, int nblk, int merge) {
+    __shared__ double2 s_p[1024];
     WState *st = P.st;
     const int MM = P.M * P.M;
     if (st->err) return;
     const unsigned long long tn = st->t + 1;
     const size_t slot = (size_t)(tn % (unsigned long long)P.rho_hist);
-    for (int k = threadIdx.x; k < MM; k += blockDim.x) {
-        double x = 0.0, y = 0.0;
-        for (int b = 0; b < nblk; ++b) {
+    const int T = 1024 / MM, k = (int)threadIdx.x % MM, j = (int)threadIdx.x / MM;
+    double x = 0.0, y = 0.0;
+    if (j < T)
+#pragma unroll 8
+        for (int b = j; b < nblk; b += T) {
             const double2 v = P.rho_part[(size_t)b * MM + k];
             x += v.x;
             y += v.y;
         }
-        P.rho_ring[slot * MM + k] = make_double2(x, y);
-    }
+    s_p[threadIdx.x] = make_double2(x, y);
     __syncthreads();
+    if ((int)threadIdx.x < MM) {
+        for (int u = 1; u < T; ++u) {
+            x += s_p[u * MM + threadIdx.x].x;
+            y += s_p[u * MM + threadIdx.x].y;
+        }
+        P.rho_ring[slot * MM + threadIdx.x] = make_double2(x, y);
+    }
     if (threadIdx.x == 0) {
         const unsigned long long groups = merge ? st->n_groups : st->n_cur;
         WRec r;
@@ -472,7 +651,7 @@ __global__ void k_w_build_lut(double2 *lut, float2 *lutf, float2 *lutlo, const d
 }
 
 // W[(a,b)][(a',b')] = U[a,a'] conj(U[b,b']) exp(-(q_a - q_b)(eta_0 q_a - conj(eta_0) q_b))
-__global__ void k_w_build_w(double2 *w, float4 *wf, const double2 *U, const double2 *eta, const double *q, int M) {
+__global__ void k_w_build_w(double2 *w, float4 *wf, float *lw, const double2 *U, const double2 *eta, const double *q, int M) {
     const int MM = M * M;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < MM * MM; i += gridDim.x * blockDim.x) {
         const int child = i / MM, par = i % MM;
@@ -490,6 +669,7 @@ __global__ void k_w_build_w(double2 *w, float4 *wf, const double2 *U, const doub
         w[i] = v;
         const float hx = (float)v.x, hy = (float)v.y;
         wf[i] = make_float4(hx, hy, (float)(v.x - (double)hx), (float)(v.y - (double)hy));
+        lw[(size_t)par * MM + child] = (float)log2(v.x * v.x + v.y * v.y);
     }
 }
 
@@ -508,7 +688,7 @@ __global__ void k_w_clear_table(WSlot *slots, unsigned long long *ttie, unsigned
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct WLayout {
-    size_t klo[2], khi[2], amps[2], slot_of, groups, trep, slots, ttie, lut, lutf, lutlo, w, wf, U, eta, q,
+    size_t klo[2], khi[2], amps[2], slot_of, groups, slots, ttie, lut, lutf, lutlo, w, wf, lw, U, eta, q,
         rho_part, rho, stats, state, total;
     unsigned long long tcap;
 };
@@ -551,7 +731,6 @@ WLayout wide_layout(const qp_config *c) {
     }
     L.slot_of = take(mp * 4);
     L.groups = take(mg * 4);
-    L.trep = take(tcap * 4);
     L.slots = take(tcap * sizeof(WSlot));
     L.ttie = take(tcap * 8);
     L.lut = take(nlut * 16);
@@ -559,10 +738,11 @@ WLayout wide_layout(const qp_config *c) {
     L.lutlo = take(nlut * 8);
     L.w = take((size_t)MM * MM * 16);
     L.wf = take((size_t)MM * MM * 16);
+    L.lw = take((size_t)MM * MM * 4);
     L.U = take((size_t)MM * 16);
     L.eta = take((size_t)c->dkmax * 16);
     L.q = take((size_t)c->M * 8);
-    L.rho_part = take((size_t)2048 * MM * 16);
+    L.rho_part = take((size_t)kWMaxBlocks * MM * 16);
     L.rho = take((size_t)R * MM * 16);
     L.stats = take((size_t)R * sizeof(WRec));
     L.total = off;
@@ -580,7 +760,8 @@ struct qp_wide {
     WParams P{};
     char *ws = nullptr;
     cudaStream_t stream = nullptr;
-    int nsm = 0, nblk = 0;
+    int nsm = 0, nblk = 0, xblk = 0;   // blocks of the table passes and of the expansion
+    size_t xsmem = 0;                  // shared memory of the expansion
     bool have_eta = false, have_state = false, failed = false;
     std::string err;
 };
@@ -604,14 +785,28 @@ qp_status wide_set_mask_params(qp_wide *w, const std::vector<int> &P) {
     for (int p : P)
         if (p >= 1) in[p - 1] = 1;
     int np = 0, nc = 0;
-    for (int p = 0; p < dk; ++p) {
-        if (in[p]) w->P.pp[np++] = p;
-        else w->P.co[nc++] = p;
-    }
+    for (int p = 0; p < dk; ++p) ++(in[p] ? np : nc);
     if (6 * np > 64) return wfail(w, QP_ERR_ARG, "wide keys: P' may hold at most 10 positions (64-bit group key)");
     if (6 * nc > 64) return wfail(w, QP_ERR_ARG, "wide keys: at most 10 positions outside P' (64-bit tie key)");
-    w->P.npp = np;
-    w->P.nco = nc;
+    for (int side = 0; side < 2; ++side) {   // runs of consecutive positions within a word of eight
+        WRuns R{};
+        for (int p = 0; p < dk;) {
+            if ((bool)in[p] != (side == 0)) {
+                ++p;
+                continue;
+            }
+            int e = p + 1;
+            while (e < dk && (e & 7) && (bool)in[e] == (side == 0)) ++e;
+            R.word[R.n] = (unsigned char)(p >> 3);
+            R.shift[R.n] = (unsigned char)(6 * (p & 7));
+            R.off[R.n] = (unsigned char)(6 * R.npos);
+            R.mask[R.n] = (1ull << (6 * (e - p))) - 1ull;
+            ++R.n;
+            R.npos += e - p;
+            p = e;
+        }
+        (side == 0 ? w->P.pp : w->P.co) = R;
+    }
     return QP_OK;
 }
 
@@ -661,7 +856,7 @@ qp_status qp_wide_create(const qp_config *cfg, void *d_workspace, size_t bytes, 
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&w->nsm, cudaDevAttrMultiProcessorCount, dev);
-    w->nblk = std::min(2048, std::max(1, w->nsm) * 4);
+    w->nblk = std::max(1, w->nsm) * 8;
     WParams &P = w->P;
     P.M = M;
     P.dkmax = cfg->dkmax;
@@ -669,26 +864,16 @@ qp_status qp_wide_create(const qp_config *cfg, void *d_workspace, size_t bytes, 
     P.rho_hist = cfg->rho_history ? cfg->rho_history : 4096;
     P.max_paths = cfg->max_paths;
     P.max_groups = cfg->max_groups ? cfg->max_groups : cfg->max_paths;
-    P.tcap_mask = L.tcap - 1;
+    P.tcap = L.tcap;
     P.theta2 = cfg->theta * cfg->theta;
     P.theta2f = (float)P.theta2;
     P.tie_rel = cfg->precision == QP_C64 ? 1e-6 : 1e-12;   // the narrow engines' windows (reading R4, R11)
     for (int i = 0; i < M; ++i) P.q[i] = cfg->q[i];
-    P.ndelta = 0;
     for (int a = 0; a < M; ++a)
-        for (int b = 0; b < M; ++b) {
-            const double d = cfg->q[a] - cfg->q[b];   // as the kernel forms it
-            int k = -1;
-            if (d != 0.0) {
-                for (int j = 0; j < P.ndelta; ++j)
-                    if (P.delta[j] == d) k = j;
-                if (k < 0) {
-                    k = P.ndelta;
-                    P.delta[P.ndelta++] = d;
-                }
-            }
-            P.dsel[a * M + b] = (signed char)k;
-        }
+        for (int b = 0; b < M; ++b) P.dq2[a * M + b] = (float)(-2.0 * 1.4426950408889634 * (cfg->q[a] - cfg->q[b]));
+    // no filter, or one in the range where squares lose precision to
+    // underflow: every child is formed
+    P.log2_theta2 = P.theta2 > (P.c64 ? 1e-36 : 1e-290) ? (float)std::log2(P.theta2) : -INFINITY;
     char *ws = w->ws;
     for (int k = 0; k < 2; ++k) {
         P.klo[k] = reinterpret_cast<unsigned long long *>(ws + L.klo[k]);
@@ -697,7 +882,6 @@ qp_status qp_wide_create(const qp_config *cfg, void *d_workspace, size_t bytes, 
     }
     P.slot_of = reinterpret_cast<unsigned *>(ws + L.slot_of);
     P.groups = reinterpret_cast<unsigned *>(ws + L.groups);
-    P.trep = reinterpret_cast<unsigned *>(ws + L.trep);
     P.slots = reinterpret_cast<WSlot *>(ws + L.slots);
     P.ttie = reinterpret_cast<unsigned long long *>(ws + L.ttie);
     P.lut = reinterpret_cast<const double2 *>(ws + L.lut);
@@ -705,6 +889,7 @@ qp_status qp_wide_create(const qp_config *cfg, void *d_workspace, size_t bytes, 
     P.lutlo = reinterpret_cast<const float2 *>(ws + L.lutlo);
     P.w = reinterpret_cast<const double2 *>(ws + L.w);
     P.wf = reinterpret_cast<const float4 *>(ws + L.wf);
+    P.lw = reinterpret_cast<const float *>(ws + L.lw);
     P.rho_part = reinterpret_cast<double2 *>(ws + L.rho_part);
     P.rho_ring = reinterpret_cast<double2 *>(ws + L.rho);
     P.stats = reinterpret_cast<WRec *>(ws + L.stats);
@@ -715,15 +900,18 @@ qp_status qp_wide_create(const qp_config *cfg, void *d_workspace, size_t bytes, 
     if (wide_set_mask_params(w, full) != QP_OK && cfg->dkmax > 0) {
         // the full mask of a long window does not fit a 64-bit group key:
         // a mask must be set before qp_wide_set_rho0
-        w->P.npp = -1;
+        w->P.pp.npos = -1;
     }
-    if (cudaFuncSetAttribute(k_w_expand<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kWMaxTabDelta * kWThreads * 16) != cudaSuccess ||
-        cudaFuncSetAttribute(k_w_expand<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kWMaxTabDelta * kWThreads * 8) != cudaSuccess) {
+    const void *fn = P.c64 ? (const void *)k_w_expand<true> : (const void *)k_w_expand<false>;
+    w->xsmem = expand_smem(MM, cfg->dkmax - 1, P.c64 != 0);
+    int res = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)expand_smem(kWMaxMM, kWMaxDk - 1, P.c64 != 0)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, fn, kWThreads, w->xsmem) != cudaSuccess || res < 1) {
         delete w;
         return QP_ERR_CUDA;
     }
+    w->xblk = std::min(kWMaxBlocks, std::max(1, w->nsm) * res);
     *out = w;
     return QP_OK;
 }
@@ -752,6 +940,7 @@ qp_status qp_wide_set_eta(qp_wide *w, const double *re, const double *im, int n)
                                                  reinterpret_cast<const double *>(ws + w->L.q), M, dk);
     k_w_build_w<<<16, 256, 0, w->stream>>>(reinterpret_cast<double2 *>(ws + w->L.w),
                                            reinterpret_cast<float4 *>(ws + w->L.wf),
+                                           reinterpret_cast<float *>(ws + w->L.lw),
                                            reinterpret_cast<const double2 *>(ws + w->L.U),
                                            reinterpret_cast<const double2 *>(ws + w->L.eta),
                                            reinterpret_cast<const double *>(ws + w->L.q), M);
@@ -791,7 +980,7 @@ qp_status qp_wide_set_rho0(qp_wide *w, const double *re, const double *im) {
     if (!w) return QP_ERR_ARG;
     if (!re) return wfail(w, QP_ERR_ARG, "rho0 required");
     if (!w->have_eta) return wfail(w, QP_ERR_STATE, "qp_wide_set_eta must come before qp_wide_set_rho0");
-    if (w->P.npp < 0) return wfail(w, QP_ERR_STATE, "set a mask whose P' fits the 64-bit group key first");
+    if (w->P.pp.npos < 0) return wfail(w, QP_ERR_STATE, "set a mask whose P' fits the 64-bit group key first");
     const int M = w->cfg.M, MM = M * M;
     std::vector<unsigned long long> lo, hi;
     std::vector<double2> amps, rho(MM);
@@ -840,30 +1029,15 @@ qp_status qp_wide_step(qp_wide *w, int nsteps) {
     qp_status r = wide_read_state(w, &s);
     if (r != QP_OK) return r;
     unsigned long long t = s.t;
-    const int g = w->nblk;
-    const int MMh = w->cfg.M * w->cfg.M;
-    // lanes per group in the expansion: complex64 is latency-bound (shorter
-    // chains per lane pay for the repeated per-group set-up); FP64 is bound
-    // by its pipe (1/64 of FP32), where the repeated set-up would cost more
-    const int sub_n = !w->P.c64 ? 1 : (MMh >= 32 ? 4 : (MMh >= 16 ? 2 : 1));
     for (int k = 0; k < nsteps; ++k, ++t) {
         const int merge = t + 1 >= (unsigned long long)w->cfg.dkmax ? 1 : 0;
         if (merge) {
-            k_w_insert<<<g, kWThreads, 0, w->stream>>>(w->P);
-            k_w_tie<false><<<g, kWThreads, 0, w->stream>>>(w->P);
-            k_w_tie<true><<<g, kWThreads, 0, w->stream>>>(w->P);
+            k_w_insert<<<w->nblk, kWThreads, 0, w->stream>>>(w->P);
+            k_w_tie<<<w->nblk, kWThreads, 0, w->stream>>>(w->P);
         }
-        const bool tab = w->P.ndelta <= kWMaxTabDelta;
-        const size_t tsm = tab ? (size_t)w->P.ndelta * kWThreads * (w->P.c64 ? 8 : 16) : 0;
-        if (w->P.c64) {
-            if (tab) k_w_expand<true, true><<<g, kWThreads, tsm, w->stream>>>(w->P, merge, sub_n);
-            else k_w_expand<true, false><<<g, kWThreads, 0, w->stream>>>(w->P, merge, sub_n);
-        } else {
-            if (tab) k_w_expand<false, true><<<g, kWThreads, tsm, w->stream>>>(w->P, merge, sub_n);
-            else k_w_expand<false, false><<<g, kWThreads, 0, w->stream>>>(w->P, merge, sub_n);
-        }
-        k_w_rho<<<g, kWThreads, 0, w->stream>>>(w->P);
-        k_w_finalize<<<1, 64, 0, w->stream>>>(w->P, g, merge);
+        if (w->P.c64) k_w_expand<true><<<w->xblk, kWThreads, w->xsmem, w->stream>>>(w->P, merge);
+        else k_w_expand<false><<<w->xblk, kWThreads, w->xsmem, w->stream>>>(w->P, merge);
+        k_w_finalize<<<1, 1024, 0, w->stream>>>(w->P, w->xblk, merge);
         QW_CUDA(w, cudaGetLastError());
     }
     return QP_OK;
