@@ -268,6 +268,15 @@ __device__ __forceinline__ unsigned atom_add_acq_rel_gpu(unsigned *p, unsigned v
     return old;
 }
 
+// Programmatic dependent launch: the stream engine's kernels are launched while the
+// kernel before them on the stream still runs (launch_pdl).  pdl_trigger lets
+// the next kernel's blocks start as this one's leave; pdl_wait returns once
+// every earlier kernel has completed and its writes are visible.  Before the
+// wait a kernel reads only what the host set up and waited for (propagator
+// and history tables).  Both do nothing in a kernel launched the plain way.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Asynchronous 16-byte global -> shared copy (both addresses 16-byte
 // aligned); cp_async_wait_all waits for this thread's copies.
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
@@ -1340,6 +1349,12 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     __shared__ double2 s_w[C64 ? 1 : MM * MM];
     __shared__ float4 s_wf[C64 ? MM * MM : 1];
     __shared__ float4 s_rt[NW][MM];
+    pdl_trigger();
+    for (int i = threadIdx.x; i < MM * MM; i += NT) {
+        if constexpr (C64) s_wf[i] = P.wtabf[i];
+        else s_w[i] = P.wtab[i];
+    }
+    pdl_wait();
     // the state and both buffers' region sizes in one trip
     if ((int)threadIdx.x < 2 * MM) s_rn[threadIdx.x] = __ldcg(P.reg_n + threadIdx.x);
     if (threadIdx.x == 32) {
@@ -1347,10 +1362,6 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
         s_t = __ldcg(&st->t);
         s_pend = __ldcg(&st->rho_pending);
         s_pnblk = __ldcg(&st->rho_nblk);
-    }
-    for (int i = threadIdx.x; i < MM * MM; i += NT) {
-        if constexpr (C64) s_wf[i] = P.wtabf[i];
-        else s_w[i] = P.wtab[i];
     }
     __syncthreads();
     if (s_err) return;
@@ -1748,12 +1759,48 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
     static_assert(!BATCH || NX == 1, "batches: P' a prefix of the window");
     constexpr bool kTileAccS = !BATCH && M * M >= 9 && C64;   // per-warp tile sums of rho (see the accumulators)
     DevState *st = P.st;
+    // Before the previous step's kernel is waited for: the propagator table
+    // and, on the chance that the window is full, its history tables (asynchronous
+    // copies, waited for before the first pass A)
+    __shared__ double2 s_w[C64 || BATCH ? 1 : MM * MM];   // FP64 weights (FP64 path only)
+    __shared__ float4 s_wf[BATCH ? 1 : MM * MM];
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    Tab tab = tab_global(P, P.dkmax, 0);
+    // (rows are whole multiples of kLutEntries entries, so every copy is
+    // 16-byte aligned)
+    auto stage_tables = [&](const Tab &from) {
+        const int n = P.nchunks * kLutEntries;
+        if constexpr (C64) {
+            float2 *hi = reinterpret_cast<float2 *>(s_dyn + Lay::lut), *lo = hi + n;
+            for (int i = threadIdx.x; i < n / 2; i += NT) {
+                cp_async16(hi + 2 * i, from.hi + 2 * i);
+                cp_async16(lo + 2 * i, from.lo + 2 * i);
+            }
+            tab.hi = hi;
+            tab.lo = lo;
+        } else {
+            double2 *et = reinterpret_cast<double2 *>(s_dyn + Lay::lut);
+            for (int i = threadIdx.x; i < n * P.ndelta; i += NT) cp_async16(et + i, from.et + i);
+            tab.et = et;
+        }
+    };
+    if constexpr (!BATCH) {
+        for (int i = threadIdx.x; i < MM * MM; i += NT) {
+            if constexpr (!C64) s_w[i] = P.wtab[i];
+            s_wf[i] = P.wtabf[i];
+        }
+        if (lut_smem && P.ndelta) stage_tables(tab);
+        pdl_wait();
+    }
     // (device state read through L2: the persistent batch kernel runs
     // several steps in one launch)
-    if (__ldcg(&st->err)) return;
     const unsigned long long t = __ldcg(&st->t), tn = t + 1;
-    // launched behind the regular kernel, which just took this step (its new t + 1)
-    if ((flags & kFlagAfterRegular) && __ldcg(&st->reg_done) == tn) return;
+    // an earlier error, or launched behind the regular kernel, which just took
+    // this step (its new t + 1)
+    if (__ldcg(&st->err) || ((flags & kFlagAfterRegular) && __ldcg(&st->reg_done) == tn)) {
+        if constexpr (!BATCH) cp_async_wait_all();
+        return;
+    }
     if constexpr (BATCH) finish_pending_rho_batch(P, st, M * M, false);   // blocks b < n_inst: instance b
     const int in = (int)(t & 1), outp = (int)(tn & 1), cs = (int)(tn % 3);
     const bool merge = tn >= (unsigned long long)P.dkmax;
@@ -1768,7 +1815,6 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
     unsigned long long *keys_out = P.keys[outp];
     AmpT *amps_out = static_cast<AmpT *>(P.amps[outp]);
 
-    extern __shared__ __align__(16) unsigned char s_dyn[];
     double2 *s_gS = reinterpret_cast<double2 *>(s_dyn + Lay::gS);
     unsigned long long *s_grep = reinterpret_cast<unsigned long long *>(s_dyn + Lay::grep);
     WT *s_wm = reinterpret_cast<WT *>(s_dyn + Lay::wm);
@@ -1783,8 +1829,6 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
     unsigned *s_xmask = reinterpret_cast<unsigned *>(s_dyn + Lay::stg);
     static_assert(NX == 1 || (Lay::stage && (size_t)Lay::NSTG * MM * sizeof(AmpT) >= (size_t)S * NX * 4),
                   "sub-group member masks live in the staging buffer");
-    __shared__ double2 s_w[C64 || BATCH ? 1 : MM * MM];   // FP64 weights (FP64 path only)
-    __shared__ float4 s_wf[BATCH ? 1 : MM * MM];
     __shared__ long long s_nr[MM], s_tile0[MM + 1];
     __shared__ unsigned s_wsum[NW][MM];
     __shared__ unsigned long long s_base[MM], s_tot[MM], s_kprev;
@@ -1812,33 +1856,19 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
     int *s_t0 = reinterpret_cast<int *>(s_dyn + Lay::lut + (((size_t)(BATCH ? P.n_inst : 1) * (MM + 1) * 16 + 15) & ~(size_t)15));
     const float tie_f = (float)tie_d;
 
-    // weights and the history tables of this window length (batches read
-    // their instance's from global memory per tile)
+    // while the window fills: the history tables of its length instead (each
+    // thread's copies follow its own earlier ones; batches read their
+    // instance's tables from global memory per tile)
     if constexpr (!BATCH)
-        for (int i = threadIdx.x; i < MM * MM; i += NT) {
-            if constexpr (!C64) s_w[i] = P.wtab[i];
-            s_wf[i] = P.wtabf[i];
-        }
-    Tab tab = tab_global(P, n_act, 0);
-    // (asynchronous copies, waited for before the first pass A: the tables
-    // arrive while the first tile loads; rows are whole multiples of
-    // kLutEntries entries, so every copy is 16-byte aligned)
-    if (!BATCH && lut_smem && P.ndelta) {
-        const int n = P.nchunks * kLutEntries;
-        if constexpr (C64) {
-            float2 *hi = reinterpret_cast<float2 *>(s_dyn + Lay::lut), *lo = hi + n;
-            for (int i = threadIdx.x; i < n / 2; i += NT) {
-                cp_async16(hi + 2 * i, tab.hi + 2 * i);
-                cp_async16(lo + 2 * i, tab.lo + 2 * i);
+        if (n_act != P.dkmax) {
+            const Tab now = tab_global(P, n_act, 0);
+            if (lut_smem && P.ndelta) {
+                cp_async_wait_all();
+                stage_tables(now);
+            } else {
+                tab = now;
             }
-            tab.hi = hi;
-            tab.lo = lo;
-        } else {
-            double2 *et = reinterpret_cast<double2 *>(s_dyn + Lay::lut);
-            for (int i = threadIdx.x; i < n * P.ndelta; i += NT) cp_async16(et + i, tab.et + i);
-            tab.et = et;
         }
-    }
     if (threadIdx.x == 0) s_any = 0;
     if constexpr (kTileAccS)
         for (int i = threadIdx.x; i < NW * MM; i += NT) (&s_wrho[0][0])[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -2882,6 +2912,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
 template <int M, bool C64, int NX, int S>
 __global__ void __launch_bounds__(kStreamThreads, (M == 2 || (M == 3 && C64)) ? 2 : 1)
     k_stream_step(Params P, int flags) {
+    pdl_trigger();
     stream_step_body<M, C64, NX, S, false>(P, flags);
 }
 
@@ -3782,6 +3813,23 @@ size_t batch_smem(const qp_ctx *c) {
     return c->P.n_inst > 1 ? (size_t)c->P.n_inst * (MM + 1) * sizeof(double2) : 0;
 }
 
+// A launch that may start while the kernel before it on the stream still runs
+// (the kernel waits for it itself: pdl_wait); plain where events between the
+// kernels time them (dep false).
+cudaError_t launch_pdl(const void *fn, int grid, int block, size_t smem, cudaStream_t stream, void **args, bool dep) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = at;
+    cfg.numAttrs = dep ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 template <int M, typename Amp>
 cudaError_t launch_step_t(qp_ctx *c, cudaEvent_t *ev) {
     constexpr bool C64 = sizeof(Amp) == sizeof(float2);
@@ -3842,7 +3890,7 @@ cudaError_t stream_residency(qp_ctx *c, const void *fn, size_t sm, size_t sm_mos
 // Grid of the stream kernel: every block resident (tiles are taken by
 // ticket, so blocks beyond the co-resident count would only start after a
 // first wave), at most bps_exp per SM and kMaxExpandBlocks in all.
-cudaError_t launch_stream_tile(qp_ctx *c, bool after_regular) {
+cudaError_t launch_stream_tile(qp_ctx *c, bool after_regular, bool dep) {
     const qp::StreamKernel k = stream_kernel(c);
     const size_t lutb = stream_lut_bytes(c, c->cfg.precision == QP_C64);
     const size_t sm = k.bytes + lutb;
@@ -3851,7 +3899,7 @@ cudaError_t launch_stream_tile(qp_ctx *c, bool after_regular) {
     const int g = std::min(c->nsm * std::min(c->bps_exp, c->scache_res), kMaxExpandBlocks);
     int flags = (lutb ? kFlagLutSmem : 0) | (after_regular ? kFlagAfterRegular : 0);
     void *args[] = {(void *)&c->P, (void *)&flags};
-    return cudaLaunchKernel(k.fn, dim3(g), dim3(kStreamThreads), args, sm, c->stream);
+    return launch_pdl(k.fn, g, kStreamThreads, sm, c->stream, args, dep);
 }
 
 // Batched stream kernel: an ordinary launch of one step (every block
@@ -3879,7 +3927,7 @@ cudaError_t launch_stream_batch(qp_ctx *c, int nsteps, bool coop) {
 // The regular stream kernel (no filter): every block resident, at most
 // kMaxExpandBlocks (block partials).
 template <int M, bool C64>
-cudaError_t launch_stream_regular(qp_ctx *c) {
+cudaError_t launch_stream_regular(qp_ctx *c, bool dep) {
     const void *fn = (const void *)k_stream_regular<M, C64>;
     const size_t lutb = stream_lut_bytes(c, C64);
     if (c->rcache_fn != fn || c->rcache_smem != lutb) {
@@ -3894,8 +3942,9 @@ cudaError_t launch_stream_regular(qp_ctx *c) {
         c->rcache_res = nb;
     }
     const int g = std::min(c->nsm * c->rcache_res, kMaxExpandBlocks);
-    k_stream_regular<M, C64><<<g, kRegThreads, lutb, c->stream>>>(c->P, lutb ? 1 : 0);
-    return cudaGetLastError();
+    int lut_smem = lutb ? 1 : 0;
+    void *args[] = {(void *)&c->P, (void *)&lut_smem};
+    return launch_pdl(fn, g, kRegThreads, lutb, c->stream, args, dep);
 }
 
 // The kernels that a step of the stream engine may need: the regular kernel,
@@ -3925,7 +3974,7 @@ cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind) {
     if (ev) cudaEventRecord(ev[0], c->stream);
     if constexpr (M < 4) {
         if (kind == kStepRegular || after_regular) {
-            cudaError_t e = launch_stream_regular<M, C64>(c);
+            cudaError_t e = launch_stream_regular<M, C64>(c, ev == nullptr);
             if (e != cudaSuccess) return e;
         }
     }
@@ -3935,7 +3984,7 @@ cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind) {
     }
     cudaError_t e = cudaSuccess;
     if (c->P.n_inst > 1) e = launch_stream_batch(c, 1, false);
-    else if (kind != kStepRegular) e = launch_stream_tile(c, after_regular);
+    else if (kind != kStepRegular) e = launch_stream_tile(c, after_regular, ev == nullptr);
     if (e != cudaSuccess) return e;
     if (ev) {
         cudaEventRecord(ev[3], c->stream);
@@ -4636,13 +4685,19 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
         if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("persistent launch: ") + cudaGetErrorString(e));
         return QP_OK;
     }
-    if (c->use_graph && c->graph_dirty) {
+    // graphs where several kernels or steps go into one; single steps of the
+    // stream engine are launched as they are (dependent launches follow each
+    // other without the graph launch's gap, and nothing is captured again
+    // after qp_set_rho0; the table engine's four kernels are 6 % slower that
+    // way)
+    const bool graphs = c->use_graph && (c->graph_steps > 1 || !c->use_stream);
+    if (graphs && c->graph_dirty) {
         drop_graphs(c);
         c->graph_dirty = false;
     }
     for (int s = 0; s < nsteps;) {
         const StepKind kind = step_kind(c, t0 + s + 1);
-        if (!c->use_graph) {
+        if (!graphs) {
             const cudaError_t e = launch_step(c, nullptr, kind);
             if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
             ++s;
