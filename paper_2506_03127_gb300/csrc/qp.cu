@@ -2799,49 +2799,48 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
                 }
             }
         }
-        if constexpr (BATCH) {
-            // the tile's part of its instance's rho(t+1) and survivor count:
-            // FP64 warp sums added to the block's sums (shared FP64 atomics)
-            double2 *acc = s_acc + (size_t)inst * (MM + 1);
+        if constexpr (kTileAcc) {
+            // the tile's rho(t+1): warp sums by halving (Kahan terms as the
+            // pairs' second words), each component in one lane.  Batches add
+            // it to the instance's block sums (shared FP64 atomics), single
+            // problems to the warp's pair (TwoSum).  (Batches widened every
+            // lane's value and reduced in FP64, 40 additions of 16 cycles per
+            // warp and tile: half of the FP64 pipe's time in the sweep)
+            constexpr int V = MM <= 4 ? 8 : 32;
+            const int idx = rs_index<V>();
+            const bool mine = idx < 2 * MM && (lane & (32 / V - 1)) == 0u;
+            typename std::conditional<C64, float, double>::type sv[V], ev[C64 ? V : 1];
 #pragma unroll
-            for (int k = 0; k < MM; ++k) {
-                double x = to_d(tacc[k].x), y = to_d(tacc[k].y);
-                if constexpr (kKahan) {
-                    x -= to_d(tcmp[k].x);
-                    y -= to_d(tcmp[k].y);
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    x += __shfl_down_sync(0xffffffffu, x, o);
-                    y += __shfl_down_sync(0xffffffffu, y, o);
-                }
-                if (lane == 0 && (x != 0.0 || y != 0.0)) {
-                    atomicAdd(&acc[k].x, x);
-                    atomicAdd(&acc[k].y, y);
+            for (int k = 0; k < V; ++k) {
+                sv[k] = 0;
+                if (k < 2 * MM) sv[k] = (k & 1) ? tacc[k >> 1].y : tacc[k >> 1].x;
+                if constexpr (C64) {
+                    ev[k] = 0;
+                    if constexpr (kKahan)
+                        if (k < 2 * MM) ev[k] = (k & 1) ? -tcmp[k >> 1].y : -tcmp[k >> 1].x;
                 }
             }
-            if (threadIdx.x == 0 && !lbfail) {
-                unsigned long long kt = 0;
-                for (int c = 0; c < MM; ++c) kt += s_tot[c];
-                atomicAdd(&acc[MM].x, (double)kt);
-            }
-        }
-        if constexpr (kTileAccS) {
-            // the tile's rho(t+1): warp sums (plain FP32), added by lane 0 to
-            // the warp's pair with TwoSum (the error kept)
-#pragma unroll
-            for (int k = 0; k < MM; ++k) {
-                auto x = tacc[k].x, y = tacc[k].y;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    x += __shfl_down_sync(0xffffffffu, x, o);
-                    y += __shfl_down_sync(0xffffffffu, y, o);
+            if constexpr (C64) warp_reduce_scatter<V>(sv, ev);
+            else warp_reduce_scatter<V>(sv);
+            if constexpr (BATCH) {
+                double *acc = reinterpret_cast<double *>(s_acc + (size_t)inst * (MM + 1));
+                if (mine) {
+                    double x;
+                    if constexpr (C64) x = f2d_exact(sv[0]) + f2d_exact(ev[0]);
+                    else x = sv[0];
+                    if (x != 0.0) atomicAdd(acc + idx, x);
                 }
-                if (lane == 0) {
-                    float4 a = s_wrho[warp][k];
-                    two_sum_acc(a.x, a.y, x);
-                    two_sum_acc(a.z, a.w, y);
-                    s_wrho[warp][k] = a;
+                if (threadIdx.x == 0 && !lbfail) {
+                    unsigned long long kt = 0;
+                    for (int c = 0; c < MM; ++c) kt += s_tot[c];
+                    atomicAdd(acc + 2 * MM, (double)kt);
+                }
+            } else if constexpr (C64) {
+                if (mine) {
+                    float2 a = reinterpret_cast<float2 *>(&s_wrho[warp][0])[idx];
+                    two_sum_acc(a.x, a.y, sv[0]);
+                    a.y += ev[0];
+                    reinterpret_cast<float2 *>(&s_wrho[warp][0])[idx] = a;
                 }
             }
         }
