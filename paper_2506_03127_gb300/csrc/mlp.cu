@@ -985,6 +985,203 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kRollThreads) k_roll
     }
 }
 
+// The rollout of networks of up to 256 columns over a cluster of eight blocks,
+// a warp per 8 columns of layers 1 and 2.  What bounds it is the latency of
+// one step: 18 + 16 + 16 dependent MMAs along k, the tanh of 2 x 16 x 256
+// values and two cluster barriers; on two blocks (a layer each) the tanh of a
+// layer (16 per thread), the features packed anew every step and the traffic of 8 warps
+// re-reading the weights made it 10.9 us per step at 16 instances.
+//   - every block holds its 32 rows of W1^T and W2^T, all of W3^T, all
+//     activations and the state: layer 3 and the update run in every block,
+//     so rho never crosses and two barriers per step remain (h1 complete, h2
+//     complete; each also frees the other's buffer for the next step);
+//   - a step's rho is one 8-column block of the feature matrix, kept in a
+//     ring of L blocks that the MMA's row addresses follow: only the new
+//     block is written;
+//   - a warp's 16 x 8 piece of h is put together in its own block and copied
+//     to the others in 16-byte rows.
+// Same MMA, k order and epilogues as k_rollout_fused and the step kernels:
+// the trajectories are the same bit for bit.
+constexpr int kClBlocks = 8, kClThreads = 128, kClCols = 32;   // columns of a block
+
+inline size_t roll_cluster_smem(int MT, int K1, int Kw) {
+    return ((size_t)kClCols * (K1 + 8) + (size_t)(kClCols + 8) * (Kw + 8) + (size_t)16 * MT * (K1 + 8) +
+            (size_t)2 * 16 * MT * (Kw + 8)) * 2 + (size_t)2 * 16 * MT * 8 * 4;
+}
+
+template <int MT>
+__global__ void __cluster_dims__(kClBlocks, 1, 1) __launch_bounds__(kClThreads) k_rollout_cluster(RollArgs a) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    extern __shared__ __align__(16) unsigned char s_roll[];
+    const int l1 = a.K1 + 8, lw = a.Kw + 8;
+    __nv_bfloat16 *sW1 = reinterpret_cast<__nv_bfloat16 *>(s_roll), *sW2 = sW1 + kClCols * l1;
+    __nv_bfloat16 *sW3 = sW2 + kClCols * lw, *sX = sW3 + 8 * lw;
+    __nv_bfloat16 *sH1 = sX + 16 * MT * l1, *sH2 = sH1 + 16 * MT * lw;
+    float *sY = reinterpret_cast<float *>(sH2 + 16 * MT * lw), *sR = sY + 16 * MT * 8;   // y; rho(t - 1)
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
+    const int c0 = rank * kClCols + warp * 8;   // this warp's columns
+    const bool busy = c0 < a.width;
+    // weights (rows past the width: zeros), activations and features zeroed
+    for (int i = tid; i < kClCols * (a.K1 / 8); i += kClThreads) {
+        const int r = i / (a.K1 / 8), c = (i % (a.K1 / 8)) * 8, n = rank * kClCols + r;
+        *reinterpret_cast<uint4 *>(sW1 + r * l1 + c) =
+            n < a.width ? *reinterpret_cast<const uint4 *>(a.w1t + (size_t)n * a.K1 + c) : make_uint4(0, 0, 0, 0);
+    }
+    for (int i = tid; i < (kClCols + 8) * (a.Kw / 8); i += kClThreads) {
+        const int r = i / (a.Kw / 8), c = (i % (a.Kw / 8)) * 8, n = r < kClCols ? rank * kClCols + r : r - kClCols;
+        const __nv_bfloat16 *src = r < kClCols ? a.w2t : a.w3t;   // (sW3 follows sW2)
+        *reinterpret_cast<uint4 *>(sW2 + r * lw + c) =
+            r >= kClCols || n < a.width ? *reinterpret_cast<const uint4 *>(src + (size_t)n * a.Kw + c) : make_uint4(0, 0, 0, 0);
+    }
+    for (int i = tid; i < 16 * MT * l1; i += kClThreads) sX[i] = __float2bfloat16_rn(0.f);
+    for (int i = tid; i < 2 * 16 * MT * lw; i += kClThreads) sH1[i] = __float2bfloat16_rn(0.f);
+    __syncthreads();
+    for (int i = tid; i < a.n * a.L * 8; i += kClThreads) {   // step s in block s % L
+        const int m = i / (a.L * 8), s = a.t_from - a.L + (i / 8) % a.L, k = i % 8;
+        sX[m * l1 + (s % a.L) * 8 + k] = __float2bfloat16_rn(a.hist[((size_t)m * a.T + s) * 8 + k]);
+    }
+    for (int i = tid; i < a.n * a.n_par; i += kClThreads)
+        sX[(i / a.n_par) * l1 + 8 * a.L + i % a.n_par] = __float2bfloat16_rn(a.par[i]);
+    for (int i = tid; i < a.n * 8; i += kClThreads)
+        sR[i] = a.hist[((size_t)(i / 8) * a.T + a.t_from - 1) * 8 + i % 8];
+    // this thread's biases: columns c0 + 2 tq, + 1 of layers 1 and 2, outputs of layer 3
+    const int n = c0 + 2 * tq;
+    const float b1x = n < a.width ? a.b1[n] : 0.f, b1y = n + 1 < a.width ? a.b1[n + 1] : 0.f;
+    const float b2x = n < a.width ? a.b2[n] : 0.f, b2y = n + 1 < a.width ? a.b2[n + 1] : 0.f;
+    const float b3x = a.b3[2 * tq], b3y = a.b3[2 * tq + 1];
+    cluster.sync();
+    // tanh of this warp's 16 x 8 pieces into its own block, then 16-byte rows to the others
+    auto spread = [&](float (&acc)[MT][4], float bx, float by, __nv_bfloat16 *sH) {
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+            for (int r = 0; r < 4; r += 2) {
+                const int m = mt * 16 + g + (r >= 2 ? 8 : 0);
+                if (m < a.n && n < a.width)   // (width is a multiple of 8)
+                    *reinterpret_cast<__nv_bfloat162 *>(sH + m * lw + n) =
+                        __floats2bfloat162_rn(tanhf(acc[mt][r] + bx), tanhf(acc[mt][r + 1] + by));
+            }
+            __syncwarp();
+            const int m = mt * 16 + (lane & 15);
+            const uint4 v = *reinterpret_cast<const uint4 *>(sH + m * lw + c0);
+#pragma unroll
+            for (int p = 0; p < kClBlocks / 2; ++p) {
+                const int peer = (lane >> 4) * (kClBlocks / 2) + p;
+                if (peer != rank) *reinterpret_cast<uint4 *>(cluster.map_shared_rank(sH, peer) + m * lw + c0) = v;
+            }
+        }
+    };
+    auto zero = [&](float (&acc)[MT][4]) {
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[mt][r] = 0.f;
+    };
+    const int brow = lane & 7, bhalf = ((lane >> 3) & 1) * 8;
+    int s0 = a.t_from % a.L;   // ring block of step t - L
+    for (int t = a.t_from; t < a.t_to; ++t) {
+        float acc[MT][4];
+        if (busy) {
+            // layer 1: logical block b of the features is ring block s0 + b
+            // (mod L), parameters and padding where they are
+            zero(acc);
+            const __nv_bfloat16 *B = sW1 + (warp * 8 + brow) * l1 + bhalf;
+#pragma unroll 6
+            for (int kk = 0; kk < a.K1; kk += 16) {
+                int blk = (kk >> 3) + (lane >> 4);
+                if (blk < a.L) {
+                    blk += s0;
+                    if (blk >= a.L) blk -= a.L;
+                }
+                unsigned b0, b1;
+                ldmatrix_x2(b0, b1, B + kk);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    unsigned a0, a1, a2, a3;
+                    ldmatrix_x4(a0, a1, a2, a3, sX + (mt * 16 + (lane & 15)) * l1 + blk * 8);
+                    mma_bf16(acc[mt], a0, a1, a2, a3, b0, b1);
+                }
+            }
+            spread(acc, b1x, b1y, sH1);
+        }
+        cluster.sync();   // h1 complete; every block is done with h2
+        if (busy) {
+            zero(acc);
+            const __nv_bfloat16 *B = sW2 + (warp * 8 + brow) * lw + bhalf;
+#pragma unroll 8
+            for (int kk = 0; kk < a.Kw; kk += 16) {
+                unsigned b0, b1;
+                ldmatrix_x2(b0, b1, B + kk);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    unsigned a0, a1, a2, a3;
+                    ldmatrix_x4(a0, a1, a2, a3, sH1 + (mt * 16 + (lane & 15)) * lw + kk + (lane >> 4) * 8);
+                    mma_bf16(acc[mt], a0, a1, a2, a3, b0, b1);
+                }
+            }
+            spread(acc, b2x, b2y, sH2);
+        }
+        cluster.sync();   // h2 complete; every block is done with h1
+        // layer 3, in every block: warp mt takes rows 16 mt
+        if (warp < MT) {
+            float y[4] = {0.f, 0.f, 0.f, 0.f};
+            const __nv_bfloat16 *B = sW3 + brow * lw + bhalf, *A = sH2 + (warp * 16 + (lane & 15)) * lw + (lane >> 4) * 8;
+#pragma unroll 8
+            for (int kk = 0; kk < a.Kw; kk += 16) {
+                unsigned b0, b1, a0, a1, a2, a3;
+                ldmatrix_x2(b0, b1, B + kk);
+                ldmatrix_x4(a0, a1, a2, a3, A + kk);
+                mma_bf16(y, a0, a1, a2, a3, b0, b1);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) sY[(warp * 16 + g + (r >= 2 ? 8 : 0)) * 8 + 2 * tq + (r & 1)] = y[r] + ((r & 1) ? b3y : b3x);
+            __syncwarp();
+            // the update of k_rollout_update for this warp's instances
+            const int i = warp * 16 + lane;
+            if (lane < 16 && i < a.n) {
+                const float *prev = sR + i * 8;
+                float d[8];
+                for (int k = 0; k < 8; ++k) d[k] = sY[i * 8 + k] / a.out_scale;
+                const float tr = 0.5f * (d[0] + d[6]);
+                d[0] -= tr;
+                d[6] -= tr;
+                float r[8];
+                for (int k = 0; k < 8; ++k) r[k] = prev[k] + d[k];
+                const float re = 0.5f * (r[2] + r[4]), im = 0.5f * (r[3] - r[5]);
+                r[2] = re;
+                r[3] = im;
+                r[4] = re;
+                r[5] = -im;
+                r[1] = 0.f;
+                r[7] = 0.f;
+                const float c = 0.5f * (r[0] + r[6]), z = 0.5f * (r[0] - r[6]);
+                const float rad = sqrtf(z * z + r[2] * r[2] + r[3] * r[3]);
+                if (c > 0.f && rad > c) {
+                    const float f = c / rad;
+                    r[0] = c + f * z;
+                    r[6] = c - f * z;
+                    r[2] *= f;
+                    r[3] *= f;
+                    r[4] = r[2];
+                    r[5] = -r[3];
+                }
+                __nv_bfloat16 *blk = sX + i * l1 + s0 * 8;   // step t takes the place of step t - L
+                float *out = a.hist + ((size_t)i * a.T + t) * 8;
+                for (int k = 0; k < 8; ++k) {
+                    sR[i * 8 + k] = r[k];
+                    blk[k] = __float2bfloat16_rn(r[k]);
+                    if (rank == 0) out[k] = r[k];
+                }
+            }
+        }
+        if (++s0 == a.L) s0 = 0;
+        __syncthreads();
+    }
+    cluster.sync();   // no block leaves while another may still write to it
+}
+
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
@@ -1482,6 +1679,17 @@ qp_status qp_surrogate_rollout(qp_mlp *m, float *d_hist, int n, int T, int L, co
         ra.t_to = t_to;
         ra.ring = ring ? 1 : 0;
         ra.out_scale = out_scale;
+        const size_t csm = roll_cluster_smem(MT, m->K1, m->Kw);
+        if (m->width <= kClBlocks * kClCols && csm <= kSmemMax) {
+            const void *fc = MT == 1 ? (const void *)k_rollout_cluster<1> : (const void *)k_rollout_cluster<2>;
+            if (cudaFuncSetAttribute(fc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm) != cudaSuccess)
+                return mfail(m, QP_ERR_CUDA, "fused rollout set-up");
+            if (MT == 1) k_rollout_cluster<1><<<kClBlocks, kClThreads, csm, m->stream>>>(ra);   // one cluster
+            else k_rollout_cluster<2><<<kClBlocks, kClThreads, csm, m->stream>>>(ra);
+            if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(m->stream) != cudaSuccess)
+                return mfail(m, QP_ERR_CUDA, "fused rollout");
+            return QP_OK;
+        }
         const void *fn = MT == 1 ? (const void *)k_rollout_fused<1> : (const void *)k_rollout_fused<2>;
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm) != cudaSuccess)
             return mfail(m, QP_ERR_CUDA, "fused rollout set-up");
