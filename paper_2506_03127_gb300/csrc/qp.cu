@@ -623,7 +623,12 @@ struct Expander {
             const int dstride = P.nchunks * kLutEntries;
             if (eq && P.ndelta) {
                 double2 ep = make_double2(1.0, 0.0), en = make_double2(1.0, 0.0);
-                for (int j = 0; j < P.nchunks; ++j) {
+                if (P.nchunks > 0) {   // the first factors as they are (8 fewer FP64 operations of 62 per group)
+                    const int i0 = (int)key_byte(rep, 0);
+                    ep = tb.et[P.d_pos * dstride + i0];
+                    en = tb.et[P.d_neg * dstride + i0];
+                }
+                for (int j = 1; j < P.nchunks; ++j) {
                     const int idx = j * kLutEntries + (int)key_byte(rep, j);
                     ep = cmul(ep, tb.et[P.d_pos * dstride + idx]);
                     en = cmul(en, tb.et[P.d_neg * dstride + idx]);
@@ -1337,8 +1342,22 @@ __device__ __forceinline__ unsigned long long lb_word(unsigned epoch, unsigned s
 // the pending rho first, the kernel took 13.3 and 21.2 us (under ncu), and
 // 100 and 40 steps through qp_step 1.72 and 1.09 ms; now 1.16 and 0.50 ms,
 // with the tile kernel's empty launch gone (step_kind).
+//
+// The host knows the counts of an unfiltered propagation (step_kind) and
+// passes them (a.tn != 0): then no block reads the device state before its
+// paths, the history tables of the step's window length are staged before
+// the previous kernel has ended, and one block publishes the step at once,
+// without the arrivals: what is left is one trip for the paths, the
+// children and the stores.  (Reading the state, then the region sizes, and
+// publishing behind the last arrival: 9 us per step at memory 5 FP64 and 8
+// c64.)  Replayed graphs, the first step and steps launched ahead of the
+// tile kernel read the state.
+struct RegArgs {
+    long long tn, ngroups;   // 0: read from the device
+    int gs;
+};
 template <int M, bool C64>
-__global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(Params P, int lut_smem) {
+__global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(Params P, int lut_smem, RegArgs a) {
     using X = Expander<M, C64>;
     using AmpT = typename X::AmpT;
     constexpr int MM = M * M, NT = kRegThreads, NW = kRegThreads / 32;
@@ -1350,51 +1369,88 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     __shared__ float4 s_wf[C64 ? MM * MM : 1];
     __shared__ float4 s_rt[NW][MM];
     pdl_trigger();
-    for (int i = threadIdx.x; i < MM * MM; i += NT) {
-        if constexpr (C64) s_wf[i] = P.wtabf[i];
-        else s_w[i] = P.wtab[i];
+    const bool known = a.tn != 0;
+    const long long G = P.region_cap;
+    unsigned long long t = 0, n_in = 0;
+    int gs = a.gs;   // members of a group; 0: not a regular step
+    long long ngroups = a.ngroups, gpr = 0;   // groups, groups per region
+    if (known) {
+        t = (unsigned long long)a.tn - 1;
+        gpr = ngroups / MM;
+        n_in = (unsigned long long)ngroups * (unsigned)gs;
+    } else {
+        pdl_wait();
+        // the state and both buffers' region sizes in one trip
+        if ((int)threadIdx.x < 2 * MM) s_rn[threadIdx.x] = __ldcg(P.reg_n + threadIdx.x);
+        if (threadIdx.x == 32) {
+            s_err = __ldcg(&st->err);
+            s_t = __ldcg(&st->t);
+            s_pend = __ldcg(&st->rho_pending);
+            s_pnblk = __ldcg(&st->rho_nblk);
+        }
+        __syncthreads();
+        if (s_err) return;
+        t = s_t;
     }
-    pdl_wait();
-    // the state and both buffers' region sizes in one trip
-    if ((int)threadIdx.x < 2 * MM) s_rn[threadIdx.x] = __ldcg(P.reg_n + threadIdx.x);
-    if (threadIdx.x == 32) {
-        s_err = __ldcg(&st->err);
-        s_t = __ldcg(&st->t);
-        s_pend = __ldcg(&st->rho_pending);
-        s_pnblk = __ldcg(&st->rho_nblk);
-    }
-    __syncthreads();
-    if (s_err) return;
-    const unsigned long long t = s_t, tn = t + 1;
+    const unsigned long long tn = t + 1;
     const int in = (int)(t & 1), outp = (int)(tn & 1), cs = (int)(tn % 3);
     const bool merge = tn >= (unsigned long long)P.dkmax;
-    const long long G = P.region_cap;
-    // groups before region r (gs members each)
-    unsigned long long n_in = 0;
+    if (!known) {
 #pragma unroll
-    for (int r = 0; r < MM; ++r) n_in += s_rn[in * MM + r];
-    int gs = 0;   // members of a group; 0: not a regular step
-    if (n_in > 0) {
-        if (!merge) gs = P.reg_fill ? 1 : 0;
-        else if (P.reg_merge && n_in == P.full_n) gs = MM;
-        else if (P.reg_merge && tn == (unsigned long long)P.dkmax && n_in == P.full_n / MM * (unsigned long long)P.nnz0) gs = P.nnz0;
+        for (int r = 0; r < MM; ++r) n_in += s_rn[in * MM + r];
+        gs = 0;
+        if (n_in > 0) {
+            if (!merge) gs = P.reg_fill ? 1 : 0;
+            else if (P.reg_merge && n_in == P.full_n) gs = MM;
+            else if (P.reg_merge && tn == (unsigned long long)P.dkmax && n_in == P.full_n / MM * (unsigned long long)P.nnz0) gs = P.nnz0;
+        }
+        if (gs == 0) {   // the tile kernel takes it
+            if (blockIdx.x == 0 && threadIdx.x == 0) st->reg_done = 0;
+            return;
+        }
+        // every region holds as many groups, except at t = 0 (the nonzero
+        // elements of rho(0), one path each)
+        const unsigned long long nr0 = n_in / MM;
+        gpr = (long long)nr0;
+        if (gs == MM) gpr = (long long)(nr0 / MM);
+        else if (gs > 1) gpr = (long long)((nr0 >> 32) == 0 ? (unsigned)nr0 / (unsigned)gs : nr0 / (unsigned)gs);
+        ngroups = t == 0 ? (long long)n_in / gs : gpr * MM;
     }
-    if (gs == 0) {   // the tile kernel takes it
-        if (blockIdx.x == 0 && threadIdx.x == 0) st->reg_done = 0;
-        return;
-    }
-    // every region holds as many groups, except at t = 0 (the nonzero
-    // elements of rho(0), one path each)
-    const unsigned long long nr0 = n_in / MM;
-    long long gpr = (long long)nr0;   // groups per region
-    if (gs == MM) gpr = (long long)(nr0 / MM);
-    else if (gs > 1) gpr = (long long)((nr0 >> 32) == 0 ? (unsigned)nr0 / (unsigned)gs : nr0 / (unsigned)gs);
-    const long long ngroups = t == 0 ? (long long)n_in / gs : gpr * MM;
     const long long nchunk = (ngroups + 31) / 32;
     const bool spare = nchunk < (long long)gridDim.x;
     const unsigned active = spare ? (unsigned)nchunk : gridDim.x;   // blocks with groups
     const unsigned arrivals = active + (spare ? 1u : 0u);
     if (blockIdx.x >= arrivals) return;
+    // the step's record and the new state (one thread)
+    auto publish = [&]() {
+        st->rho_nblk = active;
+        st->rho_pending = tn;
+        StepCounts c;
+        c.groups = (unsigned long long)(merge ? ngroups : (long long)n_in);
+        c.n_out = (unsigned long long)ngroups * MM;
+        st->cnt_out[cs] = c.n_out;
+        st->cnt_groups[cs] = (unsigned long long)ngroups;
+        publish_step(P, st, tn, MM, c);
+    };
+    // counts known: the spare block, or the last one, publishes the step and
+    // leaves the region sizes; it alone reads the state
+    const bool publisher = known && blockIdx.x == arrivals - 1;
+    auto publish_known = [&]() -> bool {   // false: an earlier error
+        if (threadIdx.x == 32) {
+            s_err = __ldcg(&st->err);
+            s_pend = __ldcg(&st->rho_pending);
+            s_pnblk = __ldcg(&st->rho_nblk);
+        }
+        __syncthreads();
+        if (s_err) return false;
+        if (ngroups > G) {   // the outputs would not fit their regions
+            if (threadIdx.x == 0) raise_err(st, kErrPaths);
+            return true;
+        }
+        if ((int)threadIdx.x < MM) P.reg_n[outp * MM + threadIdx.x] = (unsigned long long)ngroups;
+        if (threadIdx.x == 0) publish();
+        return true;
+    };
     // the last block to arrive publishes the step, for which it needs the
     // step's counters only; every block then writes its partial of rho, which
     // the next step's kernel (or a read-time finalisation) sums once this
@@ -1402,23 +1458,18 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     // (ordered before it by the barrier) and acquires the others' in the last
     // block.
     auto arrive = [&]() {
+        if (known) return;
         __syncthreads();
         if (threadIdx.x == 0 && atom_add_acq_rel_gpu(P.fin_count, 1u) == arrivals - 1) {
-            if (__ldcg(&st->err)) {   // a failed step is not published
-                *P.fin_count = 0;
-            } else {
-                st->rho_nblk = active;
-                st->rho_pending = tn;
-                StepCounts c;
-                c.groups = (unsigned long long)(merge ? ngroups : (long long)n_in);
-                c.n_out = (unsigned long long)ngroups * MM;
-                st->cnt_out[cs] = c.n_out;
-                st->cnt_groups[cs] = (unsigned long long)ngroups;
-                publish_step(P, st, tn, MM, c);
-            }
+            if (__ldcg(&st->err)) *P.fin_count = 0;   // a failed step is not published
+            else publish();
         }
     };
     if (blockIdx.x == active) {   // the spare block: the previous step's rho
+        if (known) {
+            pdl_wait();
+            if (!publish_known()) return;
+        }
         arrive();
         if (s_pend) phase_finalize_stream<C64>(P, s_pend, (int)s_pnblk, MM);
         return;
@@ -1434,8 +1485,14 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     Tab tab = tab_global(P, n_act, 0);
     const long long step_chunks = (long long)active * NW;
     const long long chunk0 = (long long)(threadIdx.x >> 5) * active + blockIdx.x;
-    // the history tables pay for their copy once a warp takes a few groups
-    if (lut_smem && P.ndelta && nchunk > 2 * step_chunks) {
+    for (int i = threadIdx.x; i < MM * MM; i += NT) {
+        if constexpr (C64) s_wf[i] = P.wtabf[i];
+        else s_w[i] = P.wtab[i];
+    }
+    // the history tables pay for their copy where it overlaps the previous
+    // kernel, or once a warp takes a few groups
+    const bool staged = lut_smem && P.ndelta && (known || nchunk > 2 * step_chunks);
+    if (staged) {
         const int n = P.nchunks * kLutEntries;
         if constexpr (C64) {
             float2 *hi = reinterpret_cast<float2 *>(s_dyn), *lo = hi + n;
@@ -1451,9 +1508,14 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
             tab.et = et;
         }
         cp_async_wait_all();
-        __syncthreads();
     }
-    if (blockIdx.x == 0) {
+    __syncthreads();
+    unsigned err = 0;
+    if (known) {
+        pdl_wait();
+        if (publisher && !publish_known()) return;
+        err = __ldcg(&st->err);   // (checked behind the first paths' loads)
+    } else if (blockIdx.x == 0) {
         if ((int)threadIdx.x < MM) P.reg_n[outp * MM + threadIdx.x] = (unsigned long long)ngroups;
         if (threadIdx.x == 0) st->reg_done = tn + 1;
     }
@@ -1553,7 +1615,7 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
         }
     };
     if (ngroups > G) {   // the outputs would not fit their regions
-        if (threadIdx.x == 0) raise_err(st, kErrPaths);
+        if (threadIdx.x == 0 && !known) raise_err(st, kErrPaths);
     } else {
         // one group per thread at a time: three blocks of eight warps per SM
         // keep more bytes in flight than two groups per thread at two blocks
@@ -1562,6 +1624,7 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
             if (g < ngroups) {
                 Members m0;
                 load(g, m0);
+                if (err) break;   // (known counts: an earlier step failed)
                 group(g, m0);
             }
         }
@@ -1579,6 +1642,7 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
         if ((nchunk - 1) % active == blockIdx.x) mg -= nchunk * 32 - ngroups;
         scount_of(P, tn)[blockIdx.x] = mg * MM;
     }
+    if (err) return;
     if (!spare && blockIdx.x == gridDim.x - 1) {   // no spare block: the previous step's rho
         __syncthreads();
         if (s_pend) phase_finalize_stream<C64>(P, s_pend, (int)s_pnblk, MM);
@@ -1744,7 +1808,7 @@ __device__ __forceinline__ unsigned long long ld_relaxed_gpu(const unsigned long
 // regular kernel was launched for the same step and may have taken it).
 constexpr int kFlagLutSmem = 1, kFlagAfterRegular = 2;
 template <int M, bool C64, int NX, int S, bool BATCH>
-__device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
+__device__ __forceinline__ void stream_step_body(const Params &P, int flags, unsigned long long tn_host) {
     const bool lut_smem = (flags & kFlagLutSmem) != 0;
     using X = Expander<M, C64>;
     using Lay = StreamLayout<M, C64, NX, S>;
@@ -1760,12 +1824,15 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
     constexpr bool kTileAccS = !BATCH && M * M >= 9 && C64;   // per-warp tile sums of rho (see the accumulators)
     DevState *st = P.st;
     // Before the previous step's kernel is waited for: the propagator table
-    // and, on the chance that the window is full, its history tables (asynchronous
-    // copies, waited for before the first pass A)
+    // and the history tables of the step's window length, or on the chance that
+    // the window is full (asynchronous copies, waited for before the first pass A)
     __shared__ double2 s_w[C64 || BATCH ? 1 : MM * MM];   // FP64 weights (FP64 path only)
     __shared__ float4 s_wf[BATCH ? 1 : MM * MM];
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    Tab tab = tab_global(P, P.dkmax, 0);
+    // (tn_host: the step index where the host launches the step itself, 0 in
+    // a replayed graph)
+    const int n_ahead = tn_host ? (int)min(tn_host, (unsigned long long)P.dkmax) : P.dkmax;
+    Tab tab = tab_global(P, n_ahead, 0);
     // (rows are whole multiples of kLutEntries entries, so every copy is
     // 16-byte aligned)
     auto stage_tables = [&](const Tab &from) {
@@ -1794,7 +1861,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
     }
     // (device state read through L2: the persistent batch kernel runs
     // several steps in one launch)
-    const unsigned long long t = __ldcg(&st->t), tn = t + 1;
+    const unsigned long long t = tn_host ? tn_host - 1 : __ldcg(&st->t), tn = t + 1;
     // an earlier error, or launched behind the regular kernel, which just took
     // this step (its new t + 1)
     if (__ldcg(&st->err) || ((flags & kFlagAfterRegular) && __ldcg(&st->reg_done) == tn)) {
@@ -1860,7 +1927,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
     // thread's copies follow its own earlier ones; batches read their
     // instance's tables from global memory per tile)
     if constexpr (!BATCH)
-        if (n_act != P.dkmax) {
+        if (n_act != n_ahead) {
             const Tab now = tab_global(P, n_act, 0);
             if (lut_smem && P.ndelta) {
                 cp_async_wait_all();
@@ -2910,9 +2977,9 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags) {
 
 template <int M, bool C64, int NX, int S>
 __global__ void __launch_bounds__(kStreamThreads, (M == 2 || (M == 3 && C64)) ? 2 : 1)
-    k_stream_step(Params P, int flags) {
+    k_stream_step(Params P, int flags, long long tn) {
     pdl_trigger();
-    stream_step_body<M, C64, NX, S, false>(P, flags);
+    stream_step_body<M, C64, NX, S, false>(P, flags, (unsigned long long)tn);
 }
 
 // Batched stream engine: nsteps steps of all instances, separated by
@@ -2925,7 +2992,7 @@ template <int M, bool C64, int S>
 __global__ void __launch_bounds__(kStreamThreads, (M == 2 || (M == 3 && C64)) ? 2 : 1)
     k_stream_batch(Params P, int nsteps) {
     for (int s = 0; s < nsteps; ++s) {
-        stream_step_body<M, C64, 1, S, true>(P, 0);
+        stream_step_body<M, C64, 1, S, true>(P, 0, 0ull);
         if (s + 1 < nsteps && grid_barrier(P.st)) break;
     }
 }
@@ -3889,7 +3956,7 @@ cudaError_t stream_residency(qp_ctx *c, const void *fn, size_t sm, size_t sm_mos
 // Grid of the stream kernel: every block resident (tiles are taken by
 // ticket, so blocks beyond the co-resident count would only start after a
 // first wave), at most bps_exp per SM and kMaxExpandBlocks in all.
-cudaError_t launch_stream_tile(qp_ctx *c, bool after_regular, bool dep) {
+cudaError_t launch_stream_tile(qp_ctx *c, bool after_regular, bool dep, int64_t tn) {
     const qp::StreamKernel k = stream_kernel(c);
     const size_t lutb = stream_lut_bytes(c, c->cfg.precision == QP_C64);
     const size_t sm = k.bytes + lutb;
@@ -3897,7 +3964,8 @@ cudaError_t launch_stream_tile(qp_ctx *c, bool after_regular, bool dep) {
     if (e != cudaSuccess) return e;
     const int g = std::min(c->nsm * std::min(c->bps_exp, c->scache_res), kMaxExpandBlocks);
     int flags = (lutb ? kFlagLutSmem : 0) | (after_regular ? kFlagAfterRegular : 0);
-    void *args[] = {(void *)&c->P, (void *)&flags};
+    long long tn_host = after_regular ? 0 : (long long)tn;
+    void *args[] = {(void *)&c->P, (void *)&flags, (void *)&tn_host};
     return launch_pdl(k.fn, g, kStreamThreads, sm, c->stream, args, dep);
 }
 
@@ -3926,7 +3994,7 @@ cudaError_t launch_stream_batch(qp_ctx *c, int nsteps, bool coop) {
 // The regular stream kernel (no filter): every block resident, at most
 // kMaxExpandBlocks (block partials).
 template <int M, bool C64>
-cudaError_t launch_stream_regular(qp_ctx *c, bool dep) {
+cudaError_t launch_stream_regular(qp_ctx *c, bool dep, RegArgs ra) {
     const void *fn = (const void *)k_stream_regular<M, C64>;
     const size_t lutb = stream_lut_bytes(c, C64);
     if (c->rcache_fn != fn || c->rcache_smem != lutb) {
@@ -3940,9 +4008,10 @@ cudaError_t launch_stream_regular(qp_ctx *c, bool dep) {
         c->rcache_smem = lutb;
         c->rcache_res = nb;
     }
-    const int g = std::min(c->nsm * c->rcache_res, kMaxExpandBlocks);
+    int g = std::min(c->nsm * c->rcache_res, kMaxExpandBlocks);
+    if (ra.tn) g = (int)std::min<long long>(g, (ra.ngroups + 31) / 32 + 1);   // no block without work
     int lut_smem = lutb ? 1 : 0;
-    void *args[] = {(void *)&c->P, (void *)&lut_smem};
+    void *args[] = {(void *)&c->P, (void *)&lut_smem, (void *)&ra};
     return launch_pdl(fn, g, kRegThreads, lutb, c->stream, args, dep);
 }
 
@@ -3964,16 +4033,37 @@ StepKind step_kind(const qp_ctx *c, int64_t tn) {
     return tn < (int64_t)P.dkmax || P.reg_merge ? kStepRegular : kStepTile;
 }
 
+// The groups of regular step tn of a propagation whose counts the host knows
+// (tn = 0: not known, as in a captured graph).  At t = 0 the regions are
+// uneven, and beyond 2^40 paths the buffers end: read from the device.
+RegArgs known_counts(const qp_ctx *c, int64_t tn) {
+    RegArgs a{0, 0, 0};
+    if (tn < 2) return a;
+    const Params &P = c->P;
+    const int MM = c->cfg.M * c->cfg.M, dk = c->cfg.dkmax;
+    // M^2 per point after the first; the first merge drops the first point
+    const int points = (int)std::min<int64_t>(tn, dk) - 1;
+    long long n = tn < dk ? P.nnz0 : 1;
+    for (int i = 0; i < points; ++i) {
+        if (n > (1ll << 40) / MM) return a;
+        n *= MM;
+    }
+    a.tn = tn;
+    a.ngroups = n;
+    a.gs = tn < dk ? 1 : tn == dk ? P.nnz0 : MM;
+    return a;
+}
+
 // One step of the stream engine (regular kernel: events 0 -> 1, tile kernel:
 // events 2 -> 3).
 template <int M, typename Amp>
-cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind) {
+cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind, int64_t tn) {
     constexpr bool C64 = sizeof(Amp) == sizeof(float2);
     const bool after_regular = kind == kStepBoth && c->P.reg_fill && M < 4;
     if (ev) cudaEventRecord(ev[0], c->stream);
     if constexpr (M < 4) {
         if (kind == kStepRegular || after_regular) {
-            cudaError_t e = launch_stream_regular<M, C64>(c, ev == nullptr);
+            cudaError_t e = launch_stream_regular<M, C64>(c, ev == nullptr, kind == kStepRegular ? known_counts(c, tn) : RegArgs{0, 0, 0});
             if (e != cudaSuccess) return e;
         }
     }
@@ -3983,7 +4073,7 @@ cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind) {
     }
     cudaError_t e = cudaSuccess;
     if (c->P.n_inst > 1) e = launch_stream_batch(c, 1, false);
-    else if (kind != kStepRegular) e = launch_stream_tile(c, after_regular, ev == nullptr);
+    else if (kind != kStepRegular) e = launch_stream_tile(c, after_regular, ev == nullptr, tn);
     if (e != cudaSuccess) return e;
     if (ev) {
         cudaEventRecord(ev[3], c->stream);
@@ -4027,7 +4117,8 @@ cudaError_t launch_post_t(qp_ctx *c, cudaEvent_t *ev) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev = nullptr, StepKind kind = kStepBoth) {
+// tn: the step where the host launches it, 0 in a graph that is replayed
+cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev, StepKind kind, int64_t tn) {
     const bool c64 = c->cfg.precision == QP_C64;
     if (c->P.post) {
         switch (c->cfg.M) {
@@ -4038,9 +4129,9 @@ cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev = nullptr, StepKind kind = kS
     }
     if (c->use_stream) {
         switch (c->cfg.M) {
-            case 2: return c64 ? launch_stream_t<2, float2>(c, ev, kind) : launch_stream_t<2, double2>(c, ev, kind);
-            case 3: return c64 ? launch_stream_t<3, float2>(c, ev, kind) : launch_stream_t<3, double2>(c, ev, kind);
-            default: return c64 ? launch_stream_t<4, float2>(c, ev, kind) : launch_stream_t<4, double2>(c, ev, kind);
+            case 2: return c64 ? launch_stream_t<2, float2>(c, ev, kind, tn) : launch_stream_t<2, double2>(c, ev, kind, tn);
+            case 3: return c64 ? launch_stream_t<3, float2>(c, ev, kind, tn) : launch_stream_t<3, double2>(c, ev, kind, tn);
+            default: return c64 ? launch_stream_t<4, float2>(c, ev, kind, tn) : launch_stream_t<4, double2>(c, ev, kind, tn);
         }
     }
     switch (c->cfg.M) {
@@ -4656,7 +4747,7 @@ static qp_status capture_graph(qp_ctx *c, int steps, StepKind kind, cudaGraphExe
     cudaGraph_t g;
     QP_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = cudaSuccess;
-    for (int s = 0; s < steps && le == cudaSuccess; ++s) le = launch_step(c, nullptr, kind);
+    for (int s = 0; s < steps && le == cudaSuccess; ++s) le = launch_step(c, nullptr, kind, 0);
     cudaError_t ce = cudaStreamEndCapture(c->stream, &g);
     if (le != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(le));
     if (ce != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(ce));
@@ -4697,7 +4788,7 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
     for (int s = 0; s < nsteps;) {
         const StepKind kind = step_kind(c, t0 + s + 1);
         if (!graphs) {
-            const cudaError_t e = launch_step(c, nullptr, kind);
+            const cudaError_t e = launch_step(c, nullptr, kind, t0 + s + 1);
             if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
             ++s;
             continue;
@@ -4962,7 +5053,7 @@ qp_status qp_profile_steps(qp_ctx *c, int nsteps, double *kernel_ms, int nk) {
     qp_status st = QP_OK;
     for (int s = 0; s < nsteps && st == QP_OK; ++s) {
         k_delay<<<1, 1, 0, c->stream>>>(50000ull);
-        cudaError_t e = launch_step(c, ev);
+        cudaError_t e = launch_step(c, ev, step_kind(c, c->host_t + 1), c->host_t + 1);
         ++c->host_t;
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[kStepKernels]);
         if (e != cudaSuccess) {
