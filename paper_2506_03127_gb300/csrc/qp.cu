@@ -361,51 +361,85 @@ __device__ __forceinline__ void phase_insert(const Params &P, unsigned long long
     DevState *st = P.st;
     const unsigned long long *keys = P.keys[t & 1];
     const Amp *amps = static_cast<const Amp *>(P.amps[t & 1]);
-    const unsigned long long stride = (unsigned long long)gridDim.x * NT;
-    for (unsigned long long base = blockIdx.x * (unsigned long long)NT; base < n; base += stride) {
-        const unsigned long long i = base + threadIdx.x;
-        bool claimed = false, found = false;
-        unsigned long long h = 0;
-        if (i < n) {
-            const unsigned long long key = __ldcg(keys + i);
-            const double2 a = load_amp(amps, i);
-            const unsigned long long mk = key & P.pmask;
-            h = table_index(P, mk);
-            for (int probe = 0; probe < kMaxProbe; ++probe) {
-                const unsigned long long cur = *(volatile unsigned long long *)&P.slots[h].mk;
-                if (cur == mk) { found = true; break; }
-                if (cur == kEmpty) {
-                    const unsigned long long prev = atomicCAS(&P.slots[h].mk, kEmpty, mk);
-                    if (prev == kEmpty) { claimed = found = true; break; }
-                    if (prev == mk) { found = true; break; }
+    // two paths per thread in flight: the pass is a chain of table latencies
+    // (key, slot, claim), one path at a time took 8.8 us for 2e5 paths
+    constexpr int U = 2;
+    const unsigned long long stride = (unsigned long long)gridDim.x * NT * U;
+    for (unsigned long long base = blockIdx.x * (unsigned long long)(NT * U); base < n; base += stride) {
+        unsigned long long key[U], h[U], mk[U], cur[U];
+        double2 a[U];
+        unsigned claimed = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned long long i = base + u * NT + threadIdx.x;
+            key[u] = 0;
+            a[u] = make_double2(0.0, 0.0);
+            if (i < n) {
+                key[u] = __ldcg(keys + i);
+                a[u] = load_amp(amps, i);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            mk[u] = key[u] & P.pmask;
+            h[u] = table_index(P, mk[u]);
+            cur[u] = mk[u];
+            if (base + u * NT + threadIdx.x < n) cur[u] = *(volatile unsigned long long *)&P.slots[h[u]].mk;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (cur[u] == kEmpty) {
+                cur[u] = atomicCAS(&P.slots[h[u]].mk, kEmpty, mk[u]);
+                if (cur[u] == kEmpty) {
+                    claimed |= 1u << u;
+                    cur[u] = mk[u];
                 }
-                h = (h + 1) & P.tcap_mask;
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned long long i = base + u * NT + threadIdx.x;
+            if (i >= n) continue;
+            bool found = cur[u] == mk[u];
+            for (int probe = 1; probe < kMaxProbe && !found; ++probe) {   // collisions (hashed tables)
+                h[u] = (h[u] + 1) & P.tcap_mask;
+                unsigned long long c = *(volatile unsigned long long *)&P.slots[h[u]].mk;
+                if (c == kEmpty) {
+                    c = atomicCAS(&P.slots[h[u]].mk, kEmpty, mk[u]);
+                    if (c == kEmpty) {
+                        claimed |= 1u << u;
+                        c = mk[u];
+                    }
+                }
+                found = c == mk[u];
             }
             if (found) {
-                atomicAdd(&P.slots[h].sre, a.x);
-                atomicAdd(&P.slots[h].sim, a.y);
+                atomicAdd(&P.slots[h[u]].sre, a[u].x);
+                atomicAdd(&P.slots[h[u]].sim, a[u].y);
                 // weight |a|^2 as ordered bits: FP32 on the C64 path (as in
                 // the stream engine), FP64 otherwise
                 unsigned long long wb;
                 if constexpr (sizeof(Amp) == sizeof(float2)) {
-                    const float ax = (float)a.x, ay = (float)a.y;   // exact: a holds FP32 values
+                    const float ax = (float)a[u].x, ay = (float)a[u].y;   // exact: a holds FP32 values
                     wb = __float_as_uint(ax * ax + ay * ay);
                 } else {
-                    wb = (unsigned long long)__double_as_longlong(a.x * a.x + a.y * a.y);
+                    wb = (unsigned long long)__double_as_longlong(a[u].x * a[u].x + a[u].y * a[u].y);
                 }
-                atomicMax(&P.slots[h].wmax, wb);
-                P.slot_of[i] = (unsigned int)h;
+                atomicMax(&P.slots[h[u]].wmax, wb);
+                P.slot_of[i] = (unsigned int)h[u];
             } else {
                 P.slot_of[i] = kNoSlot;
                 raise_err(st, kErrProbe);
             }
         }
-        const Append ap = block_append<NT>(claimed ? 1u : 0u, cnt_groups);
-        if (claimed) {
-            const unsigned long long g = ap.base + ap.excl;
-            if (g < (unsigned long long)P.max_groups) P.groups[g] = (unsigned int)h;
-            else raise_err(st, kErrGroups);
-        }
+        const Append ap = block_append<NT>(__popc(claimed), cnt_groups);
+        unsigned long long g = ap.base + ap.excl;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (claimed & (1u << u)) {
+                if (g < (unsigned long long)P.max_groups) P.groups[g] = (unsigned int)h[u];
+                else raise_err(st, kErrGroups);
+                ++g;
+            }
     }
 }
 
@@ -670,52 +704,98 @@ struct Expander {
     }
 };
 
+// Sums of V values over the warp by halving (a power of two V <= 32): in round
+// o a lane keeps one half of its values and hands the other half to lane ^ o,
+// so the rounds cost V/2 + V/4 + ... additions instead of 5 V (FP64: the
+// pipe takes a warp's addition 16 cycles, and 24 warps per SM reduce their
+// accumulators at the end of a step kernel).  On return v[0] is the warp's
+// sum of value rs_index<V>(lane).  The result does not depend on the lane.
+template <int V>
+__device__ __forceinline__ int rs_index() {
+    int idx = 0;
+#pragma unroll
+    for (int n = V / 2, o = 16; n >= 1; n >>= 1, o >>= 1)
+        if (lane_id() & o) idx += n;
+    return idx;
+}
+template <int V>
+__device__ __forceinline__ void warp_reduce_scatter(double (&v)[V]) {
+    const unsigned lane = lane_id();
+    int o = 16;
+#pragma unroll
+    for (int n = V / 2; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0u;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double give = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+}
+// the same for FP32 pairs (s + e, the rounding error of every addition kept
+// in e: TwoSum)
+template <int V>
+__device__ __forceinline__ void warp_reduce_scatter(float (&s)[V], float (&e)[V]) {
+    const unsigned lane = lane_id();
+    int o = 16;
+#pragma unroll
+    for (int n = V / 2; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0u;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float gs = up ? s[i] : s[i + n], ge = up ? e[i] : e[i + n];
+            float ks = up ? s[i + n] : s[i], ke = up ? e[i + n] : e[i];
+            const float b = __shfl_xor_sync(0xffffffffu, gs, o), f = __shfl_xor_sync(0xffffffffu, ge, o);
+            two_sum_acc(ks, ke, b);
+            s[i] = ks;
+            e[i] = ke + f;
+        }
+    }
+    for (; o >= 1; o >>= 1) {
+        const float b = __shfl_xor_sync(0xffffffffu, s[0], o), f = __shfl_xor_sync(0xffffffffu, e[0], o);
+        two_sum_acc(s[0], e[0], b);
+        e[0] += f;
+    }
+}
+
 // Block partial of the threads' rho accumulators into out[0 .. MM): per
 // component the thread's value is hi + lo.  C64 (FP32 sum and compensation):
-// each warp reduces with error-free additions (TwoSum, every rounding error
-// carried into the lo part) and widens to FP64 once, in lane 0, so that the
-// reduction stays off the FP64 pipe (1/64 of the FP32 rate on this part);
-// FP64 accumulators (lo unused) reduce with FP64 shuffles.  Warps are summed
-// in FP64, in warp order.  s_r: [NW][MM] scratch; every thread of the block
+// each warp reduces by halving with error-free additions (TwoSum, every
+// rounding error carried into the lo part) and widens to FP64 once per
+// component, so that the reduction stays off the FP64 pipe (1/64 of the FP32
+// rate on this part); FP64 accumulators (lo unused) by halving in FP64.  Warps
+// are summed in FP64, in warp order.  s_r: [NW][MM] scratch; every thread of the block
 // calls it.
 template <int MM, int NW, bool C64>
 __device__ __forceinline__ void block_rho_partial(const typename std::conditional<C64, float2, double2>::type *hi,
                                                   const float2 *lo, double2 (*s_r)[MM], double2 *out) {
-    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    constexpr int V = MM <= 4 ? 8 : 32;   // 2 M*M components, padded
+    const unsigned warp = threadIdx.x >> 5;
+    const int idx = rs_index<V>();
+    typename std::conditional<C64, float, double>::type sv[V], ev[C64 ? V : 1];
 #pragma unroll
-    for (int k = 0; k < MM; ++k) {
+    for (int k = 0; k < V; ++k) {
+        sv[k] = 0;
+        if (k < 2 * MM) sv[k] = (k & 1) ? hi[k >> 1].y : hi[k >> 1].x;
         if constexpr (C64) {
-            float sx = hi[k].x, ex = lo[k].x, sy = hi[k].y, ey = lo[k].y;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float bx = __shfl_down_sync(0xffffffffu, sx, o), fx = __shfl_down_sync(0xffffffffu, ex, o);
-                const float by = __shfl_down_sync(0xffffffffu, sy, o), fy = __shfl_down_sync(0xffffffffu, ey, o);
-                const float tx = sx + bx, vx = tx - sx;
-                ex += fx + ((sx - (tx - vx)) + (bx - vx));
-                sx = tx;
-                const float ty = sy + by, vy = ty - sy;
-                ey += fy + ((sy - (ty - vy)) + (by - vy));
-                sy = ty;
-            }
-            if (lane == 0) s_r[warp][k] = make_double2(f2d_exact(sx) + f2d_exact(ex), f2d_exact(sy) + f2d_exact(ey));
-        } else {
-            double x = hi[k].x, y = hi[k].y;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                x += __shfl_down_sync(0xffffffffu, x, o);
-                y += __shfl_down_sync(0xffffffffu, y, o);
-            }
-            if (lane == 0) s_r[warp][k] = make_double2(x, y);
+            ev[k] = 0;
+            if (k < 2 * MM) ev[k] = (k & 1) ? lo[k >> 1].y : lo[k >> 1].x;
         }
     }
+    if constexpr (C64) warp_reduce_scatter<V>(sv, ev);
+    else warp_reduce_scatter<V>(sv);
+    if (idx < 2 * MM && (lane_id() & (32 / V - 1)) == 0u) {
+        double v;
+        if constexpr (C64) v = f2d_exact(sv[0]) + f2d_exact(ev[0]);
+        else v = sv[0];
+        reinterpret_cast<double *>(&s_r[warp][0])[idx] = v;
+    }
     __syncthreads();
-    if (threadIdx.x < MM) {
-        double x = 0.0, y = 0.0;
-        for (int w = 0; w < NW; ++w) {
-            x += s_r[w][threadIdx.x].x;
-            y += s_r[w][threadIdx.x].y;
-        }
-        out[threadIdx.x] = make_double2(x, y);
+    if (threadIdx.x < 2 * MM) {
+        double x = 0.0;
+        for (int w = 0; w < NW; ++w) x += reinterpret_cast<const double *>(&s_r[w][0])[threadIdx.x];
+        reinterpret_cast<double *>(out)[threadIdx.x] = x;
     }
 }
 
@@ -963,61 +1043,6 @@ __device__ __forceinline__ double2 *rho_part_of(const Params &P, unsigned long l
     return P.rho_part + (size_t)(tn & 1) * kMaxExpandBlocks * P.n_inst * (MM + 1);
 }
 
-// Sums of V values over the warp by halving (a power of two V <= 32): in round
-// o a lane keeps one half of its values and hands the other half to lane ^ o,
-// so the rounds cost V/2 + V/4 + ... additions instead of 5 V (FP64: the
-// pipe takes a warp's addition 16 cycles, and 24 warps per SM reduce their
-// accumulators at the end of a step kernel).  On return v[0] is the warp's
-// sum of value rs_index<V>(lane).  The result does not depend on the lane.
-template <int V>
-__device__ __forceinline__ int rs_index() {
-    int idx = 0;
-#pragma unroll
-    for (int n = V / 2, o = 16; n >= 1; n >>= 1, o >>= 1)
-        if (lane_id() & o) idx += n;
-    return idx;
-}
-template <int V>
-__device__ __forceinline__ void warp_reduce_scatter(double (&v)[V]) {
-    const unsigned lane = lane_id();
-    int o = 16;
-#pragma unroll
-    for (int n = V / 2; n >= 1; n >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0u;
-#pragma unroll
-        for (int i = 0; i < n; ++i) {
-            const double give = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-        }
-    }
-    for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-}
-// the same for FP32 pairs (s + e, the rounding error of every addition kept
-// in e: TwoSum)
-template <int V>
-__device__ __forceinline__ void warp_reduce_scatter(float (&s)[V], float (&e)[V]) {
-    const unsigned lane = lane_id();
-    int o = 16;
-#pragma unroll
-    for (int n = V / 2; n >= 1; n >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0u;
-#pragma unroll
-        for (int i = 0; i < n; ++i) {
-            const float gs = up ? s[i] : s[i + n], ge = up ? e[i] : e[i + n];
-            float ks = up ? s[i + n] : s[i], ke = up ? e[i + n] : e[i];
-            const float b = __shfl_xor_sync(0xffffffffu, gs, o), f = __shfl_xor_sync(0xffffffffu, ge, o);
-            two_sum_acc(ks, ke, b);
-            s[i] = ks;
-            e[i] = ke + f;
-        }
-    }
-    for (; o >= 1; o >>= 1) {
-        const float b = __shfl_xor_sync(0xffffffffu, s[0], o), f = __shfl_xor_sync(0xffffffffu, e[0], o);
-        two_sum_acc(s[0], e[0], b);
-        e[0] += f;
-    }
-}
-
 // Stream engine: each block stores its partial of rho per end point, C64 as
 // an FP32 sum and the rounding error of every addition (the warps' sums by
 // halving, then the warps folded by one thread per component, all with
@@ -1188,6 +1213,44 @@ __global__ void k_rho_read_to(Params P, int MM, int finalize, double2 *dst, long
     }
 }
 
+// Blocks of the extension that have a group or path; the others return at
+// once and leave no partial.
+__device__ __forceinline__ int expand_blocks(int grid, unsigned long long n) {
+    const unsigned long long b = (n + kExpandThreads - 1) / kExpandThreads;
+    return b < (unsigned long long)grid ? max(1, (int)b) : grid;
+}
+
+// Single problems: rho(tn) and the survivor count from the nblk per-block
+// partials, by the block that calls it.  A thread adds every T-th element of
+// the contiguous partials, T a multiple of a row, so that it keeps to one
+// component and a warp reads whole lines; 16 loads in flight.
+template <int MM>
+__device__ __forceinline__ void finalize_single(const Params &P, unsigned long long tn, const double2 *part, int nblk) {
+    constexpr int N = 2 * (MM + 1), T = kExpandThreads / N * N, U = 16;
+    __shared__ double s_p[kExpandThreads];
+    const double *src = reinterpret_cast<const double *>(part);
+    double a = 0.0;
+    if ((int)threadIdx.x < T)
+        for (int i0 = (int)threadIdx.x; i0 < nblk * N; i0 += U * T) {
+            double v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[u] = i0 + u * T < nblk * N ? __ldcg(src + i0 + u * T) : 0.0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) a += v[u];
+        }
+    s_p[threadIdx.x] = a;
+    __syncthreads();
+    const size_t slot = (size_t)(tn % (unsigned long long)P.rho_hist);
+    if ((int)threadIdx.x < N) {
+        for (int u = 1; u < T / N; ++u) a += s_p[threadIdx.x + u * N];
+        if ((int)threadIdx.x < 2 * MM) reinterpret_cast<double *>(P.rho_ring + slot * MM)[threadIdx.x] = a;
+        else if ((int)threadIdx.x == 2 * MM) P.inst_kept[slot] = (long long)(a + 0.5);
+    }
+}
+
+// Extension of the step's groups or paths.  Single problems: the last block to
+// arrive also finalises and publishes the step (a kernel of its own for that
+// took 10 us of a 41 us step at 9e4 groups); batches leave it to k_finalize.
 template <int M, bool C64, bool BATCH>
 __global__ void __launch_bounds__(kExpandThreads) k_expand(Params P) {
     DevState *st = P.st;
@@ -1195,19 +1258,35 @@ __global__ void __launch_bounds__(kExpandThreads) k_expand(Params P) {
     const unsigned long long t = st->t, tn = t + 1;
     const bool merge = tn >= (unsigned long long)P.dkmax;
     const unsigned long long n = merge ? st->cnt_groups[tn % 3] : st->n_cur;
+    const int nact = expand_blocks((int)gridDim.x, n);
+    if ((int)blockIdx.x >= nact) return;
     phase_expand<M, C64, kExpandThreads, BATCH>(P, t, n, merge, &st->cnt_out[tn % 3], rho_part_of(P, tn, M * M));
+    if constexpr (!BATCH) {
+        __shared__ bool s_last;   // (phase_expand ends with a barrier)
+        if (threadIdx.x == 0) s_last = atom_add_acq_rel_gpu(P.fin_count, 1u) == (unsigned)nact - 1u;
+        __syncthreads();
+        if (!s_last) return;
+        if (__ldcg(&st->err)) {   // a failed step is not published
+            if (threadIdx.x == 0) *P.fin_count = 0;
+            return;
+        }
+        finalize_single<M * M>(P, tn, rho_part_of(P, tn, M * M), nact);
+        if (threadIdx.x == 0) publish_step(P, st, tn, M * M, step_counts(P, st, tn));
+    }
 }
 
 #if QP_UNIT == 0
-// Step finalisation of the multi-kernel path: block i finalises instance i;
+// Step finalisation of batches (multi-kernel path): block i finalises instance i;
 // the last block to finish publishes the step (counts, t, next counters).
 __global__ void __launch_bounds__(256) k_finalize(Params P, int MM, int nblk) {
     DevState *st = P.st;
     __shared__ bool s_last;
     if (st->err) return;
     const unsigned long long t = st->t, tn = t + 1;
+    const StepCounts sc = step_counts(P, st, tn);
+    const int nact = expand_blocks(nblk, sc.groups);
     for (int inst = blockIdx.x; inst < P.n_inst; inst += gridDim.x)
-        phase_finalize(P, tn, inst, rho_part_of(P, tn, MM), nblk, MM);
+        phase_finalize(P, tn, inst, rho_part_of(P, tn, MM), nact, MM);
     if (threadIdx.x == 0) {
         __threadfence();
         s_last = atomicAdd(P.fin_count, 1u) == gridDim.x - 1;
@@ -3912,7 +3991,7 @@ cudaError_t launch_step_t(qp_ctx *c, cudaEvent_t *ev) {
     else
         k_expand<M, C64, false><<<g_exp, kExpandThreads, 0, c->stream>>>(c->P);
     if (ev) cudaEventRecord(ev[3], c->stream);
-    k_finalize<<<std::max(1, std::min(c->P.n_inst, 1024)), 256, 0, c->stream>>>(c->P, M * M, g_exp);
+    if (c->P.n_inst > 1) k_finalize<<<std::min(c->P.n_inst, 1024), 256, 0, c->stream>>>(c->P, M * M, g_exp);
     if (ev) cudaEventRecord(ev[4], c->stream);
     return cudaGetLastError();
 }
@@ -5570,7 +5649,6 @@ extern "C" qp_status qp_step_noalloc(const qp_config *cfg, const double *eta_re,
         case 3: k_expand<3, false, false><<<g_exp, kExpandThreads, 0, stream>>>(P); break;
         default: k_expand<4, false, false><<<g_exp, kExpandThreads, 0, stream>>>(P); break;
     }
-    k_finalize<<<1, 256, 0, stream>>>(P, MM, g_exp);
     if (cudaGetLastError() != cudaSuccess) return QP_ERR_CUDA;
     if (cudaStreamSynchronize(stream) != cudaSuccess) return QP_ERR_CUDA;
     DevState s;
