@@ -2357,28 +2357,22 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             ngroups = (int)s_ng;
             __syncthreads();
         }
-        auto slot_of = [&](int sg, unsigned long long key) -> int {
-            if constexpr (NX > 1) {
-                const unsigned m = s_xm[sg];
-                return s_sb[sg] + __popc(m & ((1u << xval(key)) - 1u));
-            } else {
-                return sg;
-            }
-        };
         // groups of runs of at most kOwnRun members (all runs once the window
         // is full) have one owner thread each, which visits the group's
-        // members (the whole run, or for NX > 1 the sub-group's mask) twice
-        // in order: walk 1 adds them (C64: FP32 with the rounding error of
-        // every addition kept, TwoSum, rounded once; FP64: FP64) and takes
-        // their maximum weight, walk 2 elects the representative.  No atomics
-        // and no stores in the loops; the result does not depend on the
-        // tiling.  FP64 sub-groups (NX > 1) stay with the shared atomics
-        // below, one entry per thread, which keeps the FP64 pipe (1/64 of the
-        // FP32 rate) to one addition per member.
-        constexpr bool kOwners = NX == 1 || C64;
-        bool any_long = !kOwners && nseg > 0;
+        // members (the whole run, or for NX > 1 the sub-group's mask) in
+        // order: it adds them (C64: FP32 with the rounding error of every
+        // addition kept, TwoSum, rounded once; FP64: FP64) and takes their
+        // largest weight; only where another weight may lie within the tie
+        // window (compared as integers, the window being at most kNear units)
+        // a second walk elects the representative.  No atomics and no stores
+        // in the loops; the result does not depend on the tiling.  (FP64
+        // sub-groups went through shared FP64 atomics, one entry per thread:
+        // compare-and-swap loops that cost more of the FP64 pipe than the
+        // owners' predicated additions.)
+        constexpr WT kNear = C64 ? 40 : 20000;
+        bool any_long = false;
         cp_async_wait_all();   // staged history tables (first tile), published by the barrier below
-        if constexpr (kOwners) {
+        {
             const int nown = NX > 1 ? ngroups : nseg;
             for (int sl = threadIdx.x; sl < nown; sl += NT) {
                 int g = sl;
@@ -2399,7 +2393,10 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 sh.x = sh.y = 0;
                 se.x = se.y = 0;
                 WT wmx = 0;
-                auto add = [&](const AmpT &a) {
+                int imx = b0;
+                bool some = false, multi = false;
+                auto add = [&](int i) {
+                    const AmpT a = s_amp[i];
                     if constexpr (C64) {
                         two_sum_acc(sh.x, se.x, a.x);
                         two_sum_acc(sh.y, se.y, a.y);
@@ -2408,23 +2405,33 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                         sh.y += a.y;
                     }
                     const WT wb = weight_bits(a);
-                    wmx = wb > wmx ? wb : wmx;
+                    if (!some || wb > wmx) {
+                        multi = some && wb - wmx <= kNear;
+                        wmx = wb;
+                        imx = i;
+                    } else if (wmx - wb <= kNear) {
+                        multi = true;
+                    }
+                    some = true;
                 };
                 unsigned mm;   // the group's members by offset in the run
                 if constexpr (NX > 1) {
                     mm = s_xmask[g * NX + x];
 #pragma unroll 4
-                    for (unsigned m = mm; m; m &= m - 1u) add(s_amp[b0 + __ffs(m) - 1]);
+                    for (unsigned m = mm; m; m &= m - 1u) add(b0 + __ffs(m) - 1);
                 } else {
                     mm = n == 32 ? 0xffffffffu : (1u << n) - 1u;
 #pragma unroll 4
-                    for (int j = 0; j < n; ++j) add(s_amp[b0 + j]);
+                    for (int j = 0; j < n; ++j) add(b0 + j);
                 }
-                unsigned long long kmin = kEmpty;
-                for (unsigned m = mm; m; m &= m - 1u) {
-                    const int i = b0 + __ffs(m) - 1;
-                    const unsigned long long key = s_key[i];
-                    if (within_tie(weight_bits(s_amp[i]), wmx) && key < kmin) kmin = key;
+                unsigned long long kmin = s_key[imx];
+                if (multi) {
+                    kmin = kEmpty;
+                    for (unsigned m = mm; m; m &= m - 1u) {
+                        const int i = b0 + __ffs(m) - 1;
+                        const unsigned long long key = s_key[i];
+                        if (within_tie(weight_bits(s_amp[i]), wmx) && key < kmin) kmin = key;
+                    }
                 }
                 if constexpr (C64) store_own_sum(s_gS + sl, make_float2(sh.x + se.x, sh.y + se.y));
                 else s_gS[sl] = make_double2(sh.x, sh.y);
@@ -2611,89 +2618,6 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                     if (lane == 0 && kmin[x] != kEmpty) atomicMin(&s_grep[sl], kmin[x]);
                 }
                 __syncthreads();
-            }
-        }
-        // FP64 sub-groups in short runs: every member adds to its group with
-        // shared FP64 atomics (consecutive members of a thread in the same
-        // slot combined first), then, after a barrier, the members within
-        // the tie window compete for the representative
-        if (!kOwners && any_runs) {
-            auto short_run = [&](int g) -> bool {
-                const long long b1 = g + 1 < nseg ? (long long)s_seg[g + 1] : ahead;
-                return b1 - s_seg[g] <= kOwnRun;
-            };
-            const bool last_short = nseg > 0 && short_run(nseg - 1);
-            {
-                int sg = segbase, cur = -1;
-                bool shrt = sg >= 0 && short_run(sg);
-                double ax = 0.0, ay = 0.0;
-                WT wmx = 0;
-#pragma unroll
-                for (int u = 0; u < EPT; ++u) {
-                    const int i = threadIdx.x * ept + u;
-                    if (hmask & (1u << u)) shrt = short_run(++sg);
-                    if (u < ept && i < cnt && shrt) {
-                        const AmpT a = s_amp[i];
-                        const int sl = slot_of(sg, s_key[i]);
-                        const WT wb = weight_bits(a);
-                        if (sl != cur) {
-                            if (cur >= 0) {
-                                atomicAdd(&s_gS[cur].x, ax);
-                                atomicAdd(&s_gS[cur].y, ay);
-                                atomicMax(&s_wm[cur], wmx);
-                            }
-                            cur = sl;   // the slot's local sum starts at its first member
-                            ax = to_d(a.x);
-                            ay = to_d(a.y);
-                            wmx = wb;
-                        } else {
-                            ax += to_d(a.x);
-                            ay += to_d(a.y);
-                            wmx = wb > wmx ? wb : wmx;
-                        }
-                    }
-                }
-                if (cur >= 0) {
-                    atomicAdd(&s_gS[cur].x, ax);
-                    atomicAdd(&s_gS[cur].y, ay);
-                    atomicMax(&s_wm[cur], wmx);
-                }
-            }
-            // a short last run's members past the tile end are in the prefetch
-            const bool tail = warp == 0 && last_short && cnt + (int)lane < ahead;
-            if (tail) {
-                const AmpT a = s_amp[cnt + lane];
-                const int sl = slot_of(nseg - 1, s_key[cnt + lane]);
-                atomicAdd(&s_gS[sl].x, to_d(a.x));
-                atomicAdd(&s_gS[sl].y, to_d(a.y));
-                atomicMax(&s_wm[sl], weight_bits(a));
-            }
-            __syncthreads();
-            {
-                int sg = segbase, cur = -1;
-                bool shrt = sg >= 0 && short_run(sg);
-                unsigned long long kmin = kEmpty;
-#pragma unroll
-                for (int u = 0; u < EPT; ++u) {
-                    const int i = threadIdx.x * ept + u;
-                    if (hmask & (1u << u)) shrt = short_run(++sg);
-                    if (u < ept && i < cnt && shrt) {
-                        const unsigned long long key = s_key[i];
-                        const int sl = slot_of(sg, key);
-                        if (sl != cur) {
-                            if (cur >= 0 && kmin != kEmpty) atomicMin(&s_grep[cur], kmin);
-                            cur = sl;
-                            kmin = kEmpty;
-                        }
-                        if (within_tie(weight_bits(s_amp[i]), s_wm[sl]) && key < kmin) kmin = key;
-                    }
-                }
-                if (cur >= 0 && kmin != kEmpty) atomicMin(&s_grep[cur], kmin);
-            }
-            if (tail) {
-                const unsigned long long key = s_key[cnt + lane];
-                const int sl = slot_of(nseg - 1, key);
-                if (within_tie(weight_bits(s_amp[cnt + lane]), s_wm[sl])) atomicMin(&s_grep[sl], key);
             }
         }
         if (any_runs) __syncthreads();
