@@ -3522,6 +3522,44 @@ __global__ void k_set_count(DevState *st, unsigned long long n) { st->n_cur = n;
 
 // ---------------------------------------------------------------- set-up kernels
 
+// The state at t = 0 of every instance, from arguments passed by value (no
+// copies from host memory): n paths per instance, key, amplitude and region
+// each, rho(0), the counts and the record of step 0.
+struct InitArgs {
+    int n;
+    unsigned long long key[16];
+    double2 amp[16], rho[16];
+    int reg[16];   // newest point a M + b
+};
+template <typename Amp>
+__global__ void __launch_bounds__(256) k_set_state(Params P, int MM, InitArgs a) {
+    const int NI = P.n_inst, R = NI * MM;
+    for (int i = threadIdx.x; i < R; i += blockDim.x) {
+        P.rho_ring[i] = a.rho[i % MM];
+        if (P.stream) P.reg_n[i] = P.reg_n[R + i] = 0ull;
+    }
+    unsigned *words = reinterpret_cast<unsigned *>(P.st);
+    for (int i = threadIdx.x; i < (int)(sizeof(DevState) / 4); i += blockDim.x) words[i] = 0u;
+    for (int i = threadIdx.x; i < NI; i += blockDim.x) P.inst_kept[i] = a.n;
+    __syncthreads();
+    for (int e = threadIdx.x; e < NI * a.n; e += blockDim.x) {
+        const int inst = e / a.n, k = e - inst * a.n, r = inst * MM + a.reg[k];
+        const size_t o = P.stream ? (size_t)r * P.region_cap : (size_t)e;
+        P.keys[0][o] = a.key[k] | (P.stream || NI == 1 ? 0ull : (unsigned long long)inst << P.inst_shift);
+        Amp v;
+        v.x = (decltype(v.x))a.amp[k].x;
+        v.y = (decltype(v.y))a.amp[k].y;
+        static_cast<Amp *>(P.amps[0])[o] = v;
+        if (P.stream) P.reg_n[r] = 1ull;
+    }
+    if (threadIdx.x == 0) {
+        const long long n = (long long)NI * a.n;
+        P.st->n_cur = (unsigned long long)n;
+        *P.fin_count = 0u;
+        P.stats_ring[0] = StepRec{0, 0, 0, n, n};
+    }
+}
+
 __global__ void k_clear_table(Slot *slots, unsigned long long *repk, unsigned long long n) {
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -4654,27 +4692,20 @@ qp_status qp_set_rho0(qp_ctx *c, const double *re, const double *im) {
     if (!c->have_eta) return fail(c, QP_ERR_STATE, "qp_set_eta must come before qp_set_rho0");
     const int M = c->cfg.M, MM = M * M, NI = c->P.n_inst;
     const int bs = c->P.bs;
-    std::vector<unsigned long long> keys;
-    std::vector<double2> amps, rho((size_t)NI * MM);
+    InitArgs ia{};
     for (int a = 0; a < M; ++a)
         for (int b = 0; b < M; ++b) {
             const double x = re[a * M + b], y = im ? im[a * M + b] : 0.0;
             if (!std::isfinite(x) || !std::isfinite(y)) return fail(c, QP_ERR_ARG, "rho0 must be finite");
-            for (int i = 0; i < NI; ++i) rho[(size_t)i * MM + a * M + b] = make_double2(x, y);
+            ia.rho[a * M + b] = make_double2(x, y);
+            if (x == 0.0 && y == 0.0) continue;
+            ia.key[ia.n] = (unsigned long long)(a | (b << bs));
+            ia.amp[ia.n] = make_double2(x, y);
+            ia.reg[ia.n] = a * M + b;
+            ++ia.n;
         }
-    long long nnz = 0;
-    for (int i = 0; i < NI; ++i)
-        for (int a = 0; a < M; ++a)
-            for (int b = 0; b < M; ++b) {
-                const double2 v = rho[(size_t)i * MM + a * M + b];
-                if (v.x != 0.0 || v.y != 0.0) {
-                    const unsigned long long ib = NI > 1 ? ((unsigned long long)i << c->P.inst_shift) : 0ull;
-                    keys.push_back(ib | (unsigned long long)(a | (b << bs)));
-                    amps.push_back(v);
-                    if (i == 0) ++nnz;
-                }
-            }
-    if ((int64_t)keys.size() > c->cfg.max_paths) return fail(c, QP_ERR_CAPACITY, "rho0 exceeds max_paths");
+    const int64_t n = (int64_t)NI * ia.n;
+    if (n > c->cfg.max_paths) return fail(c, QP_ERR_CAPACITY, "rho0 exceeds max_paths");
     // engine of this propagation
     if (!c->P.post && c->cfg.engine == QP_ENGINE_STREAM && c->stream_nx == 0)
         return fail(c, QP_ERR_ARG, "the stream engine needs a mask whose P' is a prefix {0..k-1} plus at most one "
@@ -4683,58 +4714,29 @@ qp_status qp_set_rho0(qp_ctx *c, const double *re, const double *im) {
                     (c->cfg.engine == QP_ENGINE_STREAM || (c->cfg.engine == QP_ENGINE_AUTO && c->stream_nx > 0));
     if (c->use_stream && c->P.region_cap < 1) return fail(c, QP_ERR_CAPACITY, "max_paths < 16 M*M (stream engine)");
     c->P.stream = c->use_stream ? 1 : 0;
-    c->P.nnz0 = (int)nnz;
+    c->P.nnz0 = ia.n;
     c->reg_track = c->use_stream;
     c->graph_dirty = true;
-    const size_t n = keys.size();
-    const size_t ab = c->cfg.precision == QP_C64 ? sizeof(float2) : sizeof(double2);
-    if (c->sym) {   // point 0 on its half interval: its self factor in the stored amplitudes
-        for (size_t i = 0; i < n; ++i) {
-            const int a = (int)(keys[i] & ((1u << bs) - 1u)), b = (int)((keys[i] >> bs) & ((1u << bs) - 1u));
-            const double qa = c->q[a], qb = c->q[b];
+    if (c->sym)   // point 0 on its half interval: its self factor in the stored amplitudes
+        for (int i = 0; i < ia.n; ++i) {
+            const double qa = c->q[ia.reg[i] / M], qb = c->q[ia.reg[i] % M];
             const qp::cplx f = std::exp(-(qa - qb) * (c->eta00 * qa - std::conj(c->eta00) * qb)) *
-                               qp::cplx(amps[i].x, amps[i].y);
-            amps[i] = make_double2(f.real(), f.imag());
+                               qp::cplx(ia.amp[i].x, ia.amp[i].y);
+            ia.amp[i] = make_double2(f.real(), f.imag());
         }
-    }
-    std::vector<float2> af(n);
-    for (size_t i = 0; i < n; ++i) af[i] = make_float2((float)amps[i].x, (float)amps[i].y);
-    const void *asrc = c->cfg.precision == QP_C64 ? (const void *)af.data() : (const void *)amps.data();
-    DevState s{};
-    s.n_cur = n;
-    if (c->use_stream) {   // one path per region (instance, newest point a*M + b); keys without the instance
-        std::vector<unsigned long long> rn((size_t)2 * NI * MM, 0ull);
-        for (size_t i = 0; i < n; ++i) {
-            const int a = (int)(keys[i] & ((1u << bs) - 1u)), b = (int)((keys[i] >> bs) & ((1u << bs) - 1u));
-            const int inst = NI > 1 ? (int)(keys[i] >> c->P.inst_shift) : 0;
-            const size_t reg = (size_t)inst * MM + (size_t)(a * M + b);
-            keys[i] &= ~c->P.instmask;
-            QP_CUDA(c, cudaMemcpyAsync(c->P.keys[0] + reg * c->P.region_cap, &keys[i], 8, cudaMemcpyHostToDevice,
-                                       c->stream));
-            QP_CUDA(c, cudaMemcpyAsync(static_cast<char *>(c->P.amps[0]) + reg * c->P.region_cap * ab,
-                                       static_cast<const char *>(asrc) + i * ab, ab, cudaMemcpyHostToDevice, c->stream));
-            rn[reg] = 1;
-        }
-        QP_CUDA(c, cudaMemcpyAsync(c->P.reg_n, rn.data(), rn.size() * 8, cudaMemcpyHostToDevice, c->stream));
-        QP_CUDA(c, cudaStreamSynchronize(c->stream));   // rn and keys are host temporaries
-    } else {
-        QP_CUDA(c, cudaMemcpyAsync(c->P.keys[0], keys.data(), n * 8, cudaMemcpyHostToDevice, c->stream));
-        QP_CUDA(c, cudaMemcpyAsync(c->P.amps[0], asrc, n * ab, cudaMemcpyHostToDevice, c->stream));
-    }
-    QP_CUDA(c, cudaMemcpyAsync(c->P.st, &s, sizeof(DevState), cudaMemcpyHostToDevice, c->stream));
-    QP_CUDA(c, cudaMemcpyAsync(c->P.rho_ring, rho.data(), (size_t)NI * MM * sizeof(double2), cudaMemcpyHostToDevice,
-                               c->stream));
-    std::vector<long long> kept0(NI, nnz);
-    QP_CUDA(c, cudaMemcpyAsync(c->P.inst_kept, kept0.data(), NI * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
-    QP_CUDA(c, cudaMemsetAsync(c->P.fin_count, 0, sizeof(unsigned int), c->stream));
-    // look-back words are tagged with the step number, which restarts at 0:
-    // words of an earlier propagation must not pass for this one's
-    QP_CUDA(c, cudaMemsetAsync(c->P.tile_state, 0, (size_t)c->L.max_tiles * M * M * 8, c->stream));
-    StepRec r0{0, 0, 0, (long long)n, (long long)n};
-    QP_CUDA(c, cudaMemcpyAsync(c->P.stats_ring, &r0, sizeof(StepRec), cudaMemcpyHostToDevice, c->stream));
-    k_clear_table<<<c->nsm * 4, 256, 0, c->stream>>>(c->P.slots, c->P.repk, c->L.tcap);
+    if (c->cfg.precision == QP_C64) k_set_state<float2><<<1, 256, 0, c->stream>>>(c->P, MM, ia);
+    else k_set_state<double2><<<1, 256, 0, c->stream>>>(c->P, MM, ia);
     QP_CUDA(c, cudaGetLastError());
-    QP_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (c->use_stream) {
+        // look-back words are tagged with the step number, which restarts at
+        // 0: words of an earlier propagation must not pass for this one's
+        QP_CUDA(c, cudaMemsetAsync(c->P.tile_state, 0, (size_t)c->L.max_tiles * MM * 8, c->stream));
+    } else if (!c->P.post) {
+        // (the stream engine has no use for the merge table, 40 bytes per
+        // slot; every propagation that has clears it here)
+        k_clear_table<<<c->nsm * 4, 256, 0, c->stream>>>(c->P.slots, c->P.repk, c->L.tcap);
+        QP_CUDA(c, cudaGetLastError());
+    }
     c->have_state = true;
     c->failed = false;
     c->host_t = 0;
