@@ -1434,6 +1434,7 @@ __device__ __forceinline__ unsigned long long lb_word(unsigned epoch, unsigned s
 struct RegArgs {
     long long tn, ngroups;   // 0: read from the device
     int gs;
+    unsigned active;         // blocks with groups; the grid has one more, which publishes
 };
 template <int M, bool C64>
 __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(Params P, int lut_smem, RegArgs a) {
@@ -1496,8 +1497,8 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
         ngroups = t == 0 ? (long long)n_in / gs : gpr * MM;
     }
     const long long nchunk = (ngroups + 31) / 32;
-    const bool spare = nchunk < (long long)gridDim.x;
-    const unsigned active = spare ? (unsigned)nchunk : gridDim.x;   // blocks with groups
+    const bool spare = known || nchunk < (long long)gridDim.x;
+    const unsigned active = known ? a.active : spare ? (unsigned)nchunk : gridDim.x;   // blocks with groups
     const unsigned arrivals = active + (spare ? 1u : 0u);
     if (blockIdx.x >= arrivals) return;
     // the step's record and the new state (one thread)
@@ -1511,9 +1512,8 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
         st->cnt_groups[cs] = (unsigned long long)ngroups;
         publish_step(P, st, tn, MM, c);
     };
-    // counts known: the spare block, or the last one, publishes the step and
-    // leaves the region sizes; it alone reads the state
-    const bool publisher = known && blockIdx.x == arrivals - 1;
+    // counts known: the spare block publishes the step and leaves the region
+    // sizes; it alone reads the state
     auto publish_known = [&]() -> bool {   // false: an earlier error
         if (threadIdx.x == 32) {
             s_err = __ldcg(&st->err);
@@ -1592,7 +1592,6 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     unsigned err = 0;
     if (known) {
         pdl_wait();
-        if (publisher && !publish_known()) return;
         err = __ldcg(&st->err);   // (checked behind the first paths' loads)
     } else if (blockIdx.x == 0) {
         if ((int)threadIdx.x < MM) P.reg_n[outp * MM + threadIdx.x] = (unsigned long long)ngroups;
@@ -4050,7 +4049,16 @@ cudaError_t launch_stream_regular(qp_ctx *c, bool dep, RegArgs ra) {
         c->rcache_res = nb;
     }
     int g = std::min(c->nsm * c->rcache_res, kMaxExpandBlocks);
-    if (ra.tn) g = (int)std::min<long long>(g, (ra.ngroups + 31) / 32 + 1);   // no block without work
+    if (ra.tn) {
+        // one block per SM while a block's warps take a chunk or two each:
+        // fewer partials of rho to sum beside the step, and the publishing
+        // block on an SM of its own (memory 8 c64, 512 chunks: 456 blocks, the
+        // last of which also summed 456 partials at its end, took 8.2 us per step)
+        const long long chunks = (ra.ngroups + 31) / 32;
+        const int most = (chunks <= 2ll * kStreamWarps * c->nsm ? std::min(g, c->nsm) : g) - 1;
+        ra.active = (unsigned)std::min<long long>(chunks, std::max(1, most));
+        g = (int)ra.active + 1;
+    }
     int lut_smem = lutb ? 1 : 0;
     void *args[] = {(void *)&c->P, (void *)&lut_smem, (void *)&ra};
     return launch_pdl(fn, g, kRegThreads, lutb, c->stream, args, dep);
@@ -4078,7 +4086,7 @@ StepKind step_kind(const qp_ctx *c, int64_t tn) {
 // (tn = 0: not known, as in a captured graph).  At t = 0 the regions are
 // uneven, and beyond 2^40 paths the buffers end: read from the device.
 RegArgs known_counts(const qp_ctx *c, int64_t tn) {
-    RegArgs a{0, 0, 0};
+    RegArgs a{0, 0, 0, 0u};
     if (tn < 2) return a;
     const Params &P = c->P;
     const int MM = c->cfg.M * c->cfg.M, dk = c->cfg.dkmax;
@@ -4104,7 +4112,7 @@ cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind, int64_t t
     if (ev) cudaEventRecord(ev[0], c->stream);
     if constexpr (M < 4) {
         if (kind == kStepRegular || after_regular) {
-            cudaError_t e = launch_stream_regular<M, C64>(c, ev == nullptr, kind == kStepRegular ? known_counts(c, tn) : RegArgs{0, 0, 0});
+            cudaError_t e = launch_stream_regular<M, C64>(c, ev == nullptr, kind == kStepRegular ? known_counts(c, tn) : RegArgs{0, 0, 0, 0u});
             if (e != cudaSuccess) return e;
         }
     }
