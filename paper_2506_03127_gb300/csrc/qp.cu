@@ -4776,6 +4776,19 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
     if (!c->have_state) return fail(c, QP_ERR_STATE, "qp_set_rho0 must come before qp_step");
     if (c->failed) return fail(c, QP_ERR_STATE, "context holds a device error; call qp_set_rho0");
     if (nsteps == 0) return QP_OK;
+    // Single stream-engine steps are launched with what the host knows of
+    // them, which a replay would repeat: a stream under capture is refused,
+    // as it is where steps run as graphs; with graphs switched off
+    // (QP_NO_GRAPH) the captured kernels read the device state.
+    const bool single = c->use_stream && (c->graph_steps == 1 || !c->use_graph);
+    bool captured = false;
+    if (single && c->stream) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        QP_CUDA(c, cudaStreamIsCapturing(c->stream, &cap));
+        captured = cap != cudaStreamCaptureStatusNone;
+        if (captured && c->use_graph && !(c->use_persistent && c->P.n_inst > 1))
+            return fail(c, QP_ERR_CUDA, "qp_step: the stream is being captured");
+    }
     const int64_t t0 = c->host_t;
     c->host_t += nsteps;
     if (c->use_persistent && !c->use_stream && !c->P.post) {
@@ -4799,9 +4812,9 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
         c->graph_dirty = false;
     }
     for (int s = 0; s < nsteps;) {
-        const StepKind kind = step_kind(c, t0 + s + 1);
+        const StepKind kind = captured ? kStepBoth : step_kind(c, t0 + s + 1);
         if (!graphs) {
-            const cudaError_t e = launch_step(c, nullptr, kind, t0 + s + 1);
+            const cudaError_t e = launch_step(c, nullptr, kind, captured ? 0 : t0 + s + 1);
             if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
             ++s;
             continue;

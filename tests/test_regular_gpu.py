@@ -88,3 +88,28 @@ def test_mask_changed_in_mid_run(first, then):
         p.close()
     assert np.abs(out[0][0] - out[1][0]).max() <= 1e-10
     assert out[0][1] == out[1][1]
+
+
+def test_a_captured_stream_is_refused():
+    """The host passes the step index to single steps, so a graph that replayed
+    them would repeat it: qp_step refuses, and the propagation goes on after."""
+    import torch
+    from paper_2506_03127_gb300 import Propagator, abi
+    c = W.random_case(54, 2, 5)
+    rho0 = _rho0(2, 4, 5)
+    p = Propagator(2, 5, c["dt"], c["q"], c["hs"], 0.0, "fp64", "stream", max_paths=1 << 14)
+    p.set_eta(c["eta"])
+    p.set_mask(None)
+    p.set_rho0(rho0)
+    p.step(8)
+    p.sync()
+    x, g = torch.zeros(1, device="cuda"), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=p.stream):
+        x.add_(1)
+        with pytest.raises(abi.QPError):
+            p.step(1)
+    p.step(4)
+    rho = p.rho(0, 13)
+    p.close()
+    ref = iquapi.propagate(2, c["q"], c["hs"], c["dt"], c["eta"], 5, None, 0.0, rho0, 12)
+    assert np.abs(rho - ref.rho).max() <= 1e-10
