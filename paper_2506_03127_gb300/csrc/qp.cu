@@ -1899,7 +1899,12 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     static_assert(NX <= 16, "slot map: 4 bits of x");
     static_assert(NW == kStreamWarps, "warp partials");
     static_assert(!BATCH || NX == 1, "batches: P' a prefix of the window");
-    constexpr bool kTileAccS = !BATCH && M * M >= 9 && C64;   // per-warp tile sums of rho (see the accumulators)
+    // C64 single problems with M >= 3 sum rho(t+1) by columns of the staged
+    // children (see the accumulators), kCsThreads floats at a time: whole rows
+    // of 2 M*M, so that a thread keeps its column and reads without conflicts
+    constexpr bool kColSum = !BATCH && C64 && MM >= 9;
+    constexpr int kCsThreads = NT / (2 * MM) * (2 * MM);
+    static_assert(!kColSum || (Lay::stage && (size_t)kCsThreads * 8 <= (size_t)Lay::NSTG * MM * sizeof(AmpT)), "column sums");
     DevState *st = P.st;
     // Before the previous step's kernel is waited for: the propagator table
     // and the history tables of the step's window length, or on the chance that
@@ -1982,7 +1987,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     __shared__ unsigned s_ticket, s_nseg, s_ng, s_hw[NW];
     __shared__ int s_St;   // tile size of this step
     __shared__ float4 s_rt[NW][MM];
-    __shared__ float4 s_wrho[kTileAccS ? NW : 1][MM];   // M >= 3 single problems: per-warp sums of rho(t+1)
+    __shared__ float4 s_wrho[kColSum ? NW : 1][MM];   // per-warp sums of rho(t+1) over the children past the staged ones
     __shared__ bool s_last;
     __shared__ int s_any;   // the block processed a tile
     // runs of more than kOwnRun members that start in the tile, and the warps'
@@ -2015,7 +2020,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             }
         }
     if (threadIdx.x == 0) s_any = 0;
-    if constexpr (kTileAccS)
+    if constexpr (kColSum)
         for (int i = threadIdx.x; i < NW * MM; i += NT) (&s_wrho[0][0])[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if constexpr (BATCH) {
         for (int i = threadIdx.x; i < P.n_inst * (MM + 1); i += NT) s_acc[i] = make_double2(0.0, 0.0);
@@ -2081,14 +2086,19 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     // rho(t+1) accumulators of this thread: FP64, or on the C64 path FP32
     // with a Kahan compensation term (M = 2; plain FP32 sums for M >= 3).
     // Single problems keep them for the whole kernel and widen them once at
-    // the end, except C64 with M >= 3 (two blocks per SM, 128 registers:
-    // kept across the tile loop, the M*M accumulators were spilled and every
-    // child's addition went through local memory), where they live for one
-    // tile's write pass and a warp sum per tile is added to a per-warp FP32
-    // pair (TwoSum).  Batches sum them per tile into their instance's block
-    // sums
+    // the end, except C64 with M >= 3 (two blocks per SM, 128 registers: the
+    // M*M accumulators were spilled): there every thread adds one column of the
+    // tile's staged children (zeros below the filter) while the look-back
+    // words of the tiles before are on their way, one FP32 pair (TwoSum) per
+    // thread for the whole kernel; children past the staging buffer (more
+    // groups than it holds: the filling window) take a thread's accumulators
+    // and a warp sum per tile.  (All children by warp sums per tile, 31
+    // additions with two shuffles each: three-level chain 16.45 -> 15.99 ms per
+    // 30 steps; M = 2, whose threads' sums last the kernel, lost 1.7 %.)
+    // Batches sum them per tile into their instance's block sums
     constexpr bool kKahan = C64 && M == 2;
-    constexpr bool kTileAcc = BATCH || kTileAccS;
+    constexpr bool kTileAcc = BATCH || kColSum;
+    float cs_s = 0.f, cs_e = 0.f;   // this thread's column sum and its rounding errors
     typename X::AccT racc[kTileAcc ? 1 : MM], rcmp[kKahan && !kTileAcc ? MM : 1];
     if constexpr (!kTileAcc) {
 #pragma unroll
@@ -2645,9 +2655,15 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             s_keep[g] = (unsigned short)keep;
 #pragma unroll
             for (int c = 0; c < MM; ++c) {
-                if (!(keep & (1u << c))) continue;
-                ++cntc[c];
-                if (Lay::stage && g < Lay::NSTG) s_stg[g * MM + c] = v[c];
+                if constexpr (kColSum) {   // (zeros below the filter: the column sums read whole rows)
+                    const bool k = (keep & (1u << c)) != 0u;
+                    cntc[c] += k ? 1u : 0u;
+                    if (g < Lay::NSTG) s_stg[g * MM + c] = k ? v[c] : make_float2(0.f, 0.f);
+                } else {
+                    if (!(keep & (1u << c))) continue;
+                    ++cntc[c];
+                    if (Lay::stage && g < Lay::NSTG) s_stg[g * MM + c] = v[c];
+                }
             }
         }
         // block exclusive scan per new point (warp shuffles, then across warps)
@@ -2703,6 +2719,24 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
         // buckets c = warp + j * NW (KB per warp: two for M = 3, 4) are
         // looked back in the same rounds: their loads are issued together
         constexpr int KB = (MM + NW - 1) / NW;
+        if constexpr (kColSum) {
+            if ((int)warp < MM && lane == 0 && !withhold) {
+#pragma unroll
+                for (int j = 0; j < KB; ++j) {
+                    const int c = (int)warp + j * NW;
+                    if (c < MM)
+                        atomicExch(P.tile_state + (size_t)c * P.max_tiles + ticket,
+                                   lb_word(epoch, ticket == lb0 ? kLbInc : kLbAgg, s_tot[c]));
+                }
+            }
+            // (while the predecessors publish theirs)
+            if ((int)threadIdx.x < kCsThreads) {
+                const float *col = reinterpret_cast<const float *>(s_stg);
+                const int nf = min(ngroups, Lay::NSTG) * (2 * MM);
+#pragma unroll 4
+                for (int i = threadIdx.x; i < nf; i += kCsThreads) two_sum_acc(cs_s, cs_e, col[i]);
+            }
+        }
         if ((int)warp < MM) {
             unsigned long long excl[KB];
             long long pred[KB];
@@ -2713,9 +2747,10 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 excl[j] = 0;
                 pred[j] = ticket - 1;
                 done[j] = c >= MM || pred[j] < lb0;
-                if (c < MM && lane == 0 && !withhold)
-                    atomicExch(P.tile_state + (size_t)c * P.max_tiles + ticket,
-                               lb_word(epoch, ticket == lb0 ? kLbInc : kLbAgg, s_tot[c]));
+                if constexpr (!kColSum)
+                    if (c < MM && lane == 0 && !withhold)
+                        atomicExch(P.tile_state + (size_t)c * P.max_tiles + ticket,
+                                   lb_word(epoch, ticket == lb0 ? kLbInc : kLbAgg, s_tot[c]));
             }
             const long long t0 = clock64();
             bool timeout = false, abort = false;   // abort: another block raised an error
@@ -2854,6 +2889,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 keys_out[(rb + c) * G + o] = (shifted | code) & wmask;
                 amps_out[(rb + c) * G + o] = v[c];
                 if constexpr (kTileAcc) {
+                    if (kColSum && g < Lay::NSTG) continue;   // in the column sums
                     if constexpr (kKahan) {
                         X::kahan_add(tacc[c], tcmp[c], v[c]);
                     } else {
@@ -2868,7 +2904,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 }
             }
         }
-        if constexpr (kTileAcc) {
+        if constexpr (kTileAcc) if (!kColSum || ngroups > Lay::NSTG) {
             // the tile's rho(t+1): warp sums by halving (Kahan terms as the
             // pairs' second words), each component in one lane.  Batches add
             // it to the instance's block sums (shared FP64 atomics), single
@@ -2916,6 +2952,8 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
         __syncthreads();
     }
     cp_async_wait_all();   // a block without a tile: its table copies
+    if constexpr (kColSum)   // (the staging buffer is free: the loop ended with a barrier)
+        if ((int)threadIdx.x < kCsThreads) reinterpret_cast<float2 *>(s_stg)[threadIdx.x] = make_float2(cs_s, cs_e);
     // arrive first: the last block to arrive publishes the step, for which
     // it needs the step's counters only; every block then writes its partial
     // of rho, which the next step's block 0 (or a read-time finalisation)
@@ -2944,20 +2982,16 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     // processed no tile writes zeros without reducing (s_any: thread 0 holds
     // block_kept; the barrier below orders it)
     float4 *mine = spart_of(P, tn, MM) + (size_t)blockIdx.x * MM;
-    if constexpr (kTileAccS) {   // the warps' pairs merged in order (thread k: end point k; zeros without a tile)
-        if ((int)threadIdx.x < MM) {
-            const int k = threadIdx.x;
-            float4 a = s_wrho[0][k];
-            for (int w = 1; w < NW; ++w) {
-                const float4 b = s_wrho[w][k];
-                const float tx = a.x + b.x, vx = tx - a.x;
-                a.y += b.y + ((a.x - (tx - vx)) + (b.x - vx));
-                a.x = tx;
-                const float ty = a.z + b.z, vy = ty - a.z;
-                a.w += b.w + ((a.z - (ty - vy)) + (b.z - vy));
-                a.z = ty;
-            }
-            mine[k] = a;
+    if constexpr (kColSum) {   // one thread per component: the column's threads, then the warps' pairs, in order
+        if ((int)threadIdx.x < 2 * MM) {
+            float2 a = make_float2(0.f, 0.f);
+            auto add = [&](float2 b) {
+                two_sum_acc(a.x, a.y, b.x);
+                a.y += b.y;
+            };
+            for (int i = threadIdx.x; i < kCsThreads; i += 2 * MM) add(reinterpret_cast<const float2 *>(s_stg)[i]);
+            for (int w = 0; w < NW; ++w) add(reinterpret_cast<const float2 *>(&s_wrho[w][0])[threadIdx.x]);
+            reinterpret_cast<float2 *>(mine)[threadIdx.x] = a;
         }
     } else {
         if (threadIdx.x == 0) s_any = block_kept > 0 || s_any;
