@@ -1731,15 +1731,13 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
 // thread each (stream engine; the prefetch past the tile end holds as many),
 // runs of up to kWarpRun by a warp, longer ones by the block.
 constexpr int kOwnRun = 32, kWarpRun = 512;
-// A C64 group sum is the float2 in the low 8 bytes of its double2 slot.
-__device__ __forceinline__ void store_own_sum(double2 *slot, float2 S) { reinterpret_cast<float2 *>(slot)[0] = S; }
 
 // Dynamic shared memory of the stream kernel for a tile of S stored paths
 // (16-byte aligned arrays).  A tile holds at most NG = S + NX - 1 groups: every
 // group has a member in the tile, except sub-groups of the tile's last run
 // whose members all lie past the tile end (at most NX - 1 of them).
-//   gS    [NG] group sums (16 B each)   grep [NG] representative keys
-//   wm    [NG] maximum weight (bits)    key/amp [S] the tile's stored paths
+//   gS    [NG] group sums               grep [NG] representative keys
+//   key/amp [S] the tile's stored paths
 //   stage [NSTG][M*M] children amplitudes of the first NSTG groups (S/2
 //         for M = 2, S/3 otherwise) between the two passes (tiles usually
 //         hold fewer groups; later ones are recomputed in pass B)
@@ -1753,16 +1751,14 @@ __device__ __forceinline__ void store_own_sum(double2 *slot, float2 S) { reinter
 template <int M, bool C64, int NX, int S>
 struct StreamLayout {
     using AmpT = typename std::conditional<C64, float2, double2>::type;
-    using WT = typename std::conditional<C64, unsigned, unsigned long long>::type;
     static constexpr int MM = M * M;
     static constexpr int NG = S + NX - 1;
     static constexpr size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
     static constexpr int NSTG = M == 2 ? S / 2 : S / 3;
     static constexpr bool stage = (size_t)NSTG * MM * sizeof(AmpT) <= 64 * 1024;
     static constexpr size_t gS = 0;
-    static constexpr size_t grep = gS + a16((size_t)NG * sizeof(double2));
-    static constexpr size_t wm = grep + a16((size_t)NG * 8);
-    static constexpr size_t key = wm + a16((size_t)NG * sizeof(WT));
+    static constexpr size_t grep = gS + a16((size_t)NG * sizeof(AmpT));
+    static constexpr size_t key = grep + a16((size_t)NG * 8);
     static constexpr size_t amp = key + a16((size_t)(S + 32) * 8);
     static constexpr size_t stg = amp + a16((size_t)(S + 32) * sizeof(AmpT));
     static constexpr size_t seg = stg + (stage ? a16((size_t)NSTG * MM * sizeof(AmpT)) : 0);
@@ -1891,7 +1887,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     using X = Expander<M, C64>;
     using Lay = StreamLayout<M, C64, NX, S>;
     using AmpT = typename X::AmpT;
-    using WT = typename Lay::WT;   // weight |a|^2 as ordered bits: FP32 (C64) or FP64
+    using WT = typename std::conditional<C64, unsigned, unsigned long long>::type;   // weight |a|^2 as ordered bits: FP32 (C64) or FP64
     constexpr int MM = M * M;
     constexpr int NT = kStreamThreads, NW = NT / 32, EPT = S / NT;
     constexpr int NG = Lay::NG;
@@ -1965,9 +1961,8 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     unsigned long long *keys_out = P.keys[outp];
     AmpT *amps_out = static_cast<AmpT *>(P.amps[outp]);
 
-    double2 *s_gS = reinterpret_cast<double2 *>(s_dyn + Lay::gS);
+    AmpT *s_gS = reinterpret_cast<AmpT *>(s_dyn + Lay::gS);
     unsigned long long *s_grep = reinterpret_cast<unsigned long long *>(s_dyn + Lay::grep);
-    WT *s_wm = reinterpret_cast<WT *>(s_dyn + Lay::wm);
     unsigned long long *s_key = reinterpret_cast<unsigned long long *>(s_dyn + Lay::key);
     AmpT *s_amp = reinterpret_cast<AmpT *>(s_dyn + Lay::amp);
     AmpT *s_stg = reinterpret_cast<AmpT *>(s_dyn + Lay::stg);
@@ -2122,7 +2117,8 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     };
     // first wave: block b prefetches tile b's stored paths into L2 (one
     // address inside the tile per 128-byte line of keys and amplitudes), so
-    // that whichever block takes tile b finds it there
+    // that whichever block takes tile b finds it there (prefetching the tile a
+    // grid further on with every tile as well cost the chain 1 %, the sweep 5 %)
     if ((long long)blockIdx.x < ntiles) {
         const long long tk = blockIdx.x;
         const int rr = region_of(tk);
@@ -2198,11 +2194,6 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             if (lane == 0) s_ra_n = __popc(okm);   // a prefix of the 32 lanes
         }
         if (threadIdx.x == 0) s_kprev = e0 > 0 ? __ldcg(kin + e0 - 1) : 0ull;
-        for (int i = threadIdx.x; i < NG; i += NT) {
-            s_gS[i] = make_double2(0.0, 0.0);
-            s_grep[i] = kEmpty;
-            s_wm[i] = 0;
-        }
         if constexpr (NX > 1) {
             for (int i = threadIdx.x; i < S; i += NT) s_xm[i] = 0u;
             for (int i = threadIdx.x; i < St * NX / 4; i += NT) reinterpret_cast<uint4 *>(s_xmask)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -2442,7 +2433,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                         if (within_tie(weight_bits(s_amp[i]), wmx) && key < kmin) kmin = key;
                     }
                 }
-                if constexpr (C64) store_own_sum(s_gS + sl, make_float2(sh.x + se.x, sh.y + se.y));
+                if constexpr (C64) s_gS[sl] = make_float2(sh.x + se.x, sh.y + se.y);
                 else s_gS[sl] = make_double2(sh.x, sh.y);
                 s_grep[sl] = kmin;
             }
@@ -2561,7 +2552,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 }
             };
             auto put_sum = [&](int sl, const AccT &sh, const AccT &se) {
-                if constexpr (C64) store_own_sum(s_gS + sl, make_float2(sh.x + se.x, sh.y + se.y));
+                if constexpr (C64) s_gS[sl] = make_float2(sh.x + se.x, sh.y + se.y);
                 else s_gS[sl] = make_double2(sh.x, sh.y);
             };
             auto length = [&](int g) { return (g + 1 < nseg ? (long long)s_seg[g + 1] : ahead) - s_seg[g]; };
@@ -2598,6 +2589,10 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                         if constexpr (C64) s_lerr[warp][x] = se[x];
                         s_lwm[warp][x] = wmx[x];
                     }
+                }
+                if (threadIdx.x < NX) {
+                    const int sl = slot(g, (int)threadIdx.x);
+                    if (sl >= 0) s_grep[sl] = kEmpty;
                 }
                 __syncthreads();
 #pragma unroll
@@ -2646,11 +2641,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             unsigned keep = 0;
             AmpT v[MM];
             if (rk != kEmpty) {
-                if constexpr (C64) {
-                    keep = X::children_tab(P, tab_t, rk, reinterpret_cast<const float2 *>(s_gS)[2 * g], w_t, wf_t, v);
-                } else {
-                    keep = X::children_tab(P, tab_t, rk, s_gS[g], w_t, wf_t, v);
-                }
+                keep = X::children_tab(P, tab_t, rk, s_gS[g], w_t, wf_t, v);
             }
             s_keep[g] = (unsigned short)keep;
 #pragma unroll
@@ -2831,7 +2822,12 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                         if (ticket > lb0 && !withhold)
                             atomicExch(P.tile_state + (size_t)c * P.max_tiles + ticket,
                                        lb_word(epoch, kLbInc, excl[j] + tot));
-                        s_base[c] = excl[j];
+                        // (a region that overflows fails the step: nothing of the tile is written)
+                        if (excl[j] + tot > (unsigned long long)G) {
+                            raise_err(st, kErrPaths);
+                            s_lbfail = 1;
+                        }
+                        s_base[c] = (unsigned long long)((rb + c) * G) + excl[j];
                         if (ticket == tlast) P.reg_n[(size_t)outp * R + rb + c] = excl[j] + tot;   // the last tile knows the sizes
                     }
                 }
@@ -2844,7 +2840,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             if (ngroups) atomicAdd(&st->cnt_groups[cs], (unsigned long long)ngroups);
             if (ticket == tlast) {
                 unsigned long long sumc = 0;
-                for (int c = 0; c < MM; ++c) sumc += s_base[c] + s_tot[c];
+                for (int c = 0; c < MM; ++c) sumc += s_base[c] - (unsigned long long)((rb + c) * G) + s_tot[c];
                 if constexpr (BATCH) atomicAdd(&st->cnt_out[cs], sumc);   // zeroed by the previous step
                 else st->cnt_out[cs] = sumc;
             }
@@ -2871,8 +2867,6 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
 #pragma unroll
                 for (int c = 0; c < MM; ++c)
                     if (keep & (1u << c)) v[c] = s_stg[g * MM + c];
-            } else if constexpr (C64) {
-                X::children_tab(P, tab_t, rk, reinterpret_cast<const float2 *>(s_gS)[2 * g], w_t, wf_t, v);
             } else {
                 X::children_tab(P, tab_t, rk, s_gS[g], w_t, wf_t, v);
             }
@@ -2881,13 +2875,9 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             for (int c = 0; c < MM; ++c) {
                 if (!(keep & (1u << c))) continue;
                 const unsigned long long o = s_base[c] + tb[c]++;
-                if ((long long)o >= G) {
-                    raise_err(st, kErrPaths);
-                    continue;
-                }
                 const unsigned long long code = (unsigned long long)((c / M) | ((c % M) << P.bs));
-                keys_out[(rb + c) * G + o] = (shifted | code) & wmask;
-                amps_out[(rb + c) * G + o] = v[c];
+                keys_out[o] = (shifted | code) & wmask;
+                amps_out[o] = v[c];
                 if constexpr (kTileAcc) {
                     if (kColSum && g < Lay::NSTG) continue;   // in the column sums
                     if constexpr (kKahan) {
