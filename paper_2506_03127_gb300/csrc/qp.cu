@@ -1898,8 +1898,11 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     // C64 single problems with M >= 3 sum rho(t+1) by columns of the staged
     // children (see the accumulators), kCsThreads floats at a time: whole rows
     // of 2 M*M, so that a thread keeps its column and reads without conflicts
-    constexpr bool kColSum = !BATCH && C64 && MM >= 9;
-    constexpr int kCsThreads = NT / (2 * MM) * (2 * MM);
+    // (batches of M = 2: by the warps that have no look-back, which then add
+    // the tile's eight sums to the instance's: 64-instance sweep 8.21 -> 7.78 ms
+    // per 100 steps against warp sums of every thread's accumulators)
+    constexpr bool kColSum = C64 && (BATCH ? MM == 4 : MM >= 9);
+    constexpr int kCsFirst = BATCH ? NT / 2 : 0, kCsThreads = (NT - kCsFirst) / (2 * MM) * (2 * MM);
     static_assert(!kColSum || (Lay::stage && (size_t)kCsThreads * 8 <= (size_t)Lay::NSTG * MM * sizeof(AmpT)), "column sums");
     DevState *st = P.st;
     // Before the previous step's kernel is waited for: the propagator table
@@ -1982,7 +1985,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     __shared__ unsigned s_ticket, s_nseg, s_ng, s_hw[NW];
     __shared__ int s_St;   // tile size of this step
     __shared__ float4 s_rt[NW][MM];
-    __shared__ float4 s_wrho[kColSum ? NW : 1][MM];   // per-warp sums of rho(t+1) over the children past the staged ones
+    __shared__ float4 s_wrho[kColSum && !BATCH ? NW : 1][MM];   // per-warp sums of rho(t+1) over the children past the staged ones
     __shared__ bool s_last;
     __shared__ int s_any;   // the block processed a tile
     // runs of more than kOwnRun members that start in the tile, and the warps'
@@ -2015,7 +2018,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             }
         }
     if (threadIdx.x == 0) s_any = 0;
-    if constexpr (kColSum)
+    if constexpr (kColSum && !BATCH)
         for (int i = threadIdx.x; i < NW * MM; i += NT) (&s_wrho[0][0])[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if constexpr (BATCH) {
         for (int i = threadIdx.x; i < P.n_inst * (MM + 1); i += NT) s_acc[i] = make_double2(0.0, 0.0);
@@ -2728,11 +2731,25 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 }
             }
             // (while the predecessors publish theirs)
-            if ((int)threadIdx.x < kCsThreads) {
+            const int cst = (int)threadIdx.x - kCsFirst;
+            if (cst >= 0 && cst < kCsThreads) {
                 const float *col = reinterpret_cast<const float *>(s_stg);
                 const int nf = min(ngroups, Lay::NSTG) * (2 * MM);
 #pragma unroll 4
-                for (int i = threadIdx.x; i < nf; i += kCsThreads) two_sum_acc(cs_s, cs_e, col[i]);
+                for (int i = cst; i < nf; i += kCsThreads) two_sum_acc(cs_s, cs_e, col[i]);
+                if constexpr (BATCH) {   // into the instance's block sums: whole warps, 2 M*M = 8 columns
+                    static_assert(kCsFirst % 32 == 0 && kCsThreads % 32 == 0 && 32 % (2 * MM) == 0, "columns of a warp");
+#pragma unroll
+                    for (int o = 2 * MM; o < 32; o <<= 1) {
+                        const float b = __shfl_xor_sync(0xffffffffu, cs_s, o), f = __shfl_xor_sync(0xffffffffu, cs_e, o);
+                        two_sum_acc(cs_s, cs_e, b);
+                        cs_e += f;
+                    }
+                    const double x = f2d_exact(cs_s) + f2d_exact(cs_e);
+                    if ((int)lane < 2 * MM && x != 0.0)
+                        atomicAdd(reinterpret_cast<double *>(s_acc + (size_t)inst * (MM + 1)) + lane, x);
+                    cs_s = cs_e = 0.f;
+                }
             }
         }
         if ((int)warp < MM) {
@@ -2843,7 +2860,10 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
         __syncthreads();
         const bool lbfail = s_lbfail != 0;
         if (threadIdx.x == 0 && !lbfail) {
-            for (int c = 0; c < MM; ++c) block_kept += s_tot[c];
+            unsigned long long kt = 0;
+            for (int c = 0; c < MM; ++c) kt += s_tot[c];
+            if constexpr (BATCH) atomicAdd(reinterpret_cast<double *>(s_acc + (size_t)inst * (MM + 1)) + 2 * MM, (double)kt);
+            block_kept += kt;
             if (ngroups) atomicAdd(&st->cnt_groups[cs], (unsigned long long)ngroups);
             if (ticket == tlast) {
                 unsigned long long sumc = 0;
@@ -2932,11 +2952,6 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                     else x = sv[0];
                     if (x != 0.0) atomicAdd(acc + idx, x);
                 }
-                if (threadIdx.x == 0 && !lbfail) {
-                    unsigned long long kt = 0;
-                    for (int c = 0; c < MM; ++c) kt += s_tot[c];
-                    atomicAdd(acc + 2 * MM, (double)kt);
-                }
             } else if constexpr (C64) {
                 if (mine) {
                     float2 a = reinterpret_cast<float2 *>(&s_wrho[warp][0])[idx];
@@ -2949,7 +2964,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
         __syncthreads();
     }
     cp_async_wait_all();   // a block without a tile: its table copies
-    if constexpr (kColSum)   // (the staging buffer is free: the loop ended with a barrier)
+    if constexpr (kColSum && !BATCH)   // (the staging buffer is free: the loop ended with a barrier)
         if ((int)threadIdx.x < kCsThreads) reinterpret_cast<float2 *>(s_stg)[threadIdx.x] = make_float2(cs_s, cs_e);
     // arrive first: the last block to arrive publishes the step, for which
     // it needs the step's counters only; every block then writes its partial
@@ -2979,7 +2994,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     // processed no tile writes zeros without reducing (s_any: thread 0 holds
     // block_kept; the barrier below orders it)
     float4 *mine = spart_of(P, tn, MM) + (size_t)blockIdx.x * MM;
-    if constexpr (kColSum) {   // one thread per component: the column's threads, then the warps' pairs, in order
+    if constexpr (kColSum && !BATCH) {   // one thread per component: the column's threads, then the warps' pairs, in order
         if ((int)threadIdx.x < 2 * MM) {
             float2 a = make_float2(0.f, 0.f);
             auto add = [&](float2 b) {
