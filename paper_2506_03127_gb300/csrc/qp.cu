@@ -2136,9 +2136,22 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
         }
     }
 
-    for (;;) {
+    // The next ticket is taken with the write pass still to come where that is
+    // short and even (C64, M = 2: headline model 3.09 -> 3.05 ms, sweep 7.80 ->
+    // 7.70 ms), so that its trip is hidden.  Elsewhere tiles would start out of
+    // order and the look-backs of later ones wait for them (three-level chain
+    // 14.65 -> 15.70 ms, FP64 headline model 3.77 -> 3.81 ms), as they would
+    // everywhere if it were taken beside the look-back.
+    constexpr bool kEarlyTicket = C64 && M == 2;
+    if constexpr (kEarlyTicket) {
         if (threadIdx.x == 0) s_ticket = atomicAdd(&st->ticket[cs], 1u);
         __syncthreads();
+    }
+    for (;;) {
+        if constexpr (!kEarlyTicket) {
+            if (threadIdx.x == 0) s_ticket = atomicAdd(&st->ticket[cs], 1u);
+            __syncthreads();
+        }
         const long long ticket = s_ticket;
         if (ticket >= ntiles) {
             // the first block without a tile sums the previous step's rho,
@@ -2771,6 +2784,11 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             bool timeout = false, abort = false;   // abort: another block raised an error
             for (;;) {
                 unsigned wv[KB][LBK];   // (state << 30) | count of this step; 0: not yet published
+                // the error flag with the words, so that a round that has to
+                // wait is one trip (chain 14.73 -> 14.65 ms, headline model 3.11 ->
+                // 3.09 ms; batches, with few tiles to wait for, lost 0.5 %)
+                unsigned failed = 0;
+                if constexpr (!BATCH) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(failed) : "l"(&st->err) : "memory");
 #pragma unroll
                 for (int j = 0; j < KB; ++j) {
                     const unsigned long long *bucket = P.tile_state + (size_t)((int)warp + j * NW) * P.max_tiles;
@@ -2822,7 +2840,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 }
                 if (all) break;
                 if (wait) {
-                    if (*(volatile unsigned *)&st->err) {
+                    if (BATCH ? *(volatile unsigned *)&st->err : failed) {
                         abort = true;
                         break;
                     }
@@ -2872,6 +2890,8 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 else st->cnt_out[cs] = sumc;
             }
         }
+        unsigned next = 0;
+        if (kEarlyTicket && threadIdx.x == 0) next = atomicAdd(&st->ticket[cs], 1u);
         // pass B: write the survivors to their regions
         if constexpr (kTbShared) {
 #pragma unroll
@@ -2961,6 +2981,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 }
             }
         }
+        if (kEarlyTicket && threadIdx.x == 0) s_ticket = next;
         __syncthreads();
     }
     cp_async_wait_all();   // a block without a tile: its table copies
