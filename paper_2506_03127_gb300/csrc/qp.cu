@@ -2218,12 +2218,17 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
         __syncthreads();
         // run heads (ept consecutive entries per thread), block scan of their count
         unsigned hmask = 0;
+        {
+            const int i0 = threadIdx.x * ept;
+            unsigned long long prev = i0 == 0 ? s_kprev : i0 <= cnt ? s_key[i0 - 1] : 0ull;
 #pragma unroll
-        for (int u = 0; u < EPT; ++u) {
-            const int i = threadIdx.x * ept + u;
-            if (u < ept && i < cnt) {
-                if (i == 0 && e0 == 0) hmask |= 1u << u;
-                else if ((s_key[i] & pref) != ((i > 0 ? s_key[i - 1] : s_kprev) & pref)) hmask |= 1u << u;
+            for (int u = 0; u < EPT; ++u) {
+                const int i = i0 + u;
+                if (u < ept && i < cnt) {
+                    const unsigned long long key = s_key[i];
+                    if (((key ^ prev) & pref) != 0ull || (i == 0 && e0 == 0)) hmask |= 1u << u;
+                    prev = key;
+                }
             }
         }
         const unsigned hc = __popc(hmask);
@@ -2408,9 +2413,8 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 typename X::AccT sh, se;
                 sh.x = sh.y = 0;
                 se.x = se.y = 0;
-                WT wmx = 0;
+                WT wmx = 0, w2 = 0;   // the two largest weights (a tie shows in both)
                 int imx = b0;
-                bool some = false, multi = false;
                 auto add = [&](int i) {
                     const AmpT a = s_amp[i];
                     if constexpr (C64) {
@@ -2421,14 +2425,11 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                         sh.y += a.y;
                     }
                     const WT wb = weight_bits(a);
-                    if (!some || wb > wmx) {
-                        multi = some && wb - wmx <= kNear;
-                        wmx = wb;
-                        imx = i;
-                    } else if (wmx - wb <= kNear) {
-                        multi = true;
-                    }
-                    some = true;
+                    const bool up = wb > wmx;
+                    const WT less = up ? wmx : wb;
+                    w2 = less > w2 ? less : w2;
+                    wmx = up ? wb : wmx;
+                    imx = up ? i : imx;
                 };
                 unsigned mm;   // the group's members by offset in the run
                 if constexpr (NX > 1) {
@@ -2441,7 +2442,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                     for (int j = 0; j < n; ++j) add(b0 + j);
                 }
                 unsigned long long kmin = s_key[imx];
-                if (multi) {
+                if (wmx - w2 <= kNear) {   // (weights of 0 too: imx may then be no member)
                     kmin = kEmpty;
                     for (unsigned m = mm; m; m &= m - 1u) {
                         const int i = b0 + __ffs(m) - 1;
