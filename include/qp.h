@@ -157,7 +157,8 @@ enum { QP_LAUNCH_GRAPH = 0,        /* CUDA graphs of the step's kernels         
                                       qp_step call, bounded grid barriers between
                                       phases (merge-table engine) or steps
                                       (batches on the stream engine); single
-                                      problems on the stream engine run graphs  */
+                                      problems on the stream engine launch their
+                                      steps one by one                          */
 typedef struct {
     int mode;                  /* QP_LAUNCH_*                                     */
     int insert_blocks_per_sm;  /* pre-merge kernels (graph mode)                 */

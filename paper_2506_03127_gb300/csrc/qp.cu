@@ -1429,7 +1429,7 @@ __device__ __forceinline__ unsigned long long lb_word(unsigned epoch, unsigned s
 // without the arrivals: what is left is one trip for the paths, the
 // children and the stores.  (Reading the state, then the region sizes, and
 // publishing behind the last arrival: 9 us per step at memory 5 FP64 and 8
-// c64.)  Replayed graphs, the first step and steps launched ahead of the
+// c64.)  Captured steps, the first step and steps launched ahead of the
 // tile kernel read the state.
 struct RegArgs {
     long long tn, ngroups;   // 0: read from the device
@@ -1912,7 +1912,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     __shared__ float4 s_wf[BATCH ? 1 : MM * MM];
     extern __shared__ __align__(16) unsigned char s_dyn[];
     // (tn_host: the step index where the host launches the step itself, 0 in
-    // a replayed graph)
+    // a captured one)
     const int n_ahead = tn_host ? (int)min(tn_host, (unsigned long long)P.dkmax) : P.dkmax;
     Tab tab = tab_global(P, n_ahead, 0);
     // (rows are whole multiples of kLutEntries entries, so every copy is
@@ -3946,8 +3946,8 @@ struct qp_ctx {
     bool use_stream = false;           // this propagation runs on the stream engine
     bool sym = false;                  // symmetric Trotter splitting (qp_set_end_points)
     qp::cplx eta00;                    // ... point 0's half-interval self coefficient
-    cudaGraphExec_t graph1[3] = {};    // one-step graphs and graphs of graph_steps steps, by StepKind
-    cudaGraphExec_t graph[3] = {};
+    cudaGraphExec_t graph1 = nullptr;  // one-step graph and graph of graph_steps steps
+    cudaGraphExec_t graph = nullptr;
     bool graph_dirty = true;           // none of them is current
     bool reg_track = false;            // path counts of an unfiltered stream propagation known on the host (step_kind)
     bool use_graph = true;
@@ -3971,11 +3971,9 @@ qp_status fail(qp_ctx *c, qp_status s, const std::string &msg) {
     } while (0)
 
 void drop_graphs(qp_ctx *c) {
-    for (int k = 0; k < 3; ++k) {
-        if (c->graph1[k]) cudaGraphExecDestroy(c->graph1[k]);
-        if (c->graph[k]) cudaGraphExecDestroy(c->graph[k]);
-        c->graph1[k] = c->graph[k] = nullptr;
-    }
+    if (c->graph1) cudaGraphExecDestroy(c->graph1);
+    if (c->graph) cudaGraphExecDestroy(c->graph);
+    c->graph1 = c->graph = nullptr;
 }
 
 constexpr int kStepKernels = 4;
@@ -4135,7 +4133,7 @@ cudaError_t launch_stream_regular(qp_ctx *c, bool dep, RegArgs ra) {
 // The kernels that a step of the stream engine may need: the regular kernel,
 // the tile kernel, or the regular kernel and behind it the tile kernel, which
 // returns at once when the regular kernel took the step.
-enum StepKind { kStepBoth = 0, kStepRegular = 1, kStepTile = 2, kStepKinds = 3 };
+enum StepKind { kStepBoth, kStepRegular, kStepTile };
 
 // Which of them step tn needs.  Without a filter every child survives, so
 // that the path counts, and with them the regular steps, are known here as
@@ -4234,7 +4232,7 @@ cudaError_t launch_post_t(qp_ctx *c, cudaEvent_t *ev) {
     return cudaGetLastError();
 }
 
-// tn: the step where the host launches it, 0 in a graph that is replayed
+// tn: the step where the host launches it, 0 in a graph
 cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev, StepKind kind, int64_t tn) {
     const bool c64 = c->cfg.precision == QP_C64;
     if (c->P.post) {
@@ -4820,7 +4818,7 @@ qp_status qp_set_rho0(qp_ctx *c, const double *re, const double *im) {
     return QP_OK;
 }
 
-static qp_status capture_graph(qp_ctx *c, int steps, StepKind kind, cudaGraphExec_t *out) {
+static qp_status capture_graph(qp_ctx *c, int steps, cudaGraphExec_t *out) {
     if (*out) {
         cudaGraphExecDestroy(*out);
         *out = nullptr;
@@ -4828,7 +4826,7 @@ static qp_status capture_graph(qp_ctx *c, int steps, StepKind kind, cudaGraphExe
     cudaGraph_t g;
     QP_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = cudaSuccess;
-    for (int s = 0; s < steps && le == cudaSuccess; ++s) le = launch_step(c, nullptr, kind, 0);
+    for (int s = 0; s < steps && le == cudaSuccess; ++s) le = launch_step(c, nullptr, kStepTile, 0);
     cudaError_t ce = cudaStreamEndCapture(c->stream, &g);
     if (le != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(le));
     if (ce != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(ce));
@@ -4844,11 +4842,17 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
     if (!c->have_state) return fail(c, QP_ERR_STATE, "qp_set_rho0 must come before qp_step");
     if (c->failed) return fail(c, QP_ERR_STATE, "context holds a device error; call qp_set_rho0");
     if (nsteps == 0) return QP_OK;
-    // Single stream-engine steps are launched with what the host knows of
-    // them, which a replay would repeat: a stream under capture is refused,
-    // as it is where steps run as graphs; with graphs switched off
-    // (QP_NO_GRAPH) the captured kernels read the device state.
-    const bool single = c->use_stream && (c->graph_steps == 1 || !c->use_graph);
+    // Steps of a single problem on the stream engine are launched one by one:
+    // the host passes what it knows of them, dependent launches follow each
+    // other without a graph launch's gap, and nothing is captured again after
+    // qp_set_rho0 (headline model, 160 steps: 14.5 us per step, in graphs of
+    // eight 14.9).  A replay would repeat what the host passed: a stream under
+    // capture is refused, as it is where steps run as graphs; with graphs
+    // switched off (QP_NO_GRAPH) the captured kernels read the device state.
+    // Batches do the same unless several steps go into a graph; the other
+    // engines go into graphs (the table engine's kernels are 6 % slower one by
+    // one).
+    const bool single = c->use_stream && (c->P.n_inst == 1 || c->graph_steps == 1);
     bool captured = false;
     if (single && c->stream) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -4869,29 +4873,23 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
         if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("persistent launch: ") + cudaGetErrorString(e));
         return QP_OK;
     }
-    // graphs where several kernels or steps go into one; single steps of the
-    // stream engine are launched as they are (dependent launches follow each
-    // other without the graph launch's gap, and nothing is captured again
-    // after qp_set_rho0; the table engine's four kernels are 6 % slower that
-    // way)
-    const bool graphs = c->use_graph && (c->graph_steps > 1 || !c->use_stream);
-    if (graphs && c->graph_dirty) {
+    if (single || !c->use_graph) {
+        for (int s = 0; s < nsteps; ++s) {
+            const int64_t tn = t0 + s + 1;
+            const cudaError_t e = launch_step(c, nullptr, captured ? kStepBoth : step_kind(c, tn), captured ? 0 : tn);
+            if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
+        }
+        return QP_OK;
+    }
+    if (c->graph_dirty) {
         drop_graphs(c);
         c->graph_dirty = false;
     }
     for (int s = 0; s < nsteps;) {
-        const StepKind kind = captured ? kStepBoth : step_kind(c, t0 + s + 1);
-        if (!graphs) {
-            const cudaError_t e = launch_step(c, nullptr, kind, captured ? 0 : t0 + s + 1);
-            if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
-            ++s;
-            continue;
-        }
-        // as many steps as need the same kernels in one graph
-        const bool many = c->graph_steps > 1 && nsteps - s >= c->graph_steps && kind == step_kind(c, t0 + s + c->graph_steps);
-        cudaGraphExec_t &g = many ? c->graph[kind] : c->graph1[kind];
+        const bool many = c->graph_steps > 1 && nsteps - s >= c->graph_steps;
+        cudaGraphExec_t &g = many ? c->graph : c->graph1;
         if (!g) {
-            const qp_status st = capture_graph(c, many ? c->graph_steps : 1, kind, &g);
+            const qp_status st = capture_graph(c, many ? c->graph_steps : 1, &g);
             if (st != QP_OK) return st;
         }
         QP_CUDA(c, cudaGraphLaunch(g, c->stream));
