@@ -18,11 +18,12 @@
 // kernel that produces it.
 //
 // Rollout (qp_surrogate_rollout): for up to 32 instances all steps run in
-// one launch of a two-block cluster (k_rollout_fused: block 0 keeps W1^T and
-// the last L steps of rho in shared memory and runs the feature packing,
+// one launch, networks of up to 256 columns on a cluster of eight blocks
+// (k_rollout_cluster), wider ones on two (k_rollout_fused: block 0 keeps W1^T
+// and the last L steps of rho in shared memory and runs the feature packing,
 // layer 1 and the update; block 1 keeps W2^T and W3^T and runs layers 2 and
 // 3; activations cross through distributed shared memory); larger batches
-// replay CUDA graphs of the per-step kernels.  Both round at the same points
+// replay CUDA graphs of the per-step kernels.  All round at the same points
 // and add the k-steps in the same order.
 //
 // Tensor-core form: warp-level mma.sync fragments.  These GEMMs are small

@@ -113,3 +113,25 @@ def test_a_captured_stream_is_refused():
     p.close()
     ref = iquapi.propagate(2, c["q"], c["hs"], c["dt"], c["eta"], 5, None, 0.0, rho0, 12)
     assert np.abs(rho - ref.rho).max() <= 1e-10
+
+
+@pytest.mark.parametrize("precision", ["fp64", "c64"])
+def test_steps_of_more_chunks_than_warps(precision):
+    """59 049 groups (1846 chunks of 32, the last ragged) on at most 1216 warps.
+    The counts that the blocks leave with their partials add up to the step's."""
+    from paper_2506_03127_gb300 import Propagator
+    M, dkmax, T = 3, 6, 8
+    c = W.random_case(55, M, dkmax)
+    rho0 = _rho0(M, 5, 9)
+    p = Propagator(M, dkmax, c["dt"], c["q"], c["hs"], 0.0, precision, "stream", max_paths=1 << 20)
+    p.set_eta(c["eta"])
+    p.set_mask(None)
+    p.set_rho0(rho0)
+    p.step(T)
+    rho, st = p.rho(0, T + 1), p.stats(1, T)
+    kept = [int(np.ravel(p.instance_counts(t))[0]) for t in range(1, T + 1)]
+    p.close()
+    ref = iquapi.propagate(M, c["q"], c["hs"], c["dt"], c["eta"], dkmax, None, 0.0, rho0, T)
+    assert [(r[1], r[3]) for r in st] == [(o.groups, o.kept) for o in ref.stats]
+    assert kept == [o.kept for o in ref.stats]
+    assert np.abs(rho - ref.rho).max() <= (1e-10 if precision == "fp64" else 2e-6 * max(1.0, np.abs(ref.rho).max()))
