@@ -13,10 +13,10 @@
 //   post-merging engine (the order of Sec. 2.1): k_post_*, a device radix
 //     sort (k_rs_*) and a reduction by key (k_rbk_*).
 // Also here: the partition of a stored set by owner rank (k_part_*), the
-// allocation-free step (qp_step_noalloc) and the C ABI.  Every kernel reads
-// the step index and the path counts from a small device-resident state
-// block, so the host never waits on a count and one captured CUDA graph
-// replays any step.  The merge-table engine's sequence:
+// allocation-free step (qp_step_noalloc) and the C ABI.  The path counts (and
+// in a graph the step index) stay in a small device-resident state block, so
+// the host never waits on a count; single problems on the stream engine are
+// passed what the host knows of a step.  The merge-table engine's sequence:
 //
 //   k_insert    pre-merge pass 1 (window full only): each stored path
 //               inserts its masked key into the merge table (open
@@ -37,8 +37,9 @@
 //               then reduced per block, survivors appended to the other
 //               ping-pong buffer (warp-aggregated atomic cursor).  The
 //               group's table slot is reset after it is read.
-//   k_finalize  one thread: publishes the new count, per-step statistics,
-//               advances t, zeroes the next rho accumulator.
+//               The last block of a single problem sums rho's block
+//               partials and publishes the step (count, statistics, t);
+//   k_finalize  the same for batches, a block per instance.
 //
 // Precision (template parameter Amp): double2 amplitudes (QP_FP64) or
 // float2 amplitudes (QP_C64) with the influence exponent accumulated in FP32
@@ -1876,8 +1877,8 @@ __device__ __forceinline__ unsigned long long ld_relaxed_gpu(const unsigned long
 // 32 * LB_K predecessors per round, bounded waits); write the survivors.
 // Output region c receives, in order, the children with newest point c of
 // all groups, so the next set is again sorted.  No atomics on the data.  The
-// last block to finish sums the blocks' partials of rho(t+1) and publishes
-// the step.  flags: kFlagLutSmem (the history tables of this window length
+// last block to finish publishes the step; the blocks' partials of rho(t+1)
+// are summed by the next step or before a read.  flags: kFlagLutSmem (the history tables of this window length
 // are copied into shared memory once per block), kFlagAfterRegular (the
 // regular kernel was launched for the same step and may have taken it).
 constexpr int kFlagLutSmem = 1, kFlagAfterRegular = 2;
