@@ -118,6 +118,8 @@ struct __align__(128) DevState {
     unsigned int post_bits;           // post-merging: significant bits of the running step's sort key
     unsigned long long post_n;        // post-merging: unmerged children of the running step
     unsigned long long scan_total;    // total of the last multi-block scan
+    unsigned long long ext_t, ext_n;  // merge table, graph mode: t and n_cur of the running step, left by k_insert
+                                      // for k_expand, whose last block rewrites t and n_cur
     unsigned int bar_count;           // grid barrier of the persistent kernel: arrivals
     unsigned int pad1[31];
     unsigned int bar_gen;             // generation (own cache line)
@@ -474,9 +476,13 @@ template <typename Amp>
 __global__ void __launch_bounds__(kInsertThreads) k_insert(Params P) {
     DevState *st = P.st;
     if (st->err) return;
-    const unsigned long long t = st->t, tn = t + 1;
+    const unsigned long long t = st->t, tn = t + 1, n = st->n_cur;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->ext_t = t;
+        st->ext_n = n;
+    }
     if (tn < (unsigned long long)P.dkmax) return;   // window not full: no merge
-    phase_insert<Amp, kInsertThreads>(P, t, st->n_cur, &st->cnt_groups[tn % 3]);
+    phase_insert<Amp, kInsertThreads>(P, t, n, &st->cnt_groups[tn % 3]);
 }
 
 template <typename Amp>
@@ -1252,13 +1258,16 @@ __device__ __forceinline__ void finalize_single(const Params &P, unsigned long l
 // Extension of the step's groups or paths.  Single problems: the last block to
 // arrive also finalises and publishes the step (a kernel of its own for that
 // took 10 us of a 41 us step at 9e4 groups); batches leave it to k_finalize.
+// Blocks without work do not arrive, so the step may be published before one
+// of them has started: what decides whether a block has work is read from
+// fields the publication leaves alone (ext_t, ext_n, this step's cnt_groups).
 template <int M, bool C64, bool BATCH>
 __global__ void __launch_bounds__(kExpandThreads) k_expand(Params P) {
     DevState *st = P.st;
     if (st->err) return;
-    const unsigned long long t = st->t, tn = t + 1;
+    const unsigned long long t = st->ext_t, tn = t + 1;
     const bool merge = tn >= (unsigned long long)P.dkmax;
-    const unsigned long long n = merge ? st->cnt_groups[tn % 3] : st->n_cur;
+    const unsigned long long n = merge ? st->cnt_groups[tn % 3] : st->ext_n;
     const int nact = expand_blocks((int)gridDim.x, n);
     if ((int)blockIdx.x >= nact) return;
     phase_expand<M, C64, kExpandThreads, BATCH>(P, t, n, merge, &st->cnt_out[tn % 3], rho_part_of(P, tn, M * M));
