@@ -1423,9 +1423,12 @@ __device__ __forceinline__ unsigned long long lb_word(unsigned epoch, unsigned s
 //
 // Work split: chunks of 32 groups (a warp's), dealt to the blocks in turn,
 // so that a small step uses as many SMs as it has chunks; blocks without a
-// chunk return at once, except the first of them, which sums the pending
+// chunk arrive at once, except the first of them, which sums the pending
 // rho of the previous step beside the others (a grid without a spare block
-// leaves that to its last block, after it has arrived).  At memory 8
+// leaves that to its last block, after it has arrived).  Where the state is
+// read from the device every block of the grid arrives once it has read it:
+// the last arrival rewrites the state, which a block that starts late would
+// otherwise take for its step's.  At memory 8
 // (1.6e4 groups, complex64) and 5 (256 groups, FP64) the step is latency:
 // with every block of the grid reducing and arriving, and block 0 summing
 // the pending rho first, the kernel took 13.3 and 21.2 us (under ncu), and
@@ -1509,8 +1512,6 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     const long long nchunk = (ngroups + 31) / 32;
     const bool spare = known || nchunk < (long long)gridDim.x;
     const unsigned active = known ? a.active : spare ? (unsigned)nchunk : gridDim.x;   // blocks with groups
-    const unsigned arrivals = active + (spare ? 1u : 0u);
-    if (blockIdx.x >= arrivals) return;
     // the step's record and the new state (one thread)
     auto publish = [&]() {
         st->rho_nblk = active;
@@ -1549,11 +1550,15 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     auto arrive = [&]() {
         if (known) return;
         __syncthreads();
-        if (threadIdx.x == 0 && atom_add_acq_rel_gpu(P.fin_count, 1u) == arrivals - 1) {
+        if (threadIdx.x == 0 && atom_add_acq_rel_gpu(P.fin_count, 1u) == gridDim.x - 1) {
             if (__ldcg(&st->err)) *P.fin_count = 0;   // a failed step is not published
             else publish();
         }
     };
+    if (blockIdx.x > active) {   // (state read from the device: a block without a chunk)
+        arrive();
+        return;
+    }
     if (blockIdx.x == active) {   // the spare block: the previous step's rho
         if (known) {
             pdl_wait();
