@@ -158,6 +158,14 @@ __device__ __forceinline__ double2 amp_of(const WParams &P, const void *amps, un
     return static_cast<const double2 *>(amps)[i];
 }
 
+// Whether the propagation has failed, the same answer for every thread of the
+// block: other blocks of a kernel may raise the error while this one reads it,
+// and threads that left alone would leave the others' shared scans without
+// their part.  Every thread of the block calls it.
+__device__ __forceinline__ bool failed_block(const WState *st) {
+    return __syncthreads_or(*(const volatile unsigned *)&st->err != 0u) != 0;
+}
+
 // The part of the table that a step of n paths uses: two slots per path at
 // most (at least a page), so that a small step stays near the L2.
 __device__ __forceinline__ unsigned long long table_slots(const WParams &P, unsigned long long n) {
@@ -171,7 +179,7 @@ __global__ void __launch_bounds__(kWThreads) k_w_insert(WParams P) {
     __shared__ unsigned s_wc[kWThreads / 32];
     __shared__ unsigned long long s_base;
     WState *st = P.st;
-    if (st->err) return;
+    if (failed_block(st)) return;
     const int in = (int)(st->t & 1);
     const unsigned long long n = st->n_cur, slots = table_slots(P, n);
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
@@ -221,7 +229,7 @@ __global__ void __launch_bounds__(kWThreads) k_w_insert(WParams P) {
         __syncthreads();
         if (claimed) {
             const unsigned long long g = s_base + s_wc[warp] + __popc(cm & ((1u << lane) - 1u));
-            if ((long long)g < P.max_groups) P.groups[g] = (unsigned)h;
+            if (g < (unsigned long long)P.max_groups) P.groups[g] = (unsigned)h;
             else atomicOr(&st->err, kWErrGroups);
         }
         __syncthreads();   // s_wc and s_base are rewritten in the next round
@@ -296,7 +304,7 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
     unsigned short *s_list = reinterpret_cast<unsigned short *>(s_par + kWThreads);
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     double2 *part = P.rho_part + (size_t)blockIdx.x * MM;
-    if (st->err) return;
+    if (failed_block(st)) return;
     const unsigned long long t = st->t, tn = t + 1;
     const int in = (int)(t & 1), outp = (int)(tn & 1);
     const unsigned long long ng = merge ? st->n_groups : st->n_cur;
@@ -547,7 +555,7 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
             __syncthreads();
             if (kept) {
                 const unsigned long long o = s_base + s_wc[warp] + __popc(km & ((1u << lane) - 1u));
-                if ((long long)o >= P.max_paths) {
+                if (o >= (unsigned long long)P.max_paths) {
                     atomicOr(&st->err, kWErrPaths);
                 } else {
                     P.klo[outp][o] = s_lo[src] | (unsigned long long)code;
