@@ -308,6 +308,14 @@ __device__ __forceinline__ void raise_err(DevState *st, unsigned int bit) {
     atomicOr(&st->err, bit);
 }
 
+// Whether the propagation has failed, the same answer for every thread of the
+// block: other blocks of a kernel may raise the error while this one reads it,
+// and threads that left alone would leave the block's barriers and shared
+// counters without their part.  Every thread of the block calls it.
+__device__ __forceinline__ bool failed_block(const DevState *st) {
+    return __syncthreads_or(*(const volatile unsigned *)&st->err != 0u) != 0;
+}
+
 // Block-wide append: exclusive offset of each thread's cnt items within the
 // block and the block's base in a global array, with one atomicAdd on the
 // global cursor per block.  All threads of the block must call it.
@@ -475,7 +483,7 @@ __device__ __forceinline__ void phase_tiebreak(const Params &P, unsigned long lo
 template <typename Amp>
 __global__ void __launch_bounds__(kInsertThreads) k_insert(Params P) {
     DevState *st = P.st;
-    if (st->err) return;
+    if (failed_block(st)) return;
     const unsigned long long t = st->t, tn = t + 1, n = st->n_cur;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->ext_t = t;
@@ -1264,7 +1272,7 @@ __device__ __forceinline__ void finalize_single(const Params &P, unsigned long l
 template <int M, bool C64, bool BATCH>
 __global__ void __launch_bounds__(kExpandThreads) k_expand(Params P) {
     DevState *st = P.st;
-    if (st->err) return;
+    if (failed_block(st)) return;
     const unsigned long long t = st->ext_t, tn = t + 1;
     const bool merge = tn >= (unsigned long long)P.dkmax;
     const unsigned long long n = merge ? st->cnt_groups[tn % 3] : st->ext_n;
@@ -1356,7 +1364,7 @@ __global__ void __launch_bounds__(kPersistThreads) k_step_persistent(Params P, i
     using Amp = typename Expander<M, C64>::AmpT;
     DevState *st = P.st;
     const int nblk = (int)gridDim.x;
-    unsigned err = *(volatile unsigned *)&st->err;
+    unsigned err = failed_block(st);
     unsigned long long t = st->t;
     unsigned long long n_in = st->n_cur;
     unsigned long long prev_groups = 0, prev_out = 0;
@@ -1961,7 +1969,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     const unsigned long long t = tn_host ? tn_host - 1 : __ldcg(&st->t), tn = t + 1;
     // an earlier error, or launched behind the regular kernel, which just took
     // this step (its new t + 1)
-    if (__ldcg(&st->err) || ((flags & kFlagAfterRegular) && __ldcg(&st->reg_done) == tn)) {
+    if (failed_block(st) || ((flags & kFlagAfterRegular) && __ldcg(&st->reg_done) == tn)) {
         if constexpr (!BATCH) cp_async_wait_all();
         return;
     }
@@ -3186,7 +3194,7 @@ __device__ __forceinline__ unsigned long long compress_masked(const Params &P, u
 template <int M, bool C64>
 __global__ void __launch_bounds__(kExpandThreads) k_post_expand(Params P) {
     DevState *st = P.st;
-    if (st->err) return;
+    if (failed_block(st)) return;
     const unsigned long long t = st->t, tn = t + 1;
     phase_expand<M, C64, kExpandThreads, false>(P, t, st->n_cur, false, &st->cnt_out[tn % 3], rho_part_of(P, tn, M * M),
                                                 P.ckeys, P.camps);
