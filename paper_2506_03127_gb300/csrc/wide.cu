@@ -38,7 +38,13 @@ namespace {
 
 constexpr int kWMaxM = 8, kWMaxDk = 16, kWMaxMM = 64;
 constexpr int kWThreads = 256;
-constexpr int kWProbe = 64;
+// Probes before the table counts as full.  Half of the slots in use are
+// allowed (max_groups groups, or as many groups as paths in table_slots):
+// there the longest probe of n keys is about ln(n) / 0.19, 72 at 1e6 and 103
+// at 4e8 (79 met with 1.7e7), and none reaches 1024; every kWProbeCheck probes
+// a path asks whether the step has failed, so that more groups than the table
+// holds end soon.
+constexpr int kWProbe = 1024, kWProbeCheck = 64;
 constexpr int kWMaxRuns = 16;       // runs of consecutive positions, each within one word of eight
 constexpr int kWMaxBlocks = 2048;   // blocks of the expansion (partials of rho)
 constexpr unsigned long long kWEmpty = ~0ull;
@@ -204,6 +210,7 @@ __global__ void __launch_bounds__(kWThreads) k_w_insert(WParams P) {
                     }
                 }
                 if (cur == gk) break;
+                if (probe % kWProbeCheck == kWProbeCheck - 1 && *(volatile unsigned *)&st->err) probe = kWProbe - 1;
             }
             if (probe == kWProbe) {
                 atomicOr(&st->err, kWErrProbe);
