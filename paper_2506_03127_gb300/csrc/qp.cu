@@ -3974,6 +3974,8 @@ struct qp_ctx {
     bool graph_dirty = true;           // none of them is current
     bool reg_track = false;            // path counts of an unfiltered stream propagation known on the host (step_kind)
     bool use_graph = true;
+    bool host_index = true;            // the host knows the step index: false once steps were recorded into a caller's
+                                       // graph, whose replays it does not see
     int64_t host_t = 0;                // steps enqueued since qp_set_rho0 (set from the device at every state read)
     void *hpin = nullptr;              // pinned host staging for rho reads (state + rows)
     size_t hpin_bytes = 0;
@@ -4193,15 +4195,16 @@ RegArgs known_counts(const qp_ctx *c, int64_t tn) {
 }
 
 // One step of the stream engine (regular kernel: events 0 -> 1, tile kernel:
-// events 2 -> 3).
+// events 2 -> 3).  Steps that read their index from the device (tn = 0) may
+// be under a caller's capture and are launched the plain way.
 template <int M, typename Amp>
 cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind, int64_t tn) {
     constexpr bool C64 = sizeof(Amp) == sizeof(float2);
-    const bool after_regular = kind == kStepBoth && c->P.reg_fill && M < 4;
+    const bool after_regular = kind == kStepBoth && c->P.reg_fill && M < 4, dep = ev == nullptr && tn != 0;
     if (ev) cudaEventRecord(ev[0], c->stream);
     if constexpr (M < 4) {
         if (kind == kStepRegular || after_regular) {
-            cudaError_t e = launch_stream_regular<M, C64>(c, ev == nullptr, kind == kStepRegular ? known_counts(c, tn) : RegArgs{0, 0, 0, 0u});
+            cudaError_t e = launch_stream_regular<M, C64>(c, dep, kind == kStepRegular ? known_counts(c, tn) : RegArgs{0, 0, 0, 0u});
             if (e != cudaSuccess) return e;
         }
     }
@@ -4211,7 +4214,7 @@ cudaError_t launch_stream_t(qp_ctx *c, cudaEvent_t *ev, StepKind kind, int64_t t
     }
     cudaError_t e = cudaSuccess;
     if (c->P.n_inst > 1) e = launch_stream_batch(c, 1, false);
-    else if (kind != kStepRegular) e = launch_stream_tile(c, after_regular, ev == nullptr, tn);
+    else if (kind != kStepRegular) e = launch_stream_tile(c, after_regular, dep, tn);
     if (e != cudaSuccess) return e;
     if (ev) {
         cudaEventRecord(ev[3], c->stream);
@@ -4255,7 +4258,7 @@ cudaError_t launch_post_t(qp_ctx *c, cudaEvent_t *ev) {
     return cudaGetLastError();
 }
 
-// tn: the step where the host launches it, 0 in a graph
+// tn: the step where the host launches it and knows its index, else 0
 cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev, StepKind kind, int64_t tn) {
     const bool c64 = c->cfg.precision == QP_C64;
     if (c->P.post) {
@@ -4277,6 +4280,12 @@ cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev, StepKind kind, int64_t tn) {
         case 3: return c64 ? launch_step_t<3, float2>(c, ev) : launch_step_t<3, double2>(c, ev);
         default: return c64 ? launch_step_t<4, float2>(c, ev) : launch_step_t<4, double2>(c, ev);
     }
+}
+
+// Step tn by the host's count, outside a graph of the context's own.
+cudaError_t launch_next(qp_ctx *c, cudaEvent_t *ev, int64_t tn) {
+    if (!c->host_index) return launch_step(c, ev, kStepBoth, 0);
+    return launch_step(c, ev, step_kind(c, tn), tn);
 }
 
 template <int M, bool C64>
@@ -4871,18 +4880,19 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
     // qp_set_rho0 (headline model, 160 steps: 14.5 us per step, in graphs of
     // eight 14.9).  A replay would repeat what the host passed: a stream under
     // capture is refused, as it is where steps run as graphs; with graphs
-    // switched off (QP_NO_GRAPH) the captured kernels read the device state.
+    // switched off (QP_NO_GRAPH) the captured kernels read the device state,
+    // and so does every later step of the context.
     // Batches do the same unless several steps go into a graph; the other
     // engines go into graphs (the table engine's kernels are 6 % slower one by
     // one).
     const bool single = c->use_stream && (c->P.n_inst == 1 || c->graph_steps == 1);
-    bool captured = false;
     if (single && c->stream) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         QP_CUDA(c, cudaStreamIsCapturing(c->stream, &cap));
-        captured = cap != cudaStreamCaptureStatusNone;
+        const bool captured = cap != cudaStreamCaptureStatusNone;
         if (captured && c->use_graph && !(c->use_persistent && c->P.n_inst > 1))
             return fail(c, QP_ERR_CUDA, "qp_step: the stream is being captured");
+        if (captured) c->host_index = false;
     }
     const int64_t t0 = c->host_t;
     c->host_t += nsteps;
@@ -4899,7 +4909,7 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
     if (single || !c->use_graph) {
         for (int s = 0; s < nsteps; ++s) {
             const int64_t tn = t0 + s + 1;
-            const cudaError_t e = launch_step(c, nullptr, captured ? kStepBoth : step_kind(c, tn), captured ? 0 : tn);
+            const cudaError_t e = launch_next(c, nullptr, tn);
             if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
         }
         return QP_OK;
@@ -5168,7 +5178,7 @@ qp_status qp_profile_steps(qp_ctx *c, int nsteps, double *kernel_ms, int nk) {
     qp_status st = QP_OK;
     for (int s = 0; s < nsteps && st == QP_OK; ++s) {
         k_delay<<<1, 1, 0, c->stream>>>(50000ull);
-        cudaError_t e = launch_step(c, ev, step_kind(c, c->host_t + 1), c->host_t + 1);
+        cudaError_t e = launch_next(c, ev, c->host_t + 1);
         ++c->host_t;
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[kStepKernels]);
         if (e != cudaSuccess) {
