@@ -373,6 +373,13 @@ qp_status qp_import_paths(qp_ctx *ctx, const uint64_t *d_keys, const void *d_amp
  * the running propagation is not on the stream engine.                    */
 qp_status qp_test_stall_lookback(qp_ctx *ctx);
 
+/* Test hook for a launch that fails in the middle of qp_step: after `after`
+ * more steps launched one by one (stream engine, single problems) the next
+ * one reports a launch failure on the host without being launched.  qp_step
+ * returns QP_ERR_CUDA, the steps before it stay enqueued and the propagation
+ * goes on from them at the next qp_step.                                    */
+qp_status qp_test_fail_launch(qp_ctx *ctx, int after);
+
 /* Test hook: out[i] = in[i] widened from FP32 to FP64 exactly as the step
  * kernels widen FP32 amplitudes and partial sums before FP64 arithmetic
  * (IEEE-754 field arithmetic in integer registers, all classes: zeros,

@@ -91,6 +91,7 @@ def _load():
         "qp_autotune": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_void_p, _dp]),
         "qp_test_stall_barrier": (ctypes.c_int, [ctypes.c_void_p]),
         "qp_test_stall_lookback": (ctypes.c_int, [ctypes.c_void_p]),
+        "qp_test_fail_launch": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
         "qp_Q_from_bath": (ctypes.c_int, [ctypes.POINTER(qp_bath), ctypes.c_double, ctypes.c_int, _dp, _dp]),
         "qp_set_end_points": (ctypes.c_int, [ctypes.c_void_p, _dp, _dp, ctypes.c_int]),
         "qp_partition_paths": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p,
@@ -297,6 +298,10 @@ def qp_set_end_points(ctx, Qh):
 
 def qp_test_stall_lookback(ctx):
     check(lib.qp_test_stall_lookback(ctx), ctx)
+
+
+def qp_test_fail_launch(ctx, after: int):
+    check(lib.qp_test_fail_launch(ctx, after), ctx)
 
 
 def qp_partition_paths(ctx, n_ranks: int, d_keys: int, d_amps: int, cap: int):

@@ -3975,7 +3975,8 @@ struct qp_ctx {
     bool reg_track = false;            // path counts of an unfiltered stream propagation known on the host (step_kind)
     bool use_graph = true;
     bool host_index = true;            // the host knows the step index: false once steps were recorded into a caller's
-                                       // graph, whose replays it does not see
+                                       // graph, whose replays it does not see, or a step was launched in part
+    int fail_after = -1;               // test hook: launches until one fails on the host (-1: none)
     int64_t host_t = 0;                // steps enqueued since qp_set_rho0 (set from the device at every state read)
     void *hpin = nullptr;              // pinned host staging for rho reads (state + rows)
     size_t hpin_bytes = 0;
@@ -4284,8 +4285,10 @@ cudaError_t launch_step(qp_ctx *c, cudaEvent_t *ev, StepKind kind, int64_t tn) {
 
 // Step tn by the host's count, outside a graph of the context's own.
 cudaError_t launch_next(qp_ctx *c, cudaEvent_t *ev, int64_t tn) {
-    if (!c->host_index) return launch_step(c, ev, kStepBoth, 0);
-    return launch_step(c, ev, step_kind(c, tn), tn);
+    if (c->fail_after >= 0 && c->fail_after-- == 0) return cudaErrorLaunchFailure;
+    const cudaError_t e = c->host_index ? launch_step(c, ev, step_kind(c, tn), tn) : launch_step(c, ev, kStepBoth, 0);
+    if (e != cudaSuccess) c->host_index = false;
+    return e;
 }
 
 template <int M, bool C64>
@@ -4894,23 +4897,25 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
             return fail(c, QP_ERR_CUDA, "qp_step: the stream is being captured");
         if (captured) c->host_index = false;
     }
-    const int64_t t0 = c->host_t;
-    c->host_t += nsteps;
+    // (host_t follows what was enqueued: a launch that fails leaves the steps
+    // before it)
     if (c->use_persistent && !c->use_stream && !c->P.post) {
         const cudaError_t e = launch_persistent(c, nsteps);
         if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("persistent launch: ") + cudaGetErrorString(e));
+        c->host_t += nsteps;
         return QP_OK;
     }
     if (c->use_persistent && c->use_stream && c->P.n_inst > 1) {   // batched stream engine: all steps, one launch
         const cudaError_t e = launch_stream_batch(c, nsteps, true);
         if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("persistent launch: ") + cudaGetErrorString(e));
+        c->host_t += nsteps;
         return QP_OK;
     }
     if (single || !c->use_graph) {
         for (int s = 0; s < nsteps; ++s) {
-            const int64_t tn = t0 + s + 1;
-            const cudaError_t e = launch_next(c, nullptr, tn);
+            const cudaError_t e = launch_next(c, nullptr, c->host_t + 1);
             if (e != cudaSuccess) return fail(c, QP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
+            ++c->host_t;
         }
         return QP_OK;
     }
@@ -4927,6 +4932,7 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
         }
         QP_CUDA(c, cudaGraphLaunch(g, c->stream));
         s += many ? c->graph_steps : 1;
+        c->host_t += many ? c->graph_steps : 1;
     }
     return QP_OK;
 }
@@ -5179,7 +5185,7 @@ qp_status qp_profile_steps(qp_ctx *c, int nsteps, double *kernel_ms, int nk) {
     for (int s = 0; s < nsteps && st == QP_OK; ++s) {
         k_delay<<<1, 1, 0, c->stream>>>(50000ull);
         cudaError_t e = launch_next(c, ev, c->host_t + 1);
-        ++c->host_t;
+        if (e == cudaSuccess) ++c->host_t;
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[kStepKernels]);
         if (e != cudaSuccess) {
             st = fail(c, QP_ERR_CUDA, std::string("profile: ") + cudaGetErrorString(e));
@@ -5371,6 +5377,13 @@ qp_status qp_test_stall_barrier(qp_ctx *c) {
     const unsigned int poison = 0x40000000u;
     QP_CUDA(c, cudaMemcpyAsync(&c->P.st->bar_count, &poison, sizeof(poison), cudaMemcpyHostToDevice, c->stream));
     QP_CUDA(c, cudaStreamSynchronize(c->stream));
+    return QP_OK;
+}
+
+qp_status qp_test_fail_launch(qp_ctx *c, int after) {
+    if (!c) return QP_ERR_ARG;
+    if (after < 0) return fail(c, QP_ERR_ARG, "after < 0");
+    c->fail_after = after;
     return QP_OK;
 }
 
