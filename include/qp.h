@@ -256,7 +256,8 @@ qp_status qp_set_mask(qp_ctx *ctx, const int *positions, int n);
 
 /* Restart the propagation at t = 0 from rho(0) (M*M row-major, Hermitian):
  * one stored path per nonzero element.  im may be NULL (real rho0).  Clears
- * any device error state.  Requires qp_set_eta to have been called.         */
+ * any device error state.  Requires qp_set_eta to have been called.  Refused
+ * (QP_ERR_CUDA) on a stream under capture.                                  */
 qp_status qp_set_rho0(qp_ctx *ctx, const double *rho0_re, const double *rho0_im);
 
 /* Enqueue nsteps propagation steps on the context's stream (asynchronous;

@@ -4002,6 +4002,15 @@ void drop_graphs(qp_ctx *c) {
     c->graph1 = c->graph = nullptr;
 }
 
+// Whether the context's stream is under a caller's capture (the default
+// stream cannot be).
+cudaError_t stream_captured(const qp_ctx *c, bool *yes) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = c->stream ? cudaStreamIsCapturing(c->stream, &cap) : cudaSuccess;
+    *yes = cap != cudaStreamCaptureStatusNone;
+    return e;
+}
+
 constexpr int kStepKernels = 4;
 
 // Launch one step; if ev is given, record ev[k] before kernel k and
@@ -4799,6 +4808,11 @@ qp_status qp_set_rho0(qp_ctx *c, const double *re, const double *im) {
     if (!c) return QP_ERR_ARG;
     if (!re) return fail(c, QP_ERR_ARG, "rho0 required");
     if (!c->have_eta) return fail(c, QP_ERR_STATE, "qp_set_eta must come before qp_set_rho0");
+    // under a capture the state would be recorded instead of set, while the
+    // context took it for set
+    bool captured = false;
+    QP_CUDA(c, stream_captured(c, &captured));
+    if (captured) return fail(c, QP_ERR_CUDA, "qp_set_rho0: the stream is being captured");
     const int M = c->cfg.M, MM = M * M, NI = c->P.n_inst;
     const int bs = c->P.bs;
     InitArgs ia{};
@@ -4889,10 +4903,9 @@ qp_status qp_step(qp_ctx *c, int nsteps) {
     // engines go into graphs (the table engine's kernels are 6 % slower one by
     // one).
     const bool single = c->use_stream && (c->P.n_inst == 1 || c->graph_steps == 1);
-    if (single && c->stream) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        QP_CUDA(c, cudaStreamIsCapturing(c->stream, &cap));
-        const bool captured = cap != cudaStreamCaptureStatusNone;
+    if (single) {
+        bool captured = false;
+        QP_CUDA(c, stream_captured(c, &captured));
         if (captured && c->use_graph && !(c->use_persistent && c->P.n_inst > 1))
             return fail(c, QP_ERR_CUDA, "qp_step: the stream is being captured");
         if (captured) c->host_index = false;

@@ -44,3 +44,30 @@ def test_capture_replay_step(M, dkmax, mask, theta, precision, monkeypatch):
     assert np.abs(rho - ref.rho).max() <= (1e-10 if precision == "fp64" else 1e-5 * max(1.0, np.abs(ref.rho).max()))
     if precision == "fp64" and not any(s.near_tie or s.near_theta for s in ref.stats):
         assert [(r[1], r[3]) for r in st] == [(o.groups, o.kept) for o in ref.stats]
+
+
+@pytest.mark.parametrize("engine", ["stream", "hash"])
+def test_a_start_under_capture_is_refused(engine):
+    """qp_set_rho0 on a stream under capture sets nothing: it is refused, the
+    capture stays valid and the running propagation goes on."""
+    import torch
+    from paper_2506_03127_gb300 import Propagator, abi
+    M, dkmax, T = 2, 5, 9
+    c = W.random_case(58, M, dkmax)
+    p = Propagator(M, dkmax, c["dt"], c["q"], c["hs"], 0.0, "fp64", engine, max_paths=1 << 14)
+    p.set_eta(c["eta"])
+    p.set_mask(None)
+    p.set_rho0(c["rho0"])
+    p.step(4)
+    p.sync()
+    x, g = torch.zeros(1, device="cuda"), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=p.stream):
+        x.add_(1)
+        with pytest.raises(abi.QPError) as e:
+            p.set_rho0(np.eye(2) / 2)
+        assert e.value.status == abi.QP_ERR_CUDA
+    p.step(T - 4)
+    rho = p.rho(0, T + 1)
+    p.close()
+    ref = iquapi.propagate(M, c["q"], c["hs"], c["dt"], c["eta"], dkmax, None, 0.0, c["rho0"], T)
+    assert np.abs(rho - ref.rho).max() <= 1e-10
