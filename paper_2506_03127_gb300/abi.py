@@ -338,7 +338,7 @@ def qp_export_paths(ctx, cap: int):
 
 
 def qp_profile_steps(ctx, nsteps: int) -> np.ndarray:
-    """Per-kernel milliseconds summed over nsteps steps (insert, tie-break, expand, finalise)."""
+    """Per-kernel milliseconds summed over nsteps steps (the kernels: qp_profile_steps in include/qp.h)."""
     ms = np.zeros(4)
     check(lib.qp_profile_steps(ctx, nsteps, _ptr(ms), 4), ctx)
     return ms

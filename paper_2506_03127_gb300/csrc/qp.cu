@@ -5196,6 +5196,16 @@ qp_status qp_profile_steps(qp_ctx *c, int nsteps, double *kernel_ms, int nk) {
     for (int k = 0; k <= kStepKernels; ++k) QP_CUDA(c, cudaEventCreate(&ev[k]));
     qp_status st = QP_OK;
     for (int s = 0; s < nsteps && st == QP_OK; ++s) {
+        // intervals without a kernel in this step hold only event overhead
+        const StepKind kind = c->host_index ? step_kind(c, c->host_t + 1) : kStepBoth;
+        bool timed[kStepKernels] = {true, true, true, true};
+        if (c->use_stream) {
+            timed[0] = kind == kStepRegular || (kind == kStepBoth && c->P.reg_fill && c->cfg.M < 4);
+            timed[1] = timed[3] = false;
+            timed[2] = kind != kStepRegular;
+        } else if (!c->P.post && c->P.n_inst == 1) {
+            timed[3] = false;   // the extension finalises the step
+        }
         k_delay<<<1, 1, 0, c->stream>>>(50000ull);
         cudaError_t e = launch_next(c, ev, c->host_t + 1);
         if (e == cudaSuccess) ++c->host_t;
@@ -5205,9 +5215,7 @@ qp_status qp_profile_steps(qp_ctx *c, int nsteps, double *kernel_ms, int nk) {
             break;
         }
         for (int k = 0; k < kStepKernels && k < nk; ++k) {
-            // stream engine: intervals without a kernel (1, 3, and 0 where
-            // no regular map is launched) hold only event overhead
-            if (c->use_stream && (k == 1 || k == 3 || (k == 0 && !(c->cfg.M == 2 && c->P.reg_fill)))) continue;
+            if (!timed[k]) continue;
             float ms = 0.f;
             cudaEventElapsedTime(&ms, ev[k], ev[k + 1]);
             kernel_ms[k] += ms;
