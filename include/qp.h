@@ -164,7 +164,9 @@ typedef struct {
     int insert_blocks_per_sm;  /* pre-merge kernels (graph mode)                 */
     int expand_blocks_per_sm;  /* extension kernel (graph mode)                  */
     int persistent_blocks;     /* grid of the persistent kernel                  */
-    int graph_steps;           /* steps captured per CUDA graph launch           */
+    int graph_steps;           /* steps captured per CUDA graph launch (no effect
+                                  on single problems of the stream engine, whose
+                                  steps are launched one by one)                 */
     int table_log2;            /* active merge-table slots = 2^table_log2        */
     int engine;                /* engine of the running propagation (QP_ENGINE_HASH
                                   or QP_ENGINE_STREAM; read-only, set at
