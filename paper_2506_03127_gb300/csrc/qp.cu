@@ -2014,7 +2014,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     // runs of more than kOwnRun members that start in the tile, and the warps'
     // sums of a run that the whole block adds
     __shared__ int s_nlong, s_long[S / kOwnRun + 2];
-    __shared__ typename X::AccT s_lsum[NW][NX], s_lerr[C64 ? NW : 1][C64 ? NX : 1];
+    __shared__ double2 s_lsum[NW][NX];
     __shared__ WT s_lwm[NW][NX];
     __shared__ int s_lbfail;   // the tile's look-back gave up (timeout, or another block's error)
     const double tie_d = 1.0 - P.tie_rel;   // R4 window, once per thread
@@ -2481,14 +2481,15 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
         // runs of more than kOwnRun members (mostly at the first merge, when
         // the whole filled window collapses onto P'): up to kWarpRun members
         // by one warp, longer ones by the block, the members dealt to the
-        // lanes.  Pass 1 adds them per sub-group (C64: FP32 TwoSum pairs
-        // merged error-free and rounded once, FP64: FP64) and takes the
-        // largest weights, pass 2 elects the representatives.  Members past
-        // the tile and its prefetch are read from global memory.  (Shared FP64
-        // atomics, a compare-and-swap loop under contention, with one warp
-        // for the members past the tile end, took 1.42 ms for the first merge
-        // of the headline model (7.7e5 paths, c64) and 7.5 ms for the chain's
-        // (3.9e7 paths).)
+        // lanes.  Pass 1 adds them per sub-group in FP64 (C64: rounded once)
+        // and takes the largest weights, pass 2 elects the representatives.
+        // Members past the tile and its prefetch are read from global memory.
+        // The first merge of the headline model (7.7e5 paths, c64) takes
+        // 0.14 ms and the chain's (3.9e7 paths) 2.18 ms.  (FP32 pairs took 0.08
+        // and 1.90 ms, but with so many members they lose bits of sums that
+        // nearly cancel; shared FP64 atomics, a compare-and-swap loop under
+        // contention, with one warp for the members past the tile end, 1.42
+        // and 7.5 ms.)
         const bool any_runs = __syncthreads_or(any_long);
         if (any_runs) {
             if (threadIdx.x == 0) s_nlong = 0;
@@ -2500,7 +2501,6 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             __syncthreads();
             const int nlong = s_nlong;
             const int in_tile = cnt + (cnt == St ? (int)s_ra_n : 0);   // entries in shared memory
-            using AccT = typename X::AccT;
             // this lane's members m0, m0 + step, ... of run g
             auto each = [&](int g, int m0, int step, auto &&f) {
                 const int b0 = s_seg[g];
@@ -2522,11 +2522,10 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 for (; i < b1; i += step) f(__ldcg(kin + e0 + i), __ldcg(ain + e0 + i));
             };
             // warp sums and largest weights per sub-group (in every lane)
-            auto warp_sums = [&](int g, int m0, int step, AccT *sh, AccT *se, WT *wmx) {
+            auto warp_sums = [&](int g, int m0, int step, double2 *sh, WT *wmx) {
 #pragma unroll
                 for (int x = 0; x < NX; ++x) {
                     sh[x].x = sh[x].y = 0;
-                    se[x].x = se[x].y = 0;
                     wmx[x] = 0;
                 }
                 each(g, m0, step, [&](unsigned long long key, const AmpT &a) {
@@ -2535,13 +2534,8 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
 #pragma unroll
                     for (int x = 0; x < NX; ++x)
                         if (NX == 1 || xv == (unsigned)x) {
-                            if constexpr (C64) {
-                                two_sum_acc(sh[x].x, se[x].x, a.x);
-                                two_sum_acc(sh[x].y, se[x].y, a.y);
-                            } else {
-                                sh[x].x += a.x;
-                                sh[x].y += a.y;
-                            }
+                            sh[x].x += to_d(a.x);
+                            sh[x].y += to_d(a.y);
                             wmx[x] = wb > wmx[x] ? wb : wmx[x];
                         }
                 });
@@ -2549,16 +2543,8 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 for (int x = 0; x < NX; ++x) {
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) {
-                        if constexpr (C64) {
-                            const float bx = __shfl_xor_sync(0xffffffffu, sh[x].x, o), by = __shfl_xor_sync(0xffffffffu, sh[x].y, o);
-                            se[x].x += __shfl_xor_sync(0xffffffffu, se[x].x, o);
-                            se[x].y += __shfl_xor_sync(0xffffffffu, se[x].y, o);
-                            two_sum_acc(sh[x].x, se[x].x, bx);
-                            two_sum_acc(sh[x].y, se[x].y, by);
-                        } else {
-                            sh[x].x += __shfl_xor_sync(0xffffffffu, sh[x].x, o);
-                            sh[x].y += __shfl_xor_sync(0xffffffffu, sh[x].y, o);
-                        }
+                        sh[x].x += __shfl_xor_sync(0xffffffffu, sh[x].x, o);
+                        sh[x].y += __shfl_xor_sync(0xffffffffu, sh[x].y, o);
                         const WT w = __shfl_xor_sync(0xffffffffu, wmx[x], o);
                         wmx[x] = w > wmx[x] ? w : wmx[x];
                     }
@@ -2591,25 +2577,25 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                     return g;
                 }
             };
-            auto put_sum = [&](int sl, const AccT &sh, const AccT &se) {
-                if constexpr (C64) s_gS[sl] = make_float2(sh.x + se.x, sh.y + se.y);
-                else s_gS[sl] = make_double2(sh.x, sh.y);
+            auto put_sum = [&](int sl, const double2 &sh) {
+                if constexpr (C64) s_gS[sl] = to_f2(sh);
+                else s_gS[sl] = sh;
             };
             auto length = [&](int g) { return (g + 1 < nseg ? (long long)s_seg[g + 1] : ahead) - s_seg[g]; };
             for (int l = (int)warp; l < nlong; l += NW) {
                 const int g = s_long[l];
                 if (length(g) > kWarpRun) continue;
-                AccT sh[NX], se[NX];
+                double2 sh[NX];
                 WT wmx[NX];
                 unsigned long long kmin[NX];
-                warp_sums(g, (int)lane, 32, sh, se, wmx);
+                warp_sums(g, (int)lane, 32, sh, wmx);
                 warp_reps(g, (int)lane, 32, wmx, kmin);
                 if (lane == 0) {
 #pragma unroll
                     for (int x = 0; x < NX; ++x) {
                         const int sl = slot(g, x);
                         if (sl >= 0) {
-                            put_sum(sl, sh[x], se[x]);
+                            put_sum(sl, sh[x]);
                             s_grep[sl] = kmin[x];
                         }
                     }
@@ -2618,15 +2604,14 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             for (int l = 0; l < nlong; ++l) {   // block-uniform
                 const int g = s_long[l];
                 if (length(g) <= kWarpRun) continue;
-                AccT sh[NX], se[NX];
+                double2 sh[NX];
                 WT wmx[NX];
                 unsigned long long kmin[NX];
-                warp_sums(g, (int)threadIdx.x, NT, sh, se, wmx);
+                warp_sums(g, (int)threadIdx.x, NT, sh, wmx);
                 if (lane == 0) {
 #pragma unroll
                     for (int x = 0; x < NX; ++x) {
                         s_lsum[warp][x] = sh[x];
-                        if constexpr (C64) s_lerr[warp][x] = se[x];
                         s_lwm[warp][x] = wmx[x];
                     }
                 }
@@ -2636,17 +2621,11 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 }
                 __syncthreads();
 #pragma unroll
-                for (int x = 0; x < NX; ++x) {   // every thread: the warps in order
+                for (int x = 0; x < NX; ++x) {   // the warps in order: the sums by one thread, the weights by all
                     sh[x] = s_lsum[0][x];
-                    if constexpr (C64) se[x] = s_lerr[0][x];
                     wmx[x] = s_lwm[0][x];
                     for (int w = 1; w < NW; ++w) {
-                        if constexpr (C64) {
-                            se[x].x += s_lerr[w][x].x;
-                            se[x].y += s_lerr[w][x].y;
-                            two_sum_acc(sh[x].x, se[x].x, s_lsum[w][x].x);
-                            two_sum_acc(sh[x].y, se[x].y, s_lsum[w][x].y);
-                        } else if (threadIdx.x == 0) {
+                        if (threadIdx.x == 0) {
                             sh[x].x += s_lsum[w][x].x;
                             sh[x].y += s_lsum[w][x].y;
                         }
@@ -2658,7 +2637,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
                 for (int x = 0; x < NX; ++x) {
                     const int sl = slot(g, x);
                     if (sl < 0) continue;
-                    if (threadIdx.x == 0) put_sum(sl, sh[x], se[x]);
+                    if (threadIdx.x == 0) put_sum(sl, sh[x]);
                     if (lane == 0 && kmin[x] != kEmpty) atomicMin(&s_grep[sl], kmin[x]);
                 }
                 __syncthreads();
