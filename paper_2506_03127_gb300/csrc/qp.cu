@@ -2945,36 +2945,40 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
             }
         }
         if constexpr (kTileAcc) if (!kColSum || ngroups > Lay::NSTG) {
-            // the tile's rho(t+1): warp sums by halving (Kahan terms as the
-            // pairs' second words), each component in one lane.  Batches add
-            // it to the instance's block sums (shared FP64 atomics), single
-            // problems to the warp's pair (TwoSum).  (Batches widened every
-            // lane's value and reduced in FP64, 40 additions of 16 cycles per
-            // warp and tile: half of the FP64 pipe's time in the sweep)
+            // the tile's rho(t+1): warp sums by halving, each component in one
+            // lane, which batches add to the instance's block sums (shared
+            // FP64 atomics), single problems to the warp's pair (TwoSum).
+            // FP32 pairs beside column sums, which are pairs too; FP64 in
+            // batches with M >= 3, as before: a lane has one or two children
+            // of a tile there, whose FP64 sum is exact but for 2^-53
+            // (pairs: off by 1e-15 instead of 1e-17 in rho of the chain).
             constexpr int V = MM <= 4 ? 8 : 32;
+            constexpr bool kPairs = kColSum;
             const int idx = rs_index<V>();
             const bool mine = idx < 2 * MM && (lane & (32 / V - 1)) == 0u;
-            typename std::conditional<C64, float, double>::type sv[V], ev[C64 ? V : 1];
+            typename std::conditional<kPairs, float, double>::type sv[V], ev[kPairs ? V : 1];
 #pragma unroll
             for (int k = 0; k < V; ++k) {
                 sv[k] = 0;
-                if (k < 2 * MM) sv[k] = (k & 1) ? tacc[k >> 1].y : tacc[k >> 1].x;
-                if constexpr (C64) {
-                    ev[k] = 0;
-                    if constexpr (kKahan)
-                        if (k < 2 * MM) ev[k] = (k & 1) ? -tcmp[k >> 1].y : -tcmp[k >> 1].x;
+                if constexpr (kPairs) ev[k] = 0;
+                if (k < 2 * MM) {
+                    const auto s = (k & 1) ? tacc[k >> 1].y : tacc[k >> 1].x;
+                    if constexpr (kPairs) sv[k] = s;
+                    else sv[k] = to_d(s);
+                    if constexpr (kKahan) {
+                        const auto e = (k & 1) ? -tcmp[k >> 1].y : -tcmp[k >> 1].x;
+                        if constexpr (kPairs) ev[k] = e;
+                        else sv[k] += to_d(e);
+                    }
                 }
             }
-            if constexpr (C64) warp_reduce_scatter<V>(sv, ev);
+            if constexpr (kPairs) warp_reduce_scatter<V>(sv, ev);
             else warp_reduce_scatter<V>(sv);
             if constexpr (BATCH) {
-                double *acc = reinterpret_cast<double *>(s_acc + (size_t)inst * (MM + 1));
-                if (mine) {
-                    double x;
-                    if constexpr (C64) x = f2d_exact(sv[0]) + f2d_exact(ev[0]);
-                    else x = sv[0];
-                    if (x != 0.0) atomicAdd(acc + idx, x);
-                }
+                double x;
+                if constexpr (kPairs) x = f2d_exact(sv[0]) + f2d_exact(ev[0]);
+                else x = sv[0];
+                if (mine && x != 0.0) atomicAdd(reinterpret_cast<double *>(s_acc + (size_t)inst * (MM + 1)) + idx, x);
             } else if constexpr (C64) {
                 if (mine) {
                     float2 a = reinterpret_cast<float2 *>(&s_wrho[warp][0])[idx];

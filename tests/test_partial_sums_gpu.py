@@ -1,6 +1,8 @@
 """Sums of the complex64 forms that are kept in FP64 (rounded once where they
 are stored): where an FP64 sum is exact in any order, nothing of it may be
 lost on the way."""
+import math
+
 import numpy as np
 import pytest
 
@@ -40,3 +42,37 @@ def test_group_sums_of_long_runs(mask, dkmax, odd, tile):
         p.close()
     assert np.array_equal(sets[0][0], sets[1][0])
     assert np.array_equal(sets[0][1], sets[1][1])
+
+
+def _rho_of(M, keys, amps):
+    """rho from a stored set, the sums correctly rounded."""
+    bs = max(1, (M - 1).bit_length())
+    mask = np.uint64((1 << bs) - 1)
+    a, b = (keys & mask).astype(int), ((keys >> np.uint64(bs)) & mask).astype(int)
+    rho = np.zeros((M, M), dtype=complex)
+    for i in range(M):
+        for j in range(M):
+            v = amps[(a == i) & (b == j)]
+            rho[i, j] = complex(math.fsum(v.real), math.fsum(v.imag))
+    return rho
+
+
+@pytest.mark.parametrize("dkmax,theta,steps", [(8, 1e-9, 14), (9, 1e-10, 12)])
+def test_rho_of_a_batch_of_three_level_chains(dkmax, theta, steps):
+    """rho(t) against the exact sum of the stored children.  Its elements are
+    below 1 and about two dozen FP64 additions lie between a child and rho (a
+    warp, the tiles of a block, the blocks), each rounded by at most 2^-54 of
+    either sign: 8 * 2^-54 allows for sqrt(24) of them and half as much again."""
+    from paper_2506_03127_gb300 import Propagator, eta_from_bath
+    c, n_inst = W.CHAIN3_STRUCTURED_DK12, 3
+    p = Propagator(3, dkmax, c.dt, c.q, c.hs_array(), theta, "c64", "stream", max_paths=n_inst << 23, n_inst=n_inst)
+    p.set_eta(eta_from_bath(c.bath, c.dt, dkmax))
+    p.set_mask(range(5))
+    p.set_rho0(c.rho0_array())
+    p.step(steps)
+    rho = p.rho(steps, 1)[0]
+    keys, amps = p.export_paths()
+    p.close()
+    inst = (keys >> np.uint64(4 * dkmax)).astype(int)
+    for i in range(n_inst):
+        assert np.abs(rho[i] - _rho_of(3, keys[inst == i], amps[inst == i])).max() <= 8 * 2.0 ** -54
