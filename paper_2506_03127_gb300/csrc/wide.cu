@@ -270,7 +270,7 @@ __device__ __forceinline__ float log2_d(double d) {
 
 inline size_t expand_smem(int MM, int nb, bool c64) {
     const size_t ct = c64 ? 8 : 16, lw = (size_t)MM * ((MM + 7) & ~3) * 4;
-    return (size_t)nb * 64 * 16 + (size_t)(kWThreads / 32) * MM * 16 + 2 * kWThreads * ct + 2 * kWThreads * 8 +
+    return (size_t)nb * 64 * 16 + (size_t)(kWThreads / 32) * MM * (c64 ? 24 : 16) + 2 * kWThreads * ct + 2 * kWThreads * 8 +
            ((lw + 15) & ~(size_t)15) + (size_t)MM * (kWThreads / 32) * 8 + kWThreads + (size_t)kWThreads * MM * 2;
 }
 
@@ -285,7 +285,9 @@ inline size_t expand_smem(int MM, int nb, bool c64) {
 // dealt evenly to the threads and a warp's children share their newest
 // point; each is formed once in full precision, filtered, added to rho(t)
 // (segments of equal newest point, then one lane's addition to its warp's
-// bin; C64: FP32 pairs, TwoSum) and written to a range reserved per 256
+// bin; C64: FP32 pairs with TwoSum, the bins of three words, which lose less
+// than the FP64 sums of before: with two, rho was off by up to 1e-15 instead
+// of 6e-17) and written to a range reserved per 256
 // candidates.  (Forming all 64 children twice, four lanes per group, with
 // rho from a second pass over the children took 0.88 ms per step and launch
 // at 2e6 groups, the two passes of rho and of its block sums 0.30 ms.)
@@ -302,7 +304,8 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
     const int lws = (MM + 7) & ~3;                    // row of the bound table (rows on different banks)
     float4 *s_lut = reinterpret_cast<float4 *>(s_dyn);   // [nb][64] history terms (C64: hi, lo; FP64: double2)
     float4 *s_rho = s_lut + nb * 64;                     // [NW][MM] (C64: re, err, im, err; FP64: double2)
-    CT *s_S = reinterpret_cast<CT *>(s_rho + NW * MM), *s_H = s_S + kWThreads;
+    float2 *s_rhof = reinterpret_cast<float2 *>(s_rho + NW * MM);   // C64: what is lost of the errors
+    CT *s_S = reinterpret_cast<CT *>(s_rhof + (C64 ? NW * MM : 0)), *s_H = s_S + kWThreads;
     unsigned long long *s_lo = reinterpret_cast<unsigned long long *>(s_H + kWThreads), *s_hi = s_lo + kWThreads;
     float *s_lw = reinterpret_cast<float *>(s_hi + kWThreads);
     unsigned *s_mask = reinterpret_cast<unsigned *>(s_lw + ((MM * lws + 3) & ~3));   // [MM][NW] candidates of a warp
@@ -329,7 +332,10 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
     }
     for (int i = threadIdx.x; i < MM * lws; i += kWThreads)
         s_lw[i] = i % lws < MM ? P.lw[(size_t)(i / lws) * MM + i % lws] : -INFINITY;
-    for (int i = threadIdx.x; i < NW * MM; i += kWThreads) s_rho[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = threadIdx.x; i < NW * MM; i += kWThreads) {
+        s_rho[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (C64) s_rhof[i] = make_float2(0.f, 0.f);
+    }
     __syncthreads();
     for (unsigned long long base = blockIdx.x * (unsigned long long)kWThreads; base < ng;
          base += (unsigned long long)gridDim.x * kWThreads) {
@@ -534,11 +540,13 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
                     float4 &bin = s_rho[warp * MM + c];
                     if constexpr (C64) {
                         float4 v = bin;
-                        two_sum_w(v.x, v.y, s.x);
-                        two_sum_w(v.z, v.w, s.y);
-                        v.y += er.x;
-                        v.w += er.y;
+                        float2 f = s_rhof[warp * MM + c];
+                        two_sum_w(v.x, er.x, s.x);
+                        two_sum_w(v.z, er.y, s.y);
+                        two_sum_w(v.y, f.x, er.x);
+                        two_sum_w(v.w, f.y, er.y);
                         bin = v;
+                        s_rhof[warp * MM + c] = f;
                     } else {
                         double2 v = reinterpret_cast<double2 &>(bin);
                         v.x += s.x;
@@ -579,15 +587,14 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
     // this block's sums of rho, the warps in order
     for (int k = threadIdx.x; k < MM; k += kWThreads) {
         if constexpr (C64) {
-            float4 v = s_rho[k];
-            for (int w = 1; w < NW; ++w) {
+            double2 v = make_double2(0.0, 0.0);
+            for (int w = 0; w < NW; ++w) {
                 const float4 b = s_rho[w * MM + k];
-                two_sum_w(v.x, v.y, b.x);
-                two_sum_w(v.z, v.w, b.z);
-                v.y += b.y;
-                v.w += b.w;
+                const float2 f = s_rhof[w * MM + k];
+                v.x += (double)b.x + ((double)b.y + (double)f.x);
+                v.y += (double)b.z + ((double)b.w + (double)f.y);
             }
-            part[k] = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+            part[k] = v;
         } else {
             double2 v = reinterpret_cast<const double2 *>(s_rho)[k];
             for (int w = 1; w < NW; ++w) {

@@ -76,3 +76,32 @@ def test_rho_of_a_batch_of_three_level_chains(dkmax, theta, steps):
     inst = (keys >> np.uint64(4 * dkmax)).astype(int)
     for i in range(n_inst):
         assert np.abs(rho[i] - _rho_of(3, keys[inst == i], amps[inst == i])).max() <= 8 * 2.0 ** -54
+
+
+@pytest.mark.parametrize("nvib", [4, 3])
+def test_rho_of_wide_keys(nvib):
+    """The same for the wide keys.  Some 35 FP64 additions (a block's eight
+    warps, 16 threads over the blocks, their sums) of partial sums no larger
+    than rho's elements lie behind a block's own sums, each rounded by half a
+    unit in the last place of either sign: twice sqrt(35) of these."""
+    from paper_2506_03127_gb300 import WidePropagator, eta_from_bath
+    steps = 16
+    w = W.reaction_coordinate(nvib, 12, (0, 1, 2, 3, 4, 5, 6, 7, 8, 10), 1e-6, steps)
+    p = WidePropagator(w.M, w.dkmax, w.dt, w.q, w.hs_array(), w.theta, "c64", max_paths=1 << 24)
+    p.set_eta(eta_from_bath(w.bath, w.dt, w.dkmax))
+    p.set_mask(w.mask)
+    for n in (steps, steps + 1):
+        p.set_rho0(w.rho0_array())
+        p.step(n)
+        rho = p.rho(n, 1)[0]
+        keys, amps = p.export_paths()
+        lo = keys[:, 0]
+        newest = (lo & np.uint64(15)).astype(int), ((lo >> np.uint64(4)) & np.uint64(15)).astype(int)
+        exact = np.zeros((w.M, w.M), dtype=complex)
+        for i in range(w.M):
+            for j in range(w.M):
+                v = amps[(newest[0] == i) & (newest[1] == j)]
+                exact[i, j] = complex(math.fsum(v.real), math.fsum(v.imag))
+        unit = 2.0 ** (np.ceil(np.log2(np.abs(rho).max())) - 54)
+        assert np.abs(rho - exact).max() <= 12 * unit
+    p.close()
