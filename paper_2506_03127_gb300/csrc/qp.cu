@@ -1452,12 +1452,20 @@ __device__ __forceinline__ unsigned long long lb_word(unsigned epoch, unsigned s
 // publishing behind the last arrival: 9 us per step at memory 5 FP64 and 8
 // c64.)  Captured steps, the first step and steps launched ahead of the
 // tile kernel read the state.
+//
+// FULL: counts known and M*M members per group, every step once the window
+// is full.  The loop is then a chain of one load, sum, table look-ups and
+// stores per thread with 24 warps per SM to hide it, so that what it decides
+// per group costs in full: with the filling window's and the first merge's
+// group sizes in the same loop memory 14 took 1.444 ms per step and 15 5.72
+// ms (c64), in a form of its own 1.376 and 5.46; memory 13 0.371 -> 0.356 ms
+// c64 and 1.671 -> 1.655 ms FP64.
 struct RegArgs {
     long long tn, ngroups;   // 0: read from the device
     int gs;
     unsigned active;         // blocks with groups; the grid has one more, which publishes
 };
-template <int M, bool C64>
+template <int M, bool C64, bool FULL>
 __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(Params P, int lut_smem, RegArgs a) {
     using X = Expander<M, C64>;
     using AmpT = typename X::AmpT;
@@ -1470,10 +1478,10 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     __shared__ float4 s_wf[C64 ? MM * MM : 1];
     __shared__ float4 s_rt[NW][MM];
     pdl_trigger();
-    const bool known = a.tn != 0;
+    const bool known = FULL || a.tn != 0;
     const long long G = P.region_cap;
     unsigned long long t = 0, n_in = 0;
-    int gs = a.gs;   // members of a group; 0: not a regular step
+    int gs = FULL ? MM : a.gs;   // members of a group; 0: not a regular step
     long long ngroups = a.ngroups, gpr = 0;   // groups, groups per region
     if (known) {
         t = (unsigned long long)a.tn - 1;
@@ -1636,7 +1644,7 @@ __global__ void __launch_bounds__(kRegThreads, M == 2 ? 3 : 1) k_stream_regular(
     auto load = [&](long long g, Members &mb) {
         int r = 0;
         long long j = g;
-        if (t == 0) {
+        if (!FULL && t == 0) {
             for (j = 0;; ++r) {   // the g-th nonempty region
                 if (s_rn[in * MM + r] && j++ == g) break;
             }
@@ -3946,9 +3954,7 @@ struct qp_ctx {
     const void *scache_fn = nullptr;   // stream kernel launched last, its dynamic shared memory and
     size_t scache_smem = 0;            // co-resident blocks per SM
     int scache_res = 0;
-    const void *rcache_fn = nullptr;   // the same for the regular stream kernel
-    size_t rcache_smem = 0;
-    int rcache_res = 0;
+    int rcache_res[2] = {0, 0};        // co-resident blocks per SM of the regular stream kernel's two forms (0: not asked)
     bool use_stream = false;           // this propagation runs on the stream engine
     bool sym = false;                  // symmetric Trotter splitting (qp_set_end_points)
     qp::cplx eta00;                    // ... point 0's half-interval self coefficient
@@ -4119,20 +4125,20 @@ cudaError_t launch_stream_batch(qp_ctx *c, int nsteps, bool coop) {
 // kMaxExpandBlocks (block partials).
 template <int M, bool C64>
 cudaError_t launch_stream_regular(qp_ctx *c, bool dep, RegArgs ra) {
-    const void *fn = (const void *)k_stream_regular<M, C64>;
+    const bool full = ra.tn && ra.gs == M * M;
+    const void *fn = full ? (const void *)k_stream_regular<M, C64, true> : (const void *)k_stream_regular<M, C64, false>;
+    int &res = c->rcache_res[full ? 1 : 0];   // (the rest of the key, M, precision and tables, is the context's)
     const size_t lutb = stream_lut_bytes(c, C64);
-    if (c->rcache_fn != fn || c->rcache_smem != lutb) {
+    if (res == 0) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxStreamLut);
         if (e != cudaSuccess) return e;
         int nb = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kRegThreads, lutb);
         if (e != cudaSuccess) return e;
         if (nb < 1) return cudaErrorInvalidConfiguration;
-        c->rcache_fn = fn;
-        c->rcache_smem = lutb;
-        c->rcache_res = nb;
+        res = nb;
     }
-    int g = std::min(c->nsm * c->rcache_res, kMaxExpandBlocks);
+    int g = std::min(c->nsm * res, kMaxExpandBlocks);
     if (ra.tn) {
         // one block per SM while a block's warps take a chunk or two each:
         // fewer partials of rho to sum beside the step, and the publishing
