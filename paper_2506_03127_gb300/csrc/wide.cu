@@ -258,12 +258,13 @@ __global__ void __launch_bounds__(kWThreads) k_w_tie(WParams P) {
     }
 }
 
-// log2 of a non-negative double to FP32 accuracy, off the FP64 pipe (zero and
-// subnormals: -inf; infinities and NaNs: +inf, which no bound drops)
+// log2 of a square to FP32 accuracy, off the FP64 pipe, never below it by more
+// than that: zero and subnormals, which a square may have underflowed to, give
+// -1022, infinities and NaNs +inf, which no bound drops
 __device__ __forceinline__ float log2_d(double d) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(d);
     const int e = (int)((u >> 52) & 0x7ffull);
-    if (e == 0) return -INFINITY;
+    if (e == 0) return -1022.f;
     if (e == 0x7ff) return INFINITY;
     return (float)(e - 1023) + log2f(__uint_as_float(0x3f800000u | (unsigned)((u >> 29) & 0x7fffffull)));
 }
@@ -691,7 +692,7 @@ __global__ void k_w_build_w(double2 *w, float4 *wf, float *lw, const double2 *U,
         w[i] = v;
         const float hx = (float)v.x, hy = (float)v.y;
         wf[i] = make_float4(hx, hy, (float)(v.x - (double)hx), (float)(v.y - (double)hy));
-        lw[(size_t)par * MM + child] = (float)log2(v.x * v.x + v.y * v.y);
+        lw[(size_t)par * MM + child] = (float)(2.0 * log2(hypot(v.x, v.y)));   // (no square to underflow)
     }
 }
 
