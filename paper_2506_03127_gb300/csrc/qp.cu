@@ -178,7 +178,7 @@ struct Params {
     long long *scount;                 // stream engine: [2][kMaxExpandBlocks] children written per block
                                        // of rho(t) per instance; element M*M holds the survivor count
     long long *inst_kept;              // [rho_hist][n_inst] stored paths per instance after each step
-    unsigned int *fin_count;           // blocks of k_finalize that are done (last one updates the state)
+    unsigned int *fin_count;           // arrivals of the step's last kernel (the last block updates the state)
     int n_inst;                        // independent instances (1 = single problem)
     int inst_shift;                    // key bit where the instance index starts (b * dkmax)
     unsigned long long instmask;       // key bits of the instance index
@@ -311,10 +311,10 @@ __device__ __forceinline__ void raise_err(DevState *st, unsigned int bit) {
 // Whether the propagation has failed, the same answer for every thread of the
 // block: other blocks of a kernel may raise the error while this one reads it,
 // and threads that left alone would leave the block's barriers and shared
-// counters without their part.  Every thread of the block calls it.
-__device__ __forceinline__ bool failed_block(const DevState *st) {
-    return __syncthreads_or(*(const volatile unsigned *)&st->err != 0u) != 0;
-}
+// counters without their part.  err: the flag as the thread reads it (a plain
+// load at a kernel's start; a volatile one cost 0.7 us per kernel in the
+// merge table's steps).  Every thread of the block calls it.
+__device__ __forceinline__ bool failed_block(unsigned err) { return __syncthreads_or(err != 0u) != 0; }
 
 // Block-wide append: exclusive offset of each thread's cnt items within the
 // block and the block's base in a global array, with one atomicAdd on the
@@ -483,7 +483,7 @@ __device__ __forceinline__ void phase_tiebreak(const Params &P, unsigned long lo
 template <typename Amp>
 __global__ void __launch_bounds__(kInsertThreads) k_insert(Params P) {
     DevState *st = P.st;
-    if (failed_block(st)) return;
+    if (failed_block(st->err)) return;
     const unsigned long long t = st->t, tn = t + 1, n = st->n_cur;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->ext_t = t;
@@ -1178,9 +1178,9 @@ __device__ __forceinline__ void phase_finalize_stream(const Params &P, unsigned 
 }
 
 // The stream kernels' last block publishes a step's counters and leaves the
-// sum of the blocks' partials of rho to block 0 of the next step (or to
-// k_rho_finalize before a read): rho(t) of a step is complete when the next
-// step starts or the host reads it.  Partials alternate by step parity, so
+// sum of the blocks' partials of rho to a block of the next step that has no
+// work of its own (or to k_rho_finalize before a read): rho(t) of a step is
+// complete when the next step ends or the host reads it.  Partials alternate by step parity, so
 // the next step's own partials never overwrite them.  Block-uniform.
 template <bool C64>
 __device__ __forceinline__ void finish_pending_rho(const Params &P, DevState *st, int MM) {
@@ -1272,7 +1272,7 @@ __device__ __forceinline__ void finalize_single(const Params &P, unsigned long l
 template <int M, bool C64, bool BATCH>
 __global__ void __launch_bounds__(kExpandThreads) k_expand(Params P) {
     DevState *st = P.st;
-    if (failed_block(st)) return;
+    if (failed_block(st->err)) return;
     const unsigned long long t = st->ext_t, tn = t + 1;
     const bool merge = tn >= (unsigned long long)P.dkmax;
     const unsigned long long n = merge ? st->cnt_groups[tn % 3] : st->ext_n;
@@ -1364,7 +1364,7 @@ __global__ void __launch_bounds__(kPersistThreads) k_step_persistent(Params P, i
     using Amp = typename Expander<M, C64>::AmpT;
     DevState *st = P.st;
     const int nblk = (int)gridDim.x;
-    unsigned err = failed_block(st);
+    unsigned err = failed_block(st->err);
     unsigned long long t = st->t;
     unsigned long long n_in = st->n_cur;
     unsigned long long prev_groups = 0, prev_out = 0;
@@ -1977,7 +1977,7 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
     const unsigned long long t = tn_host ? tn_host - 1 : __ldcg(&st->t), tn = t + 1;
     // an earlier error, or launched behind the regular kernel, which just took
     // this step (its new t + 1)
-    if (failed_block(st) || ((flags & kFlagAfterRegular) && __ldcg(&st->reg_done) == tn)) {
+    if (failed_block(__ldcg(&st->err)) || ((flags & kFlagAfterRegular) && __ldcg(&st->reg_done) == tn)) {
         if constexpr (!BATCH) cp_async_wait_all();
         return;
     }
@@ -3004,8 +3004,8 @@ __device__ __forceinline__ void stream_step_body(const Params &P, int flags, uns
         if ((int)threadIdx.x < kCsThreads) reinterpret_cast<float2 *>(s_stg)[threadIdx.x] = make_float2(cs_s, cs_e);
     // arrive first: the last block to arrive publishes the step, for which
     // it needs the step's counters only; every block then writes its partial
-    // of rho, which the next step's block 0 (or a read-time finalisation)
-    // sums once this kernel has ended
+    // of rho, which the first block without a tile of the next step (or a
+    // read-time finalisation) sums once this kernel has ended
     __syncthreads();
     if (threadIdx.x == 0) {
         // one acquire-release add: releases this block's writes (ordered
@@ -3185,7 +3185,7 @@ __device__ __forceinline__ unsigned long long compress_masked(const Params &P, u
 template <int M, bool C64>
 __global__ void __launch_bounds__(kExpandThreads) k_post_expand(Params P) {
     DevState *st = P.st;
-    if (failed_block(st)) return;
+    if (failed_block(st->err)) return;
     const unsigned long long t = st->t, tn = t + 1;
     phase_expand<M, C64, kExpandThreads, false>(P, t, st->n_cur, false, &st->cnt_out[tn % 3], rho_part_of(P, tn, M * M),
                                                 P.ckeys, P.camps);

@@ -169,7 +169,7 @@ __device__ __forceinline__ double2 amp_of(const WParams &P, const void *amps, un
 // and threads that left alone would leave the others' shared scans without
 // their part.  Every thread of the block calls it.
 __device__ __forceinline__ bool failed_block(const WState *st) {
-    return __syncthreads_or(*(const volatile unsigned *)&st->err != 0u) != 0;
+    return __syncthreads_or(st->err != 0u) != 0;
 }
 
 // The part of the table that a step of n paths uses: two slots per path at
