@@ -47,7 +47,8 @@
 // group sums are FP64 atomic sums in the merge table (k_insert), while the
 // stream kernels add a group's FP32 members in FP32 with the rounding error
 // of every addition kept in a second word (TwoSum) and round the pair once
-// to FP32, the precision the children are formed in.
+// to FP32, the precision the children are formed in (runs of more than 32
+// members: FP64, rounded once).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1440,8 +1441,9 @@ __device__ __forceinline__ unsigned long long lb_word(unsigned epoch, unsigned s
 // (1.6e4 groups, complex64) and 5 (256 groups, FP64) the step is latency:
 // with every block of the grid reducing and arriving, and block 0 summing
 // the pending rho first, the kernel took 13.3 and 21.2 us (under ncu), and
-// 100 and 40 steps through qp_step 1.72 and 1.09 ms; now 1.16 and 0.50 ms,
-// with the tile kernel's empty launch gone (step_kind).
+// 100 and 40 steps through qp_step 1.72 and 1.09 ms; this split took them to
+// 1.16 and 0.50 ms, with the tile kernel's empty launch gone (step_kind), and
+// the counts from the host to 0.43 and 0.23 ms:
 //
 // The host knows the counts of an unfiltered propagation (step_kind) and
 // passes them (a.tn != 0): then no block reads the device state before its
