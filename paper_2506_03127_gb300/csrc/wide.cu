@@ -286,9 +286,10 @@ inline size_t expand_smem(int MM, int nb, bool c64) {
 // dealt evenly to the threads and a warp's children share their newest
 // point; each is formed once in full precision, filtered, added to rho(t)
 // (segments of equal newest point, then one lane's addition to its warp's
-// bin; C64: FP32 pairs with TwoSum, the bins of three words, which lose less
-// than the FP64 sums of before: with two, rho was off by up to 1e-15 instead
-// of 6e-17) and written to a range reserved per 256
+// bin; C64: sums of three FP32 words with TwoSum, as close to the exact sum as
+// FP64 ones, 1e-16 at most in rho, at 16.8 ms per 20 steps of the eight-state
+// model, FP64 17.7 to 17.9; pairs, 16.4 ms, left up to 1e-15) and written to a
+// range reserved per 256
 // candidates.  (Forming all 64 children twice, four lanes per group, with
 // rho from a second pass over the children took 0.88 ms per step and launch
 // at 2e6 groups, the two passes of rho and of its block sums 0.30 ms.)
@@ -512,8 +513,8 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
             // rho(t+1): the kept children of a segment of equal c, added by
             // its last lane to the warp's bin
             {
-                CT s = child, er;
-                er.x = er.y = 0;
+                CT s = child, er, ef;   // C64: three words
+                er.x = er.y = ef.x = ef.y = 0;
                 if (!kept) s.x = s.y = 0;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -521,12 +522,30 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
                     const bool add = (int)lane >= o && cu == c;
                     if constexpr (C64) {
                         const float bx = __shfl_up_sync(0xffffffffu, s.x, o), by = __shfl_up_sync(0xffffffffu, s.y, o);
-                        const float ex = __shfl_up_sync(0xffffffffu, er.x, o), ey = __shfl_up_sync(0xffffffffu, er.y, o);
+                        float ex = 0.f, ey = 0.f, fx = 0.f, fy = 0.f;   // (the words that are there after o = 1, 2)
+                        if (o > 1) {
+                            ex = __shfl_up_sync(0xffffffffu, er.x, o);
+                            ey = __shfl_up_sync(0xffffffffu, er.y, o);
+                        }
+                        if (o > 2) {
+                            fx = __shfl_up_sync(0xffffffffu, ef.x, o);
+                            fy = __shfl_up_sync(0xffffffffu, ef.y, o);
+                        }
                         if (add) {
-                            two_sum_w(s.x, er.x, bx);
-                            two_sum_w(s.y, er.y, by);
-                            er.x += ex;
-                            er.y += ey;
+                            float gx = 0.f, gy = 0.f;
+                            two_sum_w(s.x, gx, bx);
+                            two_sum_w(s.y, gy, by);
+                            if (o == 1) {
+                                er.x = gx;
+                                er.y = gy;
+                            } else {
+                                two_sum_w(er.x, ef.x, gx);
+                                two_sum_w(er.y, ef.y, gy);
+                                two_sum_w(er.x, ef.x, ex);
+                                two_sum_w(er.y, ef.y, ey);
+                                ef.x += fx;
+                                ef.y += fy;
+                            }
                         }
                     } else {
                         const double bx = __shfl_up_sync(0xffffffffu, s.x, o), by = __shfl_up_sync(0xffffffffu, s.y, o);
@@ -542,10 +561,15 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
                     if constexpr (C64) {
                         float4 v = bin;
                         float2 f = s_rhof[warp * MM + c];
-                        two_sum_w(v.x, er.x, s.x);
-                        two_sum_w(v.z, er.y, s.y);
+                        float gx = 0.f, gy = 0.f;
+                        two_sum_w(v.x, gx, s.x);
+                        two_sum_w(v.z, gy, s.y);
+                        two_sum_w(v.y, f.x, gx);
+                        two_sum_w(v.w, f.y, gy);
                         two_sum_w(v.y, f.x, er.x);
                         two_sum_w(v.w, f.y, er.y);
+                        f.x += ef.x;
+                        f.y += ef.y;
                         bin = v;
                         s_rhof[warp * MM + c] = f;
                     } else {
