@@ -616,8 +616,9 @@ __global__ void __launch_bounds__(kWThreads) k_w_expand(WParams P, int merge) {
             for (int w = 0; w < NW; ++w) {
                 const float4 b = s_rho[w * MM + k];
                 const float2 f = s_rhof[w * MM + k];
-                v.x += (double)b.x + ((double)b.y + (double)f.x);
-                v.y += (double)b.z + ((double)b.w + (double)f.y);
+                // (the errors of an infinite sum are not numbers)
+                v.x += isfinite(b.x) ? (double)b.x + ((double)b.y + (double)f.x) : (double)b.x;
+                v.y += isfinite(b.z) ? (double)b.z + ((double)b.w + (double)f.y) : (double)b.z;
             }
             part[k] = v;
         } else {

@@ -105,3 +105,18 @@ def test_rho_of_wide_keys(nvib):
         unit = 2.0 ** (np.ceil(np.log2(np.abs(rho).max())) - 54)
         assert np.abs(rho - exact).max() <= 12 * unit
     p.close()
+
+
+def test_infinite_amplitudes_of_wide_keys():
+    """At the second step eta_1 = -1 multiplies the children (0, 1) of (0, 1) by
+    exp(4): 54 times 0.58^2 of 6e37 is beyond FP32.  The child, and rho with
+    it, is infinite, not undefined (as a plain sum would have it)."""
+    from paper_2506_03127_gb300 import WidePropagator
+    p = WidePropagator(2, 3, 1.0, (1.0, -1.0), np.array([[0.0, 0.7], [0.7, 0.0]]), 1e-10, "c64", max_paths=1 << 10)
+    p.set_eta(np.array([0.0, -1.0, 0.0]))
+    p.set_mask((0, 1, 2))
+    p.set_rho0(np.array([[0.0, 6e37], [0.0, 0.0]]))
+    p.step(2)
+    rho = p.rho(2, 1)[0]
+    p.close()
+    assert np.isposinf(rho[0, 1].real) and np.isfinite(rho[0, 1].imag)
